@@ -65,9 +65,10 @@ typedef struct spi_options {
     int ordering;    /* spi_ordering */
     int rhs_block;   /* right-hand sides per block in spi_diag_inverse, 1..512 (rounded up to a
                         multiple of 8 in mixed precision); 0 = automatic: the first variance call
-                        times a few candidate sizes on the factor and keeps the fastest (32 in
-                        FP64, 64-128 in mixed precision on the SPI workloads; Sec. 4.3 groups 128
-                        right-hand sides on a CPU core) */
+                        times a few candidate sizes on the factor and keeps the fastest (64-128 in
+                        mixed precision on the SPI workloads); the FP64 form on the tensor cores
+                        takes 16, 32 or 64 by the number of right-hand sides (Sec. 4.3 groups
+                        128 right-hand sides on a CPU core) */
     int relax;       /* supernode amalgamation: max explicit zeros per parent-child merge as a
                         percentage of the merged panel, plus merges of very small supernodes and
                         grouping of sibling leaf fronts; 0 = fundamental supernodes only;
@@ -146,7 +147,11 @@ typedef struct spi_options {
                         tiles also let the mixed solve take 128 columns per step there.  0 = the
                         default (32); < 0 = none (SIMT variances, 32-column solve steps).
                         Variance blocks of more than 128 right-hand sides (rhs_block > 128) stay
-                        on the SIMT kernel */
+                        on the SIMT kernel.  FP64 form: >= 0 the variances run on the tensor
+                        cores from exact integer pieces of the operands, at FP64 accuracy
+                        (blocks of 16, 32 or 64 right-hand sides, chosen by their number when
+                        rhs_block = 0; other rhs_block values, and a device without memory for
+                        the packed operands, take the SIMT kernel); < 0 the SIMT kernel */
 } spi_options;
 
 typedef struct spi_stats {

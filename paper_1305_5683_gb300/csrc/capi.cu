@@ -137,6 +137,11 @@ struct spi_ctx {
     // diag_tc_min_pivots pivots and their ancestors)
     DiagTcHost dtc_h;
     DevDiagTc dtc;
+    // variances of the FP64 form on the tensor cores: set up at the first variance call
+    // (-1: not yet, 0: not in use, 1: ready)
+    int fx_state = -1;
+    DiagFxHost fx_h;
+    DevDiagFx fx;
     double last_diag_tc_flops = 0;
     // the mixed solve's plan with 128-column steps for those supernodes (their inverted
     // diagonal tiles); the FP64-panel paths keep SP
@@ -309,6 +314,52 @@ int ensure_device(spi_ctx* c) {
     return SPI_OK;
 }
 
+void free_fx(DevDiagFx& t) {
+    for (void* a : t.allocs) cudaFree(a);
+    t = DevDiagFx();
+}
+
+// Buffers of the FP64 form's tensor-core variances (operands are prepared from the factor
+// by every call).  Without the memory for them the SIMT kernel serves alone.
+int ensure_fx(spi_ctx* c) {
+    if (c->fx_state >= 0) return SPI_OK;
+    c->fx_state = 0;
+    if (mixed_of(c) || c->opt.pivoting || c->opt.diag_tc_min_pivots < 0 || c->S.n == 0) return SPI_OK;
+    DiagFxHost& h = c->fx_h;
+    build_diag_fx(c->S, h);
+    DevDiagFx& t = c->fx;
+    t = DevDiagFx();
+    const size_t nb = (size_t)c->opt.batch, n = (size_t)c->S.n;
+    const int64_t before = c->device_bytes;
+    std::vector<void*>* tr = &t.allocs;
+    auto alloc = [&]() -> cudaError_t {
+        cudaError_t e = dev_upload(c, &t.pptr, h.pptr, tr);
+        if (e == cudaSuccess) e = dev_upload(c, &t.tptr, h.tptr, tr);
+        if (e == cudaSuccess) e = dev_upload(c, &t.tiles, h.tiles, tr);
+        if (e == cudaSuccess) e = dev_upload(c, &t.tdiag, h.tdiag, tr);
+        if (e == cudaSuccess) e = dev_upload(c, &t.dtiles, h.dtiles, tr);
+        if (e == cudaSuccess) e = dev_alloc(c, &t.pack, diag_fx_pack_bytes(h.npieces) * nb, tr);
+        if (e == cudaSuccess) e = dev_alloc(c, &t.rexp, (size_t)h.ntiles * kFxRows * nb, tr);
+        if (e == cudaSuccess) e = dev_alloc(c, &t.fr, n * nb, tr);
+        if (e == cudaSuccess) e = dev_alloc(c, &t.xinv, (size_t)h.ndt * kFxRows * kFxRows * nb, tr);
+        return e;
+    };
+    const cudaError_t e = alloc();
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        free_fx(t);
+        c->device_bytes = before;
+        return SPI_OK;
+    }
+    CK(e);
+    CK(diag_fx_setup());
+    t.npieces = h.npieces;
+    t.ntiles = h.ntiles;
+    t.ndt = h.ndt;
+    c->fx_state = 1;
+    return SPI_OK;
+}
+
 void free_plan(DevDiagPlan& p) {
     for (void* a : p.allocs) cudaFree(a);
     p = DevDiagPlan();
@@ -333,6 +384,15 @@ int upload_plan(spi_ctx* c, const DiagPlan& h, DevDiagPlan& d) {
     CK(dev_upload(c, &d.urel, h.urel, tr));
     CK(dev_upload(c, &d.zbase, h.zbase, tr));
     d.zsize = h.zbase.empty() ? 0 : h.zbase.back();
+    d.fx = c->fx_state == 1 && (h.B == 16 || h.B == 32 || h.B == kFxMaxBlock);
+    if (d.fx) {
+        std::vector<int32_t> tiles, dts;
+        diag_fx_used(c->S, c->fx_h, h, tiles, dts);
+        d.fx_ntiles = (int64_t)tiles.size();
+        d.fx_ndt = (int64_t)dts.size();
+        CK(dev_upload(c, &d.fx_tiles, tiles, tr));
+        CK(dev_upload(c, &d.fx_dts, dts, tr));
+    }
     // FP64 elements per band are enough for both element types
     CK(dev_alloc(c, &d.Z, (size_t)std::max<int64_t>(d.zsize, 1) * (size_t)c->opt.batch, tr));
     return SPI_OK;
@@ -763,6 +823,8 @@ void reset_device(spi_ctx* c) {
     free_plan(c->plan_all);
     free_plan(c->plan_sub);
     free_plan(c->plan_blk);
+    free_fx(c->fx);
+    c->fx_state = -1;
     free_factor_plan(c->dfp);
     c->plan_all_ready = c->plan_sub_ready = c->plan_blk_ready = false;
     for (auto* g : {&c->g_factor, &c->g_solve, &c->g_solve_dag}) {
@@ -1150,9 +1212,17 @@ void launch_diag(spi_ctx* c, const DevDiagPlan& p, int nb, int64_t nout, double*
                                 tc ? c->dtc.tc : nullptr, st);
         if (tc) launch_diag_inv_tc(c->dsym, p, c->dtc, c->d_D, out, nb, bs, c->d_status, c->opt.wait_limit, st);
     } else {
-        launch_diag_inverse(dev_sol(c), p, c->d_L, c->d_D, out, nb, bs, c->diag_smem_pad, st);
+        if (p.fx) launch_diag_fx(c->dsym, p, c->fx, c->d_L, c->d_D, out, nb, bs, c->d_status, st);
+        else launch_diag_inverse(dev_sol(c), p, c->d_L, c->d_D, out, nb, bs, c->diag_smem_pad, st);
     }
 }
+
+// Right-hand sides per block of the FP64 form's tensor-core variances.  A block has an SM
+// to itself and its tiles cost nearly as much for 16 columns as for 64, so blocks are as
+// large as leaves every one of the 152 SMs one (P = 300, 467 right-hand sides: 134 us with
+// 16, 183 with 64; P = 2,003, 3,199: 255 with 16, 232 with 32, 313 with 64; forest of 48,
+// 51,264: 1.64 ms with 32, 1.39 with 64).
+int fx_block(int64_t nrhs) { return nrhs <= 152 * 16 ? 16 : nrhs <= 152 * 32 ? 32 : 64; }
 
 // Build the plan for the pivots `piv`; with an automatic block size (the
 // autotuner), time each candidate once on the current factor and keep the
@@ -1160,7 +1230,12 @@ void launch_diag(spi_ctx* c, const DevDiagPlan& p, int nb, int64_t nout, double*
 int make_plan(spi_ctx* c, const std::vector<int32_t>& piv, const std::vector<int32_t>& pos, DevDiagPlan& dst,
               int nb, int64_t nout, double* out, cudaStream_t st) {
     std::vector<int> cands;
+    {
+        const int rc = ensure_fx(c);
+        if (rc) return rc;
+    }
     if (c->opt.rhs_block > 0) cands.push_back(c->opt.rhs_block);
+    else if (c->fx_state == 1) cands.push_back(fx_block((int64_t)piv.size() * nb));
     else if (c->rhs_block_used > 0) cands.push_back(c->rhs_block_used);
     else if (mixed_of(c)) cands = {32, 64, 128};
     else cands = {16, 32, 64};
@@ -1594,8 +1669,10 @@ int inverse_block_impl(spi_ctx* c, std::vector<int32_t>& key, double* od, cudaSt
         std::vector<int32_t> piv((size_t)nidx), pos((size_t)nidx);
         for (int64_t t = 0; t < nidx; ++t) { piv[t] = S.iperm[key[t]]; pos[t] = (int32_t)t; }
         DiagPlan h;
-        build_diag_plan(S, piv, pos, c->rhs_block_used > 0 ? c->rhs_block_used : 32, h);
-        int rc = upload_plan(c, h, c->plan_blk);
+        int rc = ensure_fx(c);
+        if (rc) return rc;
+        build_diag_plan(S, piv, pos, c->fx_state == 1 ? fx_block(nidx) : c->rhs_block_used > 0 ? c->rhs_block_used : 32, h);
+        rc = upload_plan(c, h, c->plan_blk);
         if (rc) return rc;
         // rows of the union of all blocks' paths (ascending pivots), and each
         // block-local Z row's position among them; a block's supernodes own
@@ -1634,7 +1711,8 @@ int inverse_block_impl(spi_ctx* c, std::vector<int32_t>& key, double* od, cudaSt
         c->plan_blk_key.swap(key);
         c->plan_blk_ready = true;
     }
-    launch_inverse_block(c->dsym, c->plan_blk, c->d_L, c->d_D, c->d_out, c->d_zg, c->blk_rows, od, nidx, st);
+    launch_inverse_block(c->dsym, c->plan_blk, c->fx_state == 1 ? &c->fx : nullptr, c->d_L, c->d_D, c->d_out,
+                         c->d_zg, c->blk_rows, od, nidx, c->d_status, st);
     return SPI_OK;
 }
 }  // namespace
@@ -2514,6 +2592,7 @@ void spi_destroy(spi_ctx* c) {
     free_plan(c->plan_all);
     free_plan(c->plan_sub);
     free_plan(c->plan_blk);
+    free_fx(c->fx);
     free_factor_plan(c->dfp);
     if (c->d_zg) cudaFree(c->d_zg);
     for (auto& kv : c->g_factor) cudaGraphExecDestroy(kv.second);

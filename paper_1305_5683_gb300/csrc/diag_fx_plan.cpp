@@ -1,0 +1,43 @@
+// diag_fx_plan.cpp -- see diag_fx_plan.h
+#include "diag_fx_plan.h"
+
+#include <algorithm>
+
+namespace spi {
+
+void build_diag_fx(const Symbolic& S, DiagFxHost& h) {
+    h = DiagFxHost();
+    h.pptr.assign(S.ns, -1);
+    h.tptr.assign(S.ns, -1);
+    for (int32_t s = 0; s < S.ns; ++s) {
+        const int32_t k = S.k_of(s), m = S.m_of(s);
+        h.pptr[s] = h.npieces;
+        h.tptr[s] = h.ntiles;
+        for (int32_t g = 0; g * kFxRows < k; ++g) {
+            const int32_t w = std::min(kFxRows, k - g * kFxRows), base = std::min(kFxRows * (g + 1), k);
+            const int32_t np = (w + kFxSub - 1) / kFxSub, nt = 1 + (m - base + kFxRows - 1) / kFxRows;
+            for (int32_t c = 0; c < w; c += kFxInvCols) h.dtiles.insert(h.dtiles.end(), {s, g, h.ndt, c});
+            for (int32_t i = 0; i < nt; ++i) {
+                h.tiles.insert(h.tiles.end(), {s, g, i, (int32_t)h.npieces});
+                h.tdiag.push_back(i == 0 ? h.ndt : -1);
+                h.npieces += np;
+                ++h.ntiles;
+            }
+            ++h.ndt;
+        }
+    }
+}
+
+void diag_fx_used(const Symbolic& S, const DiagFxHost& h, const DiagPlan& dp, std::vector<int32_t>& tiles,
+                  std::vector<int32_t>& dts) {
+    std::vector<uint8_t> used(S.ns, 0);
+    for (int32_t s : dp.us) used[s] = 1;
+    tiles.clear();
+    dts.clear();
+    for (size_t t = 0; 4 * t < h.tiles.size(); ++t)
+        if (used[h.tiles[4 * t]]) tiles.push_back((int32_t)t);
+    for (size_t t = 0; 4 * t < h.dtiles.size(); ++t)
+        if (used[h.dtiles[4 * t]]) dts.push_back((int32_t)t);
+}
+
+}  // namespace spi

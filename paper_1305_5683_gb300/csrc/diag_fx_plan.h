@@ -1,0 +1,36 @@
+// diag_fx_plan.h -- host plan of the FP64 variance kernel on the tensor cores
+// (diag_fx.cu): the packed left-operand tiles of every supernode.
+#pragma once
+#include <cstdint>
+#include <vector>
+
+#include "analysis.h"
+
+namespace spi {
+
+constexpr int kFxRows = 128;    // rows of a tile (the MMA's M) and columns of a K chunk
+constexpr int kFxSub = 16;      // columns of one packed piece of a tile (the MMA's K)
+constexpr int kFxInvCols = 8;   // columns of a diagonal tile's inverse per CTA
+constexpr int kFxMaxBlock = 64; // right-hand sides of a block the kernel takes
+
+struct DiagFxHost {
+    int64_t npieces = 0;          // packed 128 x 16 pieces (per band)
+    int32_t ntiles = 0, ndt = 0;  // 128 x 128 tiles, inverted diagonal tiles (per band)
+    std::vector<int64_t> pptr;    // [ns] first packed piece of the supernode
+    std::vector<int32_t> tptr;    // [ns] first tile of the supernode
+    std::vector<int32_t> tiles;   // [ntiles][4]: supernode, chunk g, tile i of the chunk (0: its
+                                  //   diagonal tile's inverse, i > 0: rows base + 128 (i - 1) ..), first piece
+    std::vector<int32_t> dtiles;  // [][4]: supernode, chunk, number of the diagonal tile, first of 8 columns
+    std::vector<int32_t> tdiag;   // [ntiles]: the diagonal tile's number (i = 0), else -1
+};
+
+// Every supernode; per 128-column chunk g of a supernode (k pivots, m rows): the inverse of its
+// unit-lower diagonal tile, then the rows from min(128 (g + 1), k) to m in
+// tiles of 128, each tile in ceil(w / 16) pieces (w the chunk's columns).
+void build_diag_fx(const Symbolic& S, DiagFxHost& h);
+// the tiles and diagonal-tile columns (positions in h.tiles / 4, h.dtiles / 4) of the
+// supernodes that plan dp walks
+void diag_fx_used(const Symbolic& S, const DiagFxHost& h, const DiagPlan& dp, std::vector<int32_t>& tiles,
+                  std::vector<int32_t>& dts);
+
+}  // namespace spi

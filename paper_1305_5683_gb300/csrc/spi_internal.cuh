@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "analysis.h"
+#include "diag_fx_plan.h"
 #include "diag_tc_plan.h"
 #include "spi.h"
 
@@ -202,6 +203,10 @@ struct DevDiagPlan {
     int32_t* rowmap = nullptr;
     double flops = 0, work_flops = 0;
     double tc_flops = 0;  // TF32 MMA flops of the tensor-core variance kernel on this plan
+    bool fx = false;      // FP64 form: on the tensor cores (diag_fx.cu), with the operand tiles of the
+                          //   plan's supernodes
+    int32_t *fx_tiles = nullptr, *fx_dts = nullptr;
+    int64_t fx_ntiles = 0, fx_ndt = 0;
     std::vector<void*> allocs;
 };
 
@@ -249,13 +254,6 @@ void launch_pick_entries(const double* G, const int64_t* src, const int64_t* dst
                          cudaStream_t st);
 // smem_min: the launches' dynamic shared memory is at least this (0: what they need)
 cudaError_t diag_kernel_setup(int B, size_t smem_min);
-// (N^-1)(I, I) for the pivots of a plan with zpiv/rowmap: the blocks' forward
-// solves (variances to var_scratch), their vectors gathered into Zg (R rows x
-// nrhs), then the Gram product into out (ldo = leading dimension, positions
-// from the plan's rhs_out).
-void launch_inverse_block(const DevSym& d, const DevDiagPlan& p, const double* L, const double* D,
-                          double* var_scratch, double* Zg, int64_t R, double* out, int64_t ldo, cudaStream_t st);
-
 // ---- diag_tc.cu: the mixed form's variances on the tensor cores for the
 // supernodes with at least min_k pivots and their ancestors
 struct DevDiagTc {
@@ -280,6 +278,32 @@ void launch_diag_tc_pack(const DevSym& d, const DevDiagTc& p, const float* L32, 
 // after launch_diag_inverse_f32 with skip = p.tc on the same plan and outputs
 void launch_diag_inv_tc(const DevSym& d, const DevDiagPlan& dp, const DevDiagTc& p, const double* D, double* out,
                         int nb, const Strides& bs, DevStatus* status, int wait_limit, cudaStream_t st);
+
+// ---- diag_fx.cu: the FP64 form's variances on the tensor cores (exact integer pieces)
+struct DevDiagFx {
+    int64_t npieces = 0, ntiles = 0, ndt = 0;
+    int64_t* pptr = nullptr;
+    int32_t *tptr = nullptr, *tiles = nullptr, *tdiag = nullptr, *dtiles = nullptr;
+    unsigned char* pack = nullptr;  // [bands][npieces] packed 128 x 16 pieces, seven digit planes each
+    int32_t* rexp = nullptr;        // [bands][ntiles][128] row exponents
+    double* xinv = nullptr;         // [bands][ndt][128 x 128] inverted diagonal tiles
+    double* fr = nullptr;           // [bands][n] s^2 / d, s the power of two next to sqrt(d)
+    std::vector<void*> allocs;
+};
+cudaError_t diag_fx_setup();
+size_t diag_fx_pack_bytes(int64_t npieces);
+// prepares the operands from the factor, then the variances of plan dp (dp.B
+// 16, 32 or 64)
+void launch_diag_fx(const DevSym& d, const DevDiagPlan& dp, const DevDiagFx& p, const double* L, const double* D,
+                    double* out, int nb, const Strides& bs, DevStatus* status, cudaStream_t st);
+
+// (N^-1)(I, I) for the pivots of a plan with zpiv/rowmap: the blocks' forward
+// solves (variances to var_scratch; on the tensor cores with fx, when the plan has fx
+// set), their vectors gathered into Zg (R rows x nrhs), then the Gram product into
+// out (ldo = leading dimension, positions from the plan's rhs_out).
+void launch_inverse_block(const DevSym& d, const DevDiagPlan& p, const DevDiagFx* fx, const double* L, const double* D,
+                          double* var_scratch, double* Zg, int64_t R, double* out, int64_t ldo, DevStatus* status,
+                          cudaStream_t st);
 
 // ---- normal.cu: N = H^T W H and b = H^T W y on the device
 struct NormalArgs {

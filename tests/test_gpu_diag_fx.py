@@ -1,0 +1,120 @@
+"""The FP64 form's variances on the tensor cores (exact integer pieces, diag_fx.cu)
+against the SIMT kernel on the same factor (diag_tc_min_pivots = -1) and the oracle.
+
+Bound: both kernels compute z = L^-1 e with a backward error of a few units in the
+last place per multiply-add, at most n of them on a path, so two of them differ by
+at most about n 2^-53 times the condition of the (scaled) triangles; 64 n 2^-53 leaves
+a factor 64 for that condition and the two operands' fixed-point grids (2^-56 of
+their largest entries)."""
+import numpy as np
+import pytest
+
+import oracle
+from spigen import SCALE, BAND, generate, generate_bands, random_spd, scaled, sky_scaled
+
+pytestmark = pytest.mark.gpu
+EPS = 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def P():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1305_5683_gb300 as P
+    P.build.build()
+    return P
+
+
+def both(P, pb, values=None, idx=None, **kw):
+    """(tensor cores, SIMT) variances of one problem."""
+    out = []
+    for more in (kw, {"diag_tc_min_pivots": -1}):
+        s = P.Solver.for_problem(pb, **more)
+        s.factor(pb.values if values is None else values)
+        out.append(s.diag_inverse(idx))
+    return out
+
+
+def rel(a, b):
+    return float((np.abs(a - b) / b).max())
+
+
+# one dense front of order n: tiles, pieces and row groups just below, at and above their
+# edges, a single column, several 128-column chunks with a ragged last one
+@pytest.mark.parametrize("n", [1, 7, 8, 9, 15, 16, 17, 31, 33, 127, 128, 129, 144, 255, 257, 400])
+@pytest.mark.parametrize("block", [16, 64])
+def test_dense_front_edges(P, n, block):
+    pb = random_spd(n, 1.0, n, dominance=0.1)
+    fx, simt = both(P, pb, rhs_block=block)
+    assert rel(fx, oracle.OracleFactor.from_problem(pb).inv_diag()) <= 64 * max(n, 16) * EPS
+    assert rel(fx, simt) <= 64 * max(n, 16) * EPS
+
+
+@pytest.mark.parametrize("block", [16, 32, 64])
+def test_spi_problem_blocks(P, block):
+    pb = generate(scaled(SCALE, 2003, seed=5))
+    fx, simt = both(P, pb, rhs_block=block)
+    assert rel(fx, simt) <= 64 * 600 * EPS  # paths of at most 600 columns
+    ref = oracle.OracleFactor.from_problem(pb).inv_diag()
+    assert rel(fx, ref) <= 1e-10
+
+
+@pytest.mark.parametrize("count", [1, 16, 17, 333, 2500])
+def test_index_subsets(P, count):
+    pb = generate(scaled(SCALE, 1500, seed=3))
+    idx = np.random.default_rng(count).permutation(pb.n)[:count].astype(np.int32)
+    fx, simt = both(P, pb, idx=idx)
+    assert rel(fx, simt) <= 64 * 600 * EPS
+
+
+def test_wide_front_and_repeat(P):
+    """A sky front of many chunks; two calls give the same bits (fixed summation order)."""
+    pb = generate(sky_scaled(600, 3.0, 12))
+    s = P.Solver.for_problem(pb)
+    s.factor(pb.values)
+    a, b = s.diag_inverse(), s.diag_inverse()
+    assert np.array_equal(a, b)
+    f = oracle.OracleFactor.from_problem(pb)
+    assert rel(a, f.inv_diag()) <= 1e-10
+
+
+def test_badly_scaled_columns(P):
+    """N' = S N S with S over 40 powers of ten: the variances are those of N over S^2, as
+    closely as the SIMT kernel gives them (the scaling by powers of two keeps the fixed-point grids on
+    the entries' own scale)."""
+    pb = generate(scaled(SCALE, 1000, seed=7))
+    s = 10.0 ** np.random.default_rng(1).uniform(-20, 20, pb.n)
+    col = np.repeat(np.arange(pb.n), np.diff(pb.colptr))
+    values = pb.values * s[col] * s[pb.rowind]
+    fx, simt = both(P, pb, values=values)
+    assert rel(fx, simt) <= 64 * 600 * EPS
+    ref = oracle.OracleFactor.from_problem(pb).inv_diag() / s ** 2
+    assert rel(fx, ref) <= 1e-10
+
+
+def test_fp64_bands_and_forest(P):
+    bands = generate_bands(scaled(BAND, 700, seed=2), 3)
+    s = P.Solver(bands.n, bands.colptr, bands.rowind, batch=3)
+    s.factor_batch(bands.values)
+    v = s.diag_inverse_batch().reshape(3, -1)
+    for k in range(3):
+        assert rel(v[k], oracle.OracleFactor.from_problem(bands.band(k)).inv_diag()) <= 1e-10
+    probs = [random_spd(m, 0.2, m) for m in (3, 40, 150)]
+    s = P.Solver.for_problems(probs)
+    s.factor(np.concatenate([p.values for p in probs]))
+    v = s.diag_inverse()
+    assert rel(v, np.concatenate([oracle.OracleFactor.from_problem(p).inv_diag() for p in probs])) <= 1e-10
+
+
+@pytest.mark.parametrize("count", [1, 16, 40, 512])
+def test_inverse_block_on_the_scaled_vectors(P, count):
+    pb = generate(scaled(SCALE, 1200, seed=9))
+    idx = np.sort(np.random.default_rng(count).permutation(pb.n)[:count]).astype(np.int32)
+    s = P.Solver.for_problem(pb)
+    s.factor(pb.values)
+    G = s.inverse_block(idx)
+    R = oracle.OracleFactor.from_problem(pb).inv_block(idx)
+    d = np.sqrt(np.diag(R))
+    assert np.abs(G - R).max() <= 1e-10 * np.abs(R).max()
+    assert (np.abs(G - R) / np.outer(d, d)).max() <= 64 * 600 * EPS + 1e-10
