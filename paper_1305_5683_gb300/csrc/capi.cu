@@ -140,8 +140,10 @@ struct spi_ctx {
     // variances of the FP64 form on the tensor cores: set up at the first variance call
     // (-1: not yet, 0: not in use, 1: ready)
     int fx_state = -1;
-    DiagFxHost fx_h;
     DevDiagFx fx;
+    DiagFxHost fx_h;
+    // the FP64 form's inverted diagonal tiles (made at the end of every factorization)
+    DevTileInv ti;
     double last_diag_tc_flops = 0;
     // the mixed solve's plan with 128-column steps for those supernodes (their inverted
     // diagonal tiles); the FP64-panel paths keep SP
@@ -302,13 +304,32 @@ int ensure_device(spi_ctx* c) {
             t.ntc = h.ntc;
             t.npt = h.npt;
             t.ndt = h.ndt;
-            t.bands = (int)nb;
+                    t.bands = (int)nb;
             build_solve_plan(S, c->SPw, c->opt.batch, h.tc.data());
             CK(dev_upload(c, &c->d_fwd_items_w, c->SPw.fwd_items));
             CK(dev_upload(c, &c->d_bwd_items_w, c->SPw.bwd_items));
-            c->wa = WideArgs{t.xinv, t.xptr, (int64_t)diag_tc_xinv_floats(h.ndt)};
+            c->wa = WideArgs{t.xinv, t.xptr, (int64_t)diag_tc_xinv_floats(h.ndt), nullptr, nullptr, nullptr, 0};
             c->wide_ready = true;
         }
+    }
+    if (!mixed_of(c) && !c->opt.pivoting && S.n > 0) {
+        build_diag_fx(S, c->fx_h);
+        const DiagFxHost& h = c->fx_h;
+        DevTileInv& t = c->ti;
+        t = DevTileInv();
+        CK(dev_upload(c, &t.dtiles, h.dtiles));
+        CK(dev_upload(c, &t.xoff, h.xoff));
+        CK(dev_upload(c, &t.xptr, h.xptr));
+        CK(dev_alloc(c, &t.xinv, (size_t)h.nx * nb));
+        CK(dev_alloc(c, &t.xinvt, (size_t)h.nx * nb));
+        t.ncta = (int64_t)h.dtiles.size() / 4;
+        t.nx = h.nx;
+        const std::vector<uint8_t> every((size_t)S.ns, 1);
+        build_solve_plan(S, c->SPw, c->opt.batch, every.data(), true);
+        CK(dev_upload(c, &c->d_fwd_items_w, c->SPw.fwd_items));
+        CK(dev_upload(c, &c->d_bwd_items_w, c->SPw.bwd_items));
+        c->wa = WideArgs{nullptr, t.xptr, 0, t.xinv, t.xinvt, t.xoff, t.nx};
+        c->wide_ready = true;
     }
     c->dev_ready = true;
     return SPI_OK;
@@ -324,9 +345,8 @@ void free_fx(DevDiagFx& t) {
 int ensure_fx(spi_ctx* c) {
     if (c->fx_state >= 0) return SPI_OK;
     c->fx_state = 0;
-    if (mixed_of(c) || c->opt.pivoting || c->opt.diag_tc_min_pivots < 0 || c->S.n == 0) return SPI_OK;
-    DiagFxHost& h = c->fx_h;
-    build_diag_fx(c->S, h);
+    if (!c->ti.xinv || c->opt.diag_tc_min_pivots < 0 || c->S.n == 0) return SPI_OK;
+    const DiagFxHost& h = c->fx_h;
     DevDiagFx& t = c->fx;
     t = DevDiagFx();
     const size_t nb = (size_t)c->opt.batch, n = (size_t)c->S.n;
@@ -337,11 +357,9 @@ int ensure_fx(spi_ctx* c) {
         if (e == cudaSuccess) e = dev_upload(c, &t.tptr, h.tptr, tr);
         if (e == cudaSuccess) e = dev_upload(c, &t.tiles, h.tiles, tr);
         if (e == cudaSuccess) e = dev_upload(c, &t.tdiag, h.tdiag, tr);
-        if (e == cudaSuccess) e = dev_upload(c, &t.dtiles, h.dtiles, tr);
         if (e == cudaSuccess) e = dev_alloc(c, &t.pack, diag_fx_pack_bytes(h.npieces) * nb, tr);
         if (e == cudaSuccess) e = dev_alloc(c, &t.rexp, (size_t)h.ntiles * kFxRows * nb, tr);
         if (e == cudaSuccess) e = dev_alloc(c, &t.fr, n * nb, tr);
-        if (e == cudaSuccess) e = dev_alloc(c, &t.xinv, (size_t)h.ndt * kFxRows * kFxRows * nb, tr);
         return e;
     };
     const cudaError_t e = alloc();
@@ -355,7 +373,6 @@ int ensure_fx(spi_ctx* c) {
     CK(diag_fx_setup());
     t.npieces = h.npieces;
     t.ntiles = h.ntiles;
-    t.ndt = h.ndt;
     c->fx_state = 1;
     return SPI_OK;
 }
@@ -386,12 +403,10 @@ int upload_plan(spi_ctx* c, const DiagPlan& h, DevDiagPlan& d) {
     d.zsize = h.zbase.empty() ? 0 : h.zbase.back();
     d.fx = c->fx_state == 1 && (h.B == 16 || h.B == 32 || h.B == kFxMaxBlock);
     if (d.fx) {
-        std::vector<int32_t> tiles, dts;
-        diag_fx_used(c->S, c->fx_h, h, tiles, dts);
+        std::vector<int32_t> tiles;
+        diag_fx_used(c->S, c->fx_h, h, tiles);
         d.fx_ntiles = (int64_t)tiles.size();
-        d.fx_ndt = (int64_t)dts.size();
         CK(dev_upload(c, &d.fx_tiles, tiles, tr));
-        CK(dev_upload(c, &d.fx_dts, dts, tr));
     }
     // FP64 elements per band are enough for both element types
     CK(dev_alloc(c, &d.Z, (size_t)std::max<int64_t>(d.zsize, 1) * (size_t)c->opt.batch, tr));
@@ -846,6 +861,7 @@ void reset_device(spi_ctx* c) {
     c->bg = spi_ctx::Background();
     c->nrm = spi_ctx::Normal();
     c->dtc = DevDiagTc();
+    c->ti = DevTileInv();
     c->wide_ready = false;
     c->dev_ready = false;
     c->factor_plan_ready = false;
@@ -1046,6 +1062,8 @@ int factor_impl(spi_ctx* c, int nb, const double* values, int values_on_device, 
         if (mixed) launch_to_f64(c->d_L32, c->d_L, S.lptr[S.ns] * nb, s2);
         // the variances' tensor-core operands (inverted diagonal tiles, packed TF32 pairs)
         if (mixed) launch_diag_tc_pack(c->dsym, c->dtc, c->d_L32, nb, c->bs, s2);
+        // the FP64 form's inverted diagonal tiles (solves, variances)
+        if (c->ti.xinv) launch_tile_inverses(c->dsym, c->ti, c->d_L, nb, c->bs, s2);
     }));
     rc = finish(c, st);
     if (rc == SPI_OK) {
@@ -1075,7 +1093,7 @@ cudaError_t solve_core(spi_ctx* c, int nb, const double* b, double* x, cudaStrea
         // the mixed form's solves read its FP32 panels (the FP64 copy holds the same values)
         // and take 128-column steps where the factorization left inverted diagonal tiles
         const float* L32 = mixed_of(c) ? c->d_L32 : nullptr;
-        const bool wide = L32 && c->wide_ready;
+        const bool wide = c->wide_ready;
         const SolvePlan& P = wide ? c->SPw : c->SP;
         const int32_t* fi = wide ? c->d_fwd_items_w : c->d_fwd_items;
         const int32_t* bi = wide ? c->d_bwd_items_w : c->d_bwd_items;
@@ -1106,7 +1124,7 @@ int choose_solve_form(spi_ctx* c, int nb, const double* bd, cudaStream_t st) {
     }
     const bool timing = c->opt.autotune > 0 || (c->opt.autotune == 0 && c->S.factor_flops >= 2e8);
     if (!timing || c->SP.dag.empty()) {
-        c->solve_dag = c->SP.dag.empty() ? 0 : 1;
+        c->solve_dag = c->SP.dag.empty() || c->wide_ready ? 0 : 1;
         return SPI_OK;
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1212,7 +1230,7 @@ void launch_diag(spi_ctx* c, const DevDiagPlan& p, int nb, int64_t nout, double*
                                 tc ? c->dtc.tc : nullptr, st);
         if (tc) launch_diag_inv_tc(c->dsym, p, c->dtc, c->d_D, out, nb, bs, c->d_status, c->opt.wait_limit, st);
     } else {
-        if (p.fx) launch_diag_fx(c->dsym, p, c->fx, c->d_L, c->d_D, out, nb, bs, c->d_status, st);
+        if (p.fx) launch_diag_fx(c->dsym, p, c->fx, c->ti, c->d_L, c->d_D, out, nb, bs, c->d_status, st);
         else launch_diag_inverse(dev_sol(c), p, c->d_L, c->d_D, out, nb, bs, c->diag_smem_pad, st);
     }
 }
@@ -1711,8 +1729,8 @@ int inverse_block_impl(spi_ctx* c, std::vector<int32_t>& key, double* od, cudaSt
         c->plan_blk_key.swap(key);
         c->plan_blk_ready = true;
     }
-    launch_inverse_block(c->dsym, c->plan_blk, c->fx_state == 1 ? &c->fx : nullptr, c->d_L, c->d_D, c->d_out,
-                         c->d_zg, c->blk_rows, od, nidx, c->d_status, st);
+    launch_inverse_block(c->dsym, c->plan_blk, c->fx_state == 1 ? &c->fx : nullptr, c->ti, c->d_L, c->d_D,
+                         c->d_out, c->d_zg, c->blk_rows, od, nidx, c->d_status, st);
     return SPI_OK;
 }
 }  // namespace
@@ -2521,10 +2539,11 @@ int spi_info(const spi_ctx* c, spi_stats* o) {
     o->tune_schur_buckets = c->tune_schur_buckets;
     o->tune_schur_tc = c->tune_schur_tc;
     int64_t ls = 0;
-    for (const Launch& l : c->SP.fwd_launches) ls += l.count > 0;
-    for (const Launch& l : c->SP.bwd_launches) ls += l.count > 0;
+    const SolvePlan& sp = c->wide_ready ? c->SPw : c->SP;
+    for (const Launch& l : sp.fwd_launches) ls += l.count > 0;
+    for (const Launch& l : sp.bwd_launches) ls += l.count > 0;
     o->launches_solve = S.n ? 2 + ls : 0;
-    o->launches_diag = S.n ? 1 : 0;
+    o->launches_diag = S.n ? (c->fx_state == 1 || c->dtc.ntc > 0 ? 2 : 1) : 0;
     o->refine_steps = c->refine_steps;
     o->solve_relres = c->solve_relres;
     o->rhs_block = c->rhs_block_used > 0 ? c->rhs_block_used : c->opt.rhs_block;

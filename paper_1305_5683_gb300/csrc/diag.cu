@@ -486,7 +486,7 @@ __global__ void k_gather_blocks(const double* __restrict__ Z, int B, const int64
 
 }  // namespace
 
-void launch_inverse_block(const DevSym& d, const DevDiagPlan& p, const DevDiagFx* fx, const double* L, const double* D,
+void launch_inverse_block(const DevSym& d, const DevDiagPlan& p, const DevDiagFx* fx, const DevTileInv& x, const double* L, const double* D,
                           double* var_scratch, double* Zg, int64_t R, double* out, int64_t ldo, DevStatus* status,
                           cudaStream_t st) {
     if (p.nblocks == 0 || p.nrhs == 0) return;
@@ -496,7 +496,7 @@ void launch_inverse_block(const DevSym& d, const DevDiagPlan& p, const DevDiagFx
     bs.n = d.n;
     cudaMemsetAsync(Zg, 0, (size_t)R * (size_t)p.nrhs * sizeof(double), st);
     const bool tc = fx && p.fx;
-    if (tc) launch_diag_fx(d, p, *fx, L, D, var_scratch, 1, bs, status, st);
+    if (tc) launch_diag_fx(d, p, *fx, x, L, D, var_scratch, 1, bs, status, st);
     else launch_t<double>(d, p, L, D, var_scratch, 1, bs, 0, st);
     k_gather_blocks<<<p.nblocks, 256, 0, st>>>(p.Z, p.B, p.zbase, p.blk_ptr, p.rowmap, p.nrhs, Zg);
     const int nt = (int)((p.nrhs + kT - 1) / kT);

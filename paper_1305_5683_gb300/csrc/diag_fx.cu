@@ -24,7 +24,7 @@
 // Per block of B <= 64 right-hand sides one CTA walks the supernodes of the
 // block's paths.  Per supernode and 128-column chunk g: the incoming values of the chunk's rows are cut into digits in
 // shared memory and multiplied by the inverse of the chunk's 128 x 128
-// diagonal tile (k_fx_tinv, FP64), which gives the chunk's y; y is cut into
+// diagonal tile (k_fx_tinv, FP64, at the end of the factorization), which gives the chunk's y; y is cut into
 // digits, its squares are added to the variances in FP64, and the front's
 // remaining rows are updated 128 at a time, Z_rows -= S^-1 L S y
 // (Z, the block's workspace, holds S^-1 times the solves' vectors throughout).  The
@@ -166,15 +166,16 @@ __device__ __forceinline__ double fx_pow2(int e) { return __hiloint2double((1023
 // vectors down the 32-row blocks, lane = row, two columns per warp.  Bound by the FP64
 // pipe (64 cycles per warp instruction) and the chain of columns, so a tile is spread
 // over w / 8 CTAs, every step is two independent multiply-adds per warp, and the values
-// passed between steps are shuffled or read from shared memory.  (One column per warp
+// passed between steps are shuffled or read from shared memory.  X's transpose is stored too.  (One column per warp
 // was quicker for one small front, 21 against 27 us, but 354 against 193 us for all of
 // P = 20,000.)
 __global__ void __launch_bounds__(128) k_fx_tinv(DevSym d, const int32_t* __restrict__ dtiles,
-                                                 const int32_t* __restrict__ list, int64_t ndt,
-                                                 const double* __restrict__ L, double* __restrict__ xinv, int64_t bsL) {
+                                                 const int64_t* __restrict__ xoff, int64_t nx,
+                                                 const double* __restrict__ L, double* __restrict__ xinv,
+                                                 double* __restrict__ xinvt, int64_t bsL) {
     static_assert(kFxInvCols == 8, "two columns for each of the four warps");
     L += blockIdx.y * bsL;
-    const int32_t* dt = dtiles + 4 * (int64_t)list[blockIdx.x];
+    const int32_t* dt = dtiles + 4 * (int64_t)blockIdx.x;
     const int s = dt[0], g = dt[1], q0 = dt[3];
     const int64_t t = dt[2];
     const int k = d.sfirst[s + 1] - d.sfirst[s];
@@ -183,15 +184,16 @@ __global__ void __launch_bounds__(128) k_fx_tinv(DevSym d, const int32_t* __rest
     const double* P = L + d.lptr[s] + c0 + (int64_t)c0 * m;  // the tile, leading dimension m
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int col = q0 + 2 * warp;
-    double* X = xinv + ((int64_t)blockIdx.y * ndt + t) * (kFxRows * kFxRows);  // column-major
+    double* X = xinv + (int64_t)blockIdx.y * nx + xoff[t];  // column-major, leading dimension w
+    double* Xt = xinvt + (int64_t)blockIdx.y * nx + xoff[t];  // its transpose
     __shared__ double xs[4][kFxRows][2];
     double (*x)[2] = xs[warp];
     if (col >= w) return;
     const bool two = col + 1 < w;
     const int jb = col / 32;
     for (int r = lane; r < 32 * jb; r += 32) {  // above the columns' own block
-        X[r + col * kFxRows] = 0.0;
-        if (two) X[r + (col + 1) * kFxRows] = 0.0;
+        X[r + col * w] = Xt[col + r * w] = 0.0;
+        if (two) X[r + (col + 1) * w] = Xt[col + 1 + r * w] = 0.0;
     }
     for (int i = jb; 32 * i < w; ++i) {
         const int r = 32 * i + lane;
@@ -222,8 +224,8 @@ __global__ void __launch_bounds__(128) k_fx_tinv(DevSym d, const int32_t* __rest
         x[r][0] = a0;
         x[r][1] = a1;
         __syncwarp();
-        if (on) X[r + col * kFxRows] = a0;
-        if (on && two) X[r + (col + 1) * kFxRows] = a1;
+        if (on) X[r + col * w] = Xt[col + r * w] = a0;
+        if (on && two) X[r + (col + 1) * w] = Xt[col + 1 + r * w] = a1;
     }
 }
 
@@ -237,7 +239,8 @@ __global__ void __launch_bounds__(128) k_fx_tinv(DevSym d, const int32_t* __rest
 __global__ void __launch_bounds__(kFxRows) k_fx_pack(DevSym d, const int32_t* __restrict__ tiles,
                                                      const int32_t* __restrict__ tdiag,
                                                      const int32_t* __restrict__ list, int64_t ntiles, int64_t npieces,
-                                                     int64_t ndt, const double* __restrict__ L,
+                                                     const int64_t* __restrict__ xoff, int64_t nx,
+                                                     const double* __restrict__ L,
                                                      const double* __restrict__ D, const double* __restrict__ xinv,
                                                      unsigned char* __restrict__ pack, int32_t* __restrict__ rexp,
                                                      double* __restrict__ fr, int64_t bsL, int64_t bsn) {
@@ -254,9 +257,9 @@ __global__ void __launch_bounds__(kFxRows) k_fx_pack(DevSym d, const int32_t* __
     bool on;
     int pivot;  // of this row
     if (i == 0) {
-        src = xinv + ((int64_t)band * ndt + tdiag[t]) * (kFxRows * kFxRows) + tid;
-        ld = kFxRows;
         on = tid < w;
+        src = xinv + (int64_t)band * nx + xoff[tdiag[t]] + (on ? tid : 0);
+        ld = w;
         pivot = f + c0 + tid;
     } else {
         const int64_t row = min(c0 + kFxRows, k) + (int64_t)(i - 1) * kFxRows + tid;
@@ -690,12 +693,18 @@ cudaError_t diag_fx_setup() {
     return cudaFuncSetAttribute(k_diag_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fx_smem(kFxMaxBlock));
 }
 
-void launch_diag_fx(const DevSym& d, const DevDiagPlan& dp, const DevDiagFx& p, const double* L, const double* D,
+void launch_tile_inverses(const DevSym& d, const DevTileInv& x, const double* L, int nb, const Strides& bs,
+                          cudaStream_t st) {
+    if (x.ncta == 0 || nb == 0) return;
+    k_fx_tinv<<<dim3((unsigned)x.ncta, nb), 128, 0, st>>>(d, x.dtiles, x.xoff, x.nx, L, x.xinv, x.xinvt, bs.L);
+}
+
+void launch_diag_fx(const DevSym& d, const DevDiagPlan& dp, const DevDiagFx& p, const DevTileInv& x, const double* L, const double* D,
                     double* out, int nb, const Strides& bs, DevStatus* status, cudaStream_t st) {
     if (dp.nblocks == 0 || nb == 0) return;
-    k_fx_tinv<<<dim3((unsigned)dp.fx_ndt, nb), 128, 0, st>>>(d, p.dtiles, dp.fx_dts, p.ndt, L, p.xinv, bs.L);
     k_fx_pack<<<dim3((unsigned)dp.fx_ntiles, nb), kFxRows, 0, st>>>(d, p.tiles, p.tdiag, dp.fx_tiles, p.ntiles, p.npieces,
-                                                                    p.ndt, L, D, p.xinv, p.pack, p.rexp, p.fr, bs.L, bs.n);
+                                                                    x.xoff, x.nx, L, D, x.xinv, p.pack, p.rexp, p.fr,
+                                                                    bs.L, bs.n);
     FxArgs a{dp.B, dp.order, dp.blk_ptr, dp.uptr, dp.us, dp.ulo, dp.uhi, dp.uzoff, dp.rel, dp.rhs_out,
              dp.rhs_zrow, dp.rhs_col, dp.urel, dp.zbase, dp.Z, p.pptr, p.tptr, p.npieces, p.ntiles, p.pack, p.rexp,
              D, p.fr};

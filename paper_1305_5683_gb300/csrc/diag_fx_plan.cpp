@@ -13,9 +13,12 @@ void build_diag_fx(const Symbolic& S, DiagFxHost& h) {
         const int32_t k = S.k_of(s), m = S.m_of(s);
         h.pptr[s] = h.npieces;
         h.tptr[s] = h.ntiles;
+        h.xptr.push_back(h.ndt);
         for (int32_t g = 0; g * kFxRows < k; ++g) {
             const int32_t w = std::min(kFxRows, k - g * kFxRows), base = std::min(kFxRows * (g + 1), k);
             const int32_t np = (w + kFxSub - 1) / kFxSub, nt = 1 + (m - base + kFxRows - 1) / kFxRows;
+            h.xoff.push_back(h.nx);
+            h.nx += (int64_t)w * w;
             for (int32_t c = 0; c < w; c += kFxInvCols) h.dtiles.insert(h.dtiles.end(), {s, g, h.ndt, c});
             for (int32_t i = 0; i < nt; ++i) {
                 h.tiles.insert(h.tiles.end(), {s, g, i, (int32_t)h.npieces});
@@ -28,16 +31,12 @@ void build_diag_fx(const Symbolic& S, DiagFxHost& h) {
     }
 }
 
-void diag_fx_used(const Symbolic& S, const DiagFxHost& h, const DiagPlan& dp, std::vector<int32_t>& tiles,
-                  std::vector<int32_t>& dts) {
+void diag_fx_used(const Symbolic& S, const DiagFxHost& h, const DiagPlan& dp, std::vector<int32_t>& tiles) {
     std::vector<uint8_t> used(S.ns, 0);
     for (int32_t s : dp.us) used[s] = 1;
     tiles.clear();
-    dts.clear();
     for (size_t t = 0; 4 * t < h.tiles.size(); ++t)
         if (used[h.tiles[4 * t]]) tiles.push_back((int32_t)t);
-    for (size_t t = 0; 4 * t < h.dtiles.size(); ++t)
-        if (used[h.dtiles[4 * t]]) dts.push_back((int32_t)t);
 }
 
 }  // namespace spi

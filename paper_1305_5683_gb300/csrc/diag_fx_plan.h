@@ -22,15 +22,16 @@ struct DiagFxHost {
                                   //   diagonal tile's inverse, i > 0: rows base + 128 (i - 1) ..), first piece
     std::vector<int32_t> dtiles;  // [][4]: supernode, chunk, number of the diagonal tile, first of 8 columns
     std::vector<int32_t> tdiag;   // [ntiles]: the diagonal tile's number (i = 0), else -1
+    std::vector<int64_t> xoff;    // [ndt] offset of the diagonal tile's inverse (w x w, column-major)
+    std::vector<int32_t> xptr;    // [ns] first diagonal tile of the supernode
+    int64_t nx = 0;               // doubles of all inverses (per band)
 };
 
 // Every supernode; per 128-column chunk g of a supernode (k pivots, m rows): the inverse of its
 // unit-lower diagonal tile, then the rows from min(128 (g + 1), k) to m in
 // tiles of 128, each tile in ceil(w / 16) pieces (w the chunk's columns).
 void build_diag_fx(const Symbolic& S, DiagFxHost& h);
-// the tiles and diagonal-tile columns (positions in h.tiles / 4, h.dtiles / 4) of the
-// supernodes that plan dp walks
-void diag_fx_used(const Symbolic& S, const DiagFxHost& h, const DiagPlan& dp, std::vector<int32_t>& tiles,
-                  std::vector<int32_t>& dts);
+// the tiles (positions in h.tiles / 4) of the supernodes that plan dp walks
+void diag_fx_used(const Symbolic& S, const DiagFxHost& h, const DiagPlan& dp, std::vector<int32_t>& tiles);
 
 }  // namespace spi

@@ -1,6 +1,7 @@
 // solve.cu -- solution phase (paper Sec. 3.2.3): forward substitution
 // z = L^-1 P b bottom-up over the supernodal tree, then x = P^T L^-T D^-1 z
-// top-down.  One launch per tree level; one CTA per supernode.
+// top-down: per tree level a chain of short launches, one per block of 32, 64 or 128
+// columns, each started while the one before it runs (launch_chained).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -12,16 +13,17 @@ namespace spi {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kFwdRows = 512;  // rows below the block per forward CTA
+constexpr int kFwdRows = 512;  // rows below the block per forward task (dependency-driven launch)
+constexpr int kStepRows = 128; // rows below the block per CTA of k_fwd_step
 constexpr int kBwdCols = 256;  // columns per backward CTA
-// In a batch of bands, a level runs each sweep in one launch, one CTA per
-// (supernode, band) looping over the supernode's 32-column steps, when its
-// largest supernode's work (k m - k^2 / 2 FMAs, on one SM) is below what the
-// launch-per-step form spends on its chain of launches (about 10 us each,
-// ~20,000 FMAs of one SM).  For a single problem the launch-per-step form
-// measured faster at every level (its rows spread over more CTAs), so it
-// keeps that form; so do the wide fronts near the root.
-constexpr int64_t kFuseFmaPerStep = 20000;
+// In a batch of bands, a level whose supernodes all have at most kFuseCols columns runs
+// each sweep in one launch, one CTA per (supernode, band).  With more columns the CTA
+// would walk its 32-column steps one after another while the launch-per-step form, whose
+// wide steps spread a front over many CTAs, is quicker from 2 to 48 bands (P = 5,000, one
+// refined solve, fronts fused up to 20,000 products per step / up to 32 columns / never:
+// 2 bands 1.53 / 0.67 / 0.68 ms, 16 bands 3.45 / 2.43 / 2.51, 48 bands 6.74 / 6.15 / 6.48).
+// A single problem keeps the launch-per-step form at every level.
+constexpr int32_t kFuseCols = 32;
 constexpr int kAncRegs = 4;  // ancestor rows per thread whose updates are summed in registers
 
 __global__ void k_permute_in(int32_t n, const int32_t* __restrict__ perm, const double* __restrict__ b,
@@ -43,9 +45,9 @@ __global__ void k_permute_out(int32_t n, const int32_t* __restrict__ perm, const
 // (D^-1 z) at pivot j: z_j / d_j, or, for a symmetric indefinite factorization,
 // D^-1 taken block by block (the 2x2 partner's z is final after the forward sweep).
 __device__ __forceinline__ double dinv_z(const DevSym& d, const double* z, const double* D, int j) {
-    if (!d.dinv_a) return z[j] / D[j];
+    if (!d.dinv_a) return __ldcg(z + j) / D[j];
     const int q = d.pair[j];
-    return d.dinv_a[j] * z[j] + (q >= 0 ? d.dinv_b[j] * z[q] : 0.0);
+    return d.dinv_a[j] * __ldcg(z + j) + (q >= 0 ? d.dinv_b[j] * __ldcg(z + q) : 0.0);
 }
 
 // Rows of x gathered per pass of the backward first pass (x[rows[t]] for a chunk of
@@ -112,102 +114,127 @@ __device__ void bwd_update(const TL* P, int64_t m, int cb, int wb, const TL* xb,
 // every CTA of supernode s solves the 32 x 32 unit-lower diagonal block
 // x_b = L_bb^-1 w_b in registers (lane r owns row r), the chunk-0 CTA stores
 // x_b into z, and each CTA subtracts L(rows, block b) x_b from its own chunk
-// of the rows below: the supernode's later pivots (plain stores: the rows of
-// a chunk belong to one CTA) and its ancestors' rows (atomics: siblings of
-// the level update the same ancestors).
+// of the rows below (two threads per row, their part of L loaded first): the
+// supernode's later pivots (plain stores: the rows of a chunk belong to one CTA) and
+// its ancestors' rows (atomics: siblings of the level update the same ancestors).
 template <typename TL>
 __global__ void __launch_bounds__(kThreads) k_fwd_step(DevSym d, const int32_t* __restrict__ items, int b,
-                                                       const TL* __restrict__ L, double* __restrict__ w,
-                                                       double* __restrict__ z, Strides bs) {
+                                                       const TL* __restrict__ L, double* w,
+                                                       double* z, Strides bs) {
     L += blockIdx.y * bs.L;
     w += blockIdx.y * bs.n;
     z += blockIdx.y * bs.n;
-    __shared__ TL xb[kT];
-    const int tid = threadIdx.x, lane = tid & 31;
+    __shared__ TL xb[kT], part[kStepRows];
+    static_assert(kThreads == 2 * kStepRows, "two threads per row");
+    const int tid = threadIdx.x, lane = tid & 31, h = tid / kStepRows;
     const int s = items[2 * blockIdx.x], chunk = items[2 * blockIdx.x + 1];
     const int f = d.sfirst[s], k = d.sfirst[s + 1] - f;
     const int64_t m = d.srowptr[s + 1] - d.srowptr[s];
     const TL* P = L + d.lptr[s];
     const int cb = b * kT, wb = min(kT, k - cb);
+    const int64_t r = cb + wb + (int64_t)chunk * kStepRows + tid % kStepRows;
+    TL l[kT / 2];
+#pragma unroll
+    for (int q = 0; q < kT / 2; ++q) l[q] = (r < m && 2 * q + h < wb) ? P[r + (int64_t)(cb + 2 * q + h) * m] : TL(0);
+    const int32_t row = r < m ? d.srows[d.srowptr[s] + r] : 0;
     if (tid < 32) {
-        // lane r holds row r of the diagonal block: 32 independent loads first
+        // lane r holds row r of the diagonal block
         TL lrow[kT];
 #pragma unroll
         for (int c = 0; c < kT; ++c)
-            lrow[c] = (c < lane && lane < wb) ? P[(cb + lane) + (int64_t)(cb + c) * m] : 0.0;
-        TL x = lane < wb ? (TL)w[f + cb + lane] : TL(0);
+            lrow[c] = (c < lane && lane < wb) ? P[(cb + lane) + (int64_t)(cb + c) * m] : TL(0);
+        chain_wait();
+        chain_next();
+        TL x = lane < wb ? (TL)__ldcg(w + f + cb + lane) : TL(0);
 #pragma unroll
         for (int c = 0; c < kT - 1; ++c) {
+            if (c + 1 >= wb) break;
             const TL xc = __shfl_sync(0xffffffffu, x, c);
             x -= lrow[c] * xc;
         }
         xb[lane] = x;
         if (chunk == 0 && lane < wb) z[f + cb + lane] = x;
+    } else {
+        chain_wait();
+        chain_next();
     }
     __syncthreads();
-    const int32_t* rows = d.srows + d.srowptr[s];
-    const int64_t r0 = cb + wb + (int64_t)chunk * kFwdRows;
-    const int64_t r1 = (m < r0 + kFwdRows) ? m : r0 + kFwdRows;
-    for (int64_t r = r0 + tid; r < r1; r += kThreads) {
-        TL acc = 0;
-#pragma unroll 8
-        for (int c = 0; c < wb; ++c) acc += P[r + (int64_t)(cb + c) * m] * xb[c];
-        if (r < k) w[f + r] -= acc;
-        else atomicAdd(w + rows[r], -(double)acc);
+    TL acc = 0;
+#pragma unroll
+    for (int q = 0; q < kT / 2; ++q) {
+        if (2 * q >= wb) break;
+        acc += l[q] * xb[2 * q + h];
+    }
+    if (h == 1) part[tid - kStepRows] = acc;
+    __syncthreads();
+    if (h == 0 && r < m) {
+        acc += part[tid];
+        if (r < k) w[f + r] = __ldcg(w + f + r) - acc;
+        else atomicAdd(w + row, -(double)acc);
     }
 }
 
 // Backward, first launch of a level: y_c = z_c / d_c - sum_{t >= k} L[t][c] x[rows[t]]
-// for a chunk of 32 of the supernode's columns, stored into w.  Warp q takes
-// the columns q, q + 8, q + 16, q + 24 of the chunk; its lanes run over the
-// rows below (coalesced column reads, the gathered x shared by the four
-// columns) and a shuffle reduction finishes each dot product.  Four partial
-// sums per thread keep the kernel's registers low enough for several CTAs
-// per SM.
+// for kInitCols of the supernode's columns, stored into w: a warp per column, its lanes
+// over the rows below (coalesced column reads; the x of 2,048 rows at a time gathered into
+// shared memory while the first loads of L are in flight), then a shuffle reduction.
+constexpr int kInitCols = kThreads / 32;
 template <typename TL>
 __global__ void __launch_bounds__(kThreads) k_bwd_init(DevSym d, const int32_t* __restrict__ items,
                                                        const TL* __restrict__ L, const double* __restrict__ D,
-                                                       const double* __restrict__ z, const double* __restrict__ x,
-                                                       double* __restrict__ w, Strides bs) {
+                                                       const double* z, const double* x,
+                                                       double* w, Strides bs) {
     L += blockIdx.y * bs.L;
     D += blockIdx.y * bs.Dn;
     z += blockIdx.y * bs.n;
     x += blockIdx.y * bs.n;
     w += blockIdx.y * bs.n;
-    constexpr int kWarps = kThreads / 32, kPer = kT / kWarps;
+    constexpr int kAhead = 16;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int s = items[2 * blockIdx.x], chunk = items[2 * blockIdx.x + 1];
     const int f = d.sfirst[s], k = d.sfirst[s + 1] - f;
     const int64_t m = d.srowptr[s + 1] - d.srowptr[s];
-    const TL* P = L + d.lptr[s];
     const int32_t* rows = d.srows + d.srowptr[s];
-    const int c0 = chunk * kT, nc = min(kT, k - c0);
+    const int c = chunk * kInitCols + warp;
+    const bool on = c < k;
+    const TL* P = L + d.lptr[s] + (int64_t)(on ? c : 0) * m;
     __shared__ TL xs[kXs];
-    TL acc[kPer];
-#pragma unroll
-    for (int q = 0; q < kPer; ++q) acc[q] = 0.0;
+    double base = 0.0;
+    bool first = true;
+    if (m == k) {
+        chain_wait();
+        chain_next();
+        base = on ? dinv_z(d, z, D, f + c) : 0.0;
+    }
+    TL acc = TL(0);
     for (int64_t t0 = k; t0 < m; t0 += kXs) {
         const int64_t t1 = m < t0 + kXs ? m : t0 + kXs;
-        __syncthreads();
-        gather_x<false>(xs, x, rows, t0, t1);
-        __syncthreads();
-#pragma unroll 4
-        for (int64_t t = t0 + lane; t < t1; t += 32) {
-            const TL xv = xs[t - t0];
+        TL l[kAhead];
 #pragma unroll
-            for (int q = 0; q < kPer; ++q) {
-                const int c = warp + kWarps * q;
-                if (c < nc) acc[q] += P[t + (int64_t)(c0 + c) * m] * xv;
-            }
+        for (int q = 0; q < kAhead; ++q) {
+            const int64_t t = t0 + lane + 32 * q;
+            l[q] = (on && t < t1) ? P[t] : TL(0);
+        }
+        if (first) {
+            chain_wait();
+            chain_next();
+            base = on ? dinv_z(d, z, D, f + c) : 0.0;
+            first = false;
+        } else {
+            __syncthreads();
+        }
+        gather_x<true>(xs, x, rows, t0, t1);
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q)
+            if (t0 + lane + 32 * q < t1) acc += l[q] * xs[lane + 32 * q];
+        if (on) {
+#pragma unroll 8
+            for (int64_t t = t0 + lane + 32 * kAhead; t < t1; t += 32) acc += P[t] * xs[t - t0];
         }
     }
-#pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-        TL v = acc[q];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        const int c = warp + kWarps * q;
-        if (lane == 0 && c < nc) w[f + c0 + c] = dinv_z(d, z, D, f + c0 + c) - v;
-    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0 && on) w[f + c] = base - acc;
 }
 
 // Backward block step b (descending): every CTA solves L_bb^T x_b = y_b in
@@ -215,8 +242,8 @@ __global__ void __launch_bounds__(kThreads) k_bwd_init(DevSym d, const int32_t* 
 // earlier columns a < 32 b: y_a -= sum_r L[32b + r][a] x_b[r].
 template <typename TL>
 __global__ void __launch_bounds__(kThreads) k_bwd_step(DevSym d, const int32_t* __restrict__ items, int b,
-                                                       const TL* __restrict__ L, double* __restrict__ w,
-                                                       double* __restrict__ x, Strides bs) {
+                                                       const TL* __restrict__ L, double* w,
+                                                       double* x, Strides bs) {
     L += blockIdx.y * bs.L;
     w += blockIdx.y * bs.n;
     x += blockIdx.y * bs.n;
@@ -232,7 +259,9 @@ __global__ void __launch_bounds__(kThreads) k_bwd_step(DevSym d, const int32_t* 
         // lane c holds column c of the diagonal block (L_bb^T row c)
         TL lcol[kT];
         bwd_block_cols(P, m, cb, wb, Lbb, lcol, lane);
-        TL y = lane < wb ? (TL)w[f + cb + lane] : TL(0);
+        chain_wait();
+        chain_next();
+        TL y = lane < wb ? (TL)__ldcg(w + f + cb + lane) : TL(0);
 #pragma unroll
         for (int r = kT - 1; r > 0; --r) {
             const TL xr = __shfl_sync(0xffffffffu, y, r);
@@ -240,9 +269,12 @@ __global__ void __launch_bounds__(kThreads) k_bwd_step(DevSym d, const int32_t* 
         }
         xb[lane] = y;
         if (chunk == 0 && lane < wb) x[f + cb + lane] = y;
+    } else {
+        chain_wait();
+        chain_next();
     }
     __syncthreads();
-    bwd_update<1, false>(P, m, cb, wb, xb, chunk * kBwdCols, min(cb, (chunk + 1) * kBwdCols), w + f);
+    bwd_update<1, true>(P, m, cb, wb, xb, chunk * kBwdCols, min(cb, (chunk + 1) * kBwdCols), w + f);
 }
 
 // Forward sweep of one level in one launch: one CTA per (supernode, band)
@@ -483,99 +515,278 @@ __global__ void k_reciprocal(int32_t n, const double* __restrict__ D, double* __
 }
 
 // ---------------------------------------------------------------------------
-// Wide steps (mixed form): the supernodes whose variances run on the tensor
-// cores have, per 128 of their columns, the inverse X_bb of the unit-lower
-// diagonal block (prepared at the end of the factorization, FP32).  Their
-// sweeps then take 128 columns per step: forward x_b = X_bb w_b and then
+// Wide steps: per 128 columns of a supernode there is the inverse X_bb of the unit-lower
+// diagonal block (made at the end of the factorization: FP32 for the mixed form's
+// tensor-core supernodes, FP64 for every supernode of the FP64 form).  The sweeps take 128
+// columns per step (64 in FP64): forward x_b = X_bb w_b and then
 // w_below -= L(rows, block b) x_b; backward x_b = X_bb^T y_b and then
-// y_a -= sum_r L[128 b + r][a] x_b[r] for the earlier columns a.  The same
-// substitution in blocks of 128, a quarter of the 32-column steps on the chain.
+// y_a -= sum_r L[cb + r][a] x_b[r] for the earlier columns a.  The same substitution in
+// wider blocks, a quarter (half) of the 32-column steps on the chain.  A step's time is
+// its latency (load, product, store, the next launch), so a CTA takes few rows or columns
+// and its part of L is loaded before x_b is known: one solve of the mixed form at P =
+// 20,000 0.79 -> 0.54 ms against 256 rows or columns per CTA, read a few at a time, and
+// with the launches chained a refined one (three solves) 2.23 -> 1.75.
 constexpr int kW = 128;
-constexpr int kFwdRowsW = 256;  // rows below per wide forward CTA
-constexpr int kBwdColsW = 256;  // earlier columns per wide backward CTA
+constexpr int kFwdRowsW = 64;  // rows below per wide forward CTA
+constexpr int kBwdColsW = 64;  // earlier columns per wide backward CTA
 
-__global__ void __launch_bounds__(kThreads) k_fwd_wide(DevSym d, const int32_t* __restrict__ items, int b,
-                                                       const float* __restrict__ L, WideArgs wa,
-                                                       double* __restrict__ w, double* __restrict__ z, Strides bs) {
+// x = X_bb v (transposed: X_bb^T v) for the w x w inverse of step b, v and x in shared
+// memory (128 entries, v zero beyond w); ends with a barrier.
+__device__ __forceinline__ void wide_apply(const WideArgs& wa, int band, int s, int b, int w, const float* v, float* x,
+                                           float* part, bool transposed) {
+    const float* X = wa.xinv + band * wa.xband + (int64_t)(wa.xptr[s] + b) * (kW * kW);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (!transposed) {
+        // a warp per row (rows warp + 8 q), 16-byte loads, all of the warp's rows before the reductions
+        constexpr int kRowsPerWarp = kW / (kThreads / 32);
+        float4 xr[kRowsPerWarp];
+#pragma unroll
+        for (int q = 0; q < kRowsPerWarp; ++q) {
+            const int r = warp + (kThreads / 32) * q;
+            xr[q] = r < w ? *reinterpret_cast<const float4*>(X + r * kW + 4 * lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        const float w0 = v[4 * lane], w1 = v[4 * lane + 1], w2 = v[4 * lane + 2], w3 = v[4 * lane + 3];
+#pragma unroll
+        for (int q = 0; q < kRowsPerWarp; ++q) {
+            float y = xr[q].x * w0 + xr[q].y * w1 + xr[q].z * w2 + xr[q].w * w3;
+            for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+            if (lane == 0) x[warp + (kThreads / 32) * q] = y;
+        }
+    } else {
+        // column c by threads c (rows [0, 64)) and c + 128, coalesced over c
+        const int c = tid % kW, h = tid / kW;
+        float y = 0.f;
+        if (64 * h < w) {
+#pragma unroll 32
+            for (int r = 64 * h; r < 64 * h + 64; ++r) y += X[r * kW + c] * v[r];
+        }
+        if (h == 1) part[c] = y;
+        __syncthreads();
+        if (h == 0) x[c] = y + part[c];
+    }
+    __syncthreads();
+}
+__global__ void __launch_bounds__(kThreads, 2) k_fwd_wide(DevSym d, const int32_t* __restrict__ items, int b,
+                                                          const float* __restrict__ L, WideArgs wa,
+                                                          double* w, double* z, Strides bs) {
     const int band = blockIdx.y;
     L += band * bs.L;
     w += band * bs.n;
     z += band * bs.n;
-    __shared__ float wv[kW], xb[kW];
+    __shared__ float wv[kW], xb[kW], part[kThreads];
     const int s = items[2 * blockIdx.x], chunk = items[2 * blockIdx.x + 1];
     const int f = d.sfirst[s], k = d.sfirst[s + 1] - f;
     const int64_t m = d.srowptr[s + 1] - d.srowptr[s];
     const float* P = L + d.lptr[s];
     const int32_t* rows = d.srows + d.srowptr[s];
     const int cb = b * kW, wb = min(kW, k - cb);
-    const float* X = wa.xinv + band * wa.xband + (int64_t)(wa.xptr[s] + b) * (kW * kW);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int kRowsPerWarp = kW / (kThreads / 32);
-    // x_b[r] = sum_c X[r][c] w[c]: a warp per row (rows warp + 8 q), 16-byte loads of the
-    // row, all of the warp's rows loaded before the reductions
-    float4 xr[kRowsPerWarp];
+    const int tid = threadIdx.x;
+    // this thread's part of L: row tid % 64 of the chunk, a quarter of the columns
+    constexpr int kQ = kW / (kThreads / kFwdRowsW);
+    const int64_t r = cb + wb + (int64_t)chunk * kFwdRowsW + tid % kFwdRowsW;
+    const int q0 = tid / kFwdRowsW * kQ;
+    float l[kQ];
 #pragma unroll
-    for (int q = 0; q < kRowsPerWarp; ++q)
-        xr[q] = *reinterpret_cast<const float4*>(X + (warp + (kThreads / 32) * q) * kW + 4 * lane);
-    if (tid < kW) wv[tid] = tid < wb ? (float)w[f + cb + tid] : 0.f;
+    for (int c = 0; c < kQ; ++c) l[c] = (r < m && q0 + c < wb) ? P[r + (int64_t)(cb + q0 + c) * m] : 0.f;
+    const int32_t row = r < m ? rows[r] : 0;
+    chain_wait();
+    chain_next();
+    if (tid < kW) wv[tid] = tid < wb ? (float)__ldcg(w + f + cb + tid) : 0.f;
     __syncthreads();
-    {
-        const float w0 = wv[4 * lane], w1 = wv[4 * lane + 1], w2 = wv[4 * lane + 2], w3 = wv[4 * lane + 3];
-#pragma unroll
-        for (int q = 0; q < kRowsPerWarp; ++q) {
-            float v = xr[q].x * w0 + xr[q].y * w1 + xr[q].z * w2 + xr[q].w * w3;
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) xb[warp + (kThreads / 32) * q] = v;
-        }
-    }
-    __syncthreads();
+    wide_apply(wa, band, s, b, wb, wv, xb, part, false);
     if (chunk == 0 && tid < wb) z[f + cb + tid] = xb[tid];
-    const int64_t r0 = cb + wb + (int64_t)chunk * kFwdRowsW;
-    const int64_t r1 = m < r0 + kFwdRowsW ? m : r0 + kFwdRowsW;
-    for (int64_t r = r0 + tid; r < r1; r += kThreads) {
-        float acc = 0.f;
-#pragma unroll 16
-        for (int c = 0; c < wb; ++c) acc += P[r + (int64_t)(cb + c) * m] * xb[c];
-        if (r < k) w[f + r] -= acc;
-        else atomicAdd(w + rows[r], -(double)acc);
+    float acc = 0.f;
+#pragma unroll
+    for (int c = 0; c < kQ; ++c)
+        if (q0 + c < wb) acc += l[c] * xb[q0 + c];
+    part[tid] = acc;
+    __syncthreads();
+    if (tid < kFwdRowsW && r < m) {
+        float sum = part[tid];
+#pragma unroll
+        for (int q = 1; q < kThreads / kFwdRowsW; ++q) sum += part[tid + q * kFwdRowsW];
+        if (r < k) w[f + r] = __ldcg(w + f + r) - sum;
+        else atomicAdd(w + row, -(double)sum);
     }
 }
 
 // (at most 128 registers: its CTAs must fit beside a variance kernel's on one SM, since
 // the two run concurrently on two streams)
 __global__ void __launch_bounds__(kThreads, 2) k_bwd_wide(DevSym d, const int32_t* __restrict__ items, int b,
-                                                       const float* __restrict__ L, WideArgs wa,
-                                                       double* __restrict__ w, double* __restrict__ x, Strides bs) {
+                                                          const float* __restrict__ L, WideArgs wa,
+                                                          double* w, double* x, Strides bs) {
     const int band = blockIdx.y;
     L += band * bs.L;
     w += band * bs.n;
     x += band * bs.n;
-    __shared__ float yv[kW], xb[kW];
+    __shared__ float yv[kW], xb[kW], part[kThreads];
     const int s = items[2 * blockIdx.x], chunk = items[2 * blockIdx.x + 1];
     const int f = d.sfirst[s], k = d.sfirst[s + 1] - f;
     const int64_t m = d.srowptr[s + 1] - d.srowptr[s];
     const float* P = L + d.lptr[s];
     const int cb = b * kW, wb = min(kW, k - cb);
-    const float* X = wa.xinv + band * wa.xband + (int64_t)(wa.xptr[s] + b) * (kW * kW);
-    const int tid = threadIdx.x;
-    __shared__ float part[kW];
-    if (tid < kW) yv[tid] = tid < wb ? (float)w[f + cb + tid] : 0.f;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // this warp's part of L: 32 of the chunk's 64 columns, 32 of the block's rows (lane = row)
+    static_assert(kThreads / 32 == (kBwdColsW / 32) * (kW / 32), "a warp per 32 x 32 piece");
+    const int a0 = chunk * kBwdColsW + 32 * (warp & 1), rr = 32 * (warp >> 1) + lane;
+    float v[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = (a0 + j < cb && rr < wb) ? P[(cb + rr) + (int64_t)(a0 + j) * m] : 0.f;
+    chain_wait();
+    chain_next();
+    if (tid < kW) yv[tid] = tid < wb ? (float)__ldcg(w + f + cb + tid) : 0.f;
     __syncthreads();
-    // x_b[c] = sum_r X[r][c] y[r] (X is zero above its diagonal): column c by threads c
-    // (rows [0, 64)) and c + 128 (rows [64, 128)), coalesced over c, 16 loads in flight
-    static_assert(kThreads == 2 * kW, "two threads per column of the diagonal tile");
-    {
-        const int c = tid % kW, h = tid / kW;
-        float v = 0.f;
-#pragma unroll 16
-        for (int r = 64 * h; r < 64 * h + 64; ++r) v += X[r * kW + c] * yv[r];
-        if (h == 1) part[c] = v;
-        __syncthreads();
-        if (h == 0) xb[c] = v + part[c];
-    }
-    __syncthreads();
+    wide_apply(wa, band, s, b, wb, yv, xb, part, true);
     if (chunk == 0 && tid < wb) x[f + cb + tid] = xb[tid];
-    bwd_update<kW / 32, false>(P, m, cb, wb, xb, chunk * kBwdColsW, min(cb, (chunk + 1) * kBwdColsW), w + f);
+    if (cb == 0) return;
+    const float xr = rr < wb ? xb[rr] : 0.f;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] *= xr;
+    const float sum = lane_sums(v, lane);  // column a0 + lane over this warp's rows
+    part[tid] = sum;
+    __syncthreads();
+    if (tid < kBwdColsW && chunk * kBwdColsW + tid < cb) {
+        float t = part[tid];
+#pragma unroll
+        for (int q = 1; q < kW / 32; ++q) t += part[tid + q * kBwdColsW];
+        double* py = w + f + chunk * kBwdColsW + tid;
+        *py = __ldcg(py) - t;
+    }
+}
+
+// The FP64 form's wide steps take 64 columns (the diagonal 64 x 64 blocks of a tile's inverse
+// are the inverses of its blocks): a warp's FP64 instruction takes its pipe 64 cycles, so every
+// thread gets 16 products of x_b = X_bb w_b (four threads per row; backward from the
+// transposed copy of X, so that the loads coalesce in both directions) and 16 of L's part,
+// at most 0.7 us each.  One solve at P = 20,000 (134 steps and 12 first passes): 2.89 ms in
+// 32-column steps, 1.81 in 128-column ones (16 us a step of FP64 work that every CTA
+// repeats), 1.29 in 64-column ones, 0.80 with the launches chained; P = 300 150 -> 66 us.
+constexpr int kW64 = 64;
+constexpr int kLpr = kThreads / kW64;    // threads per row or column
+constexpr int kPer64 = kW64 / kLpr;      // products of each
+
+// This thread's part of the w x w block X at columns 64 b of supernode s (or of X^T, from the
+// transposed copy), and x = X v once v is in shared memory.
+__device__ __forceinline__ void wide_load64(const WideArgs& wa, int band, int s, int b, int k, int w, bool transposed,
+                                            double (&xv)[kPer64]) {
+    const int t = wa.xptr[s] + b / 2, o = (b & 1) * kW64, ld = min(kW, k - (b / 2) * kW);
+    const double* X = (transposed ? wa.xinvt64 : wa.xinv64) + band * wa.xband64 + wa.xoff64[t] + o + (int64_t)o * ld;
+    const int r = threadIdx.x % kW64, h = threadIdx.x / kW64;
+#pragma unroll
+    for (int q = 0; q < kPer64; ++q) {
+        const int c = kLpr * q + h;
+        xv[q] = (r < w && c < w && (transposed ? c >= r : c <= r)) ? X[r + c * ld] : 0.0;
+    }
+}
+__device__ __forceinline__ void wide_apply64(const double (&xv)[kPer64], int w, const double* v, double* x,
+                                             double (*part)[kW64]) {
+    const int r = threadIdx.x % kW64, h = threadIdx.x / kW64;
+    double y = 0.0;
+#pragma unroll
+    for (int q = 0; q < kPer64; ++q) {
+        if (kLpr * q >= w) break;
+        y = fma(xv[q], v[kLpr * q + h], y);
+    }
+    part[h][r] = y;
+    __syncthreads();
+    if (h == 0) x[r] = (part[0][r] + part[1][r]) + (part[2][r] + part[3][r]);
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(kThreads, 2) k_fwd_wide64(DevSym d, const int32_t* __restrict__ items, int b,
+                                                            const double* __restrict__ L, WideArgs wa,
+                                                            double* w, double* z, Strides bs) {
+    const int band = blockIdx.y;
+    L += band * bs.L;
+    w += band * bs.n;
+    z += band * bs.n;
+    __shared__ double wv[kW64], xb[kW64], part[kLpr][kW64];
+    const int s = items[2 * blockIdx.x], chunk = items[2 * blockIdx.x + 1];
+    const int f = d.sfirst[s], k = d.sfirst[s + 1] - f;
+    const int64_t m = d.srowptr[s + 1] - d.srowptr[s];
+    const double* P = L + d.lptr[s];
+    const int32_t* rows = d.srows + d.srowptr[s];
+    const int cb = b * kW64, wb = min(kW64, k - cb);
+    const int tid = threadIdx.x, h = tid / kW64;
+    // this thread's part of L, in flight while x_b is formed: a row of the chunk, every fourth column
+    const int64_t r = cb + wb + (int64_t)chunk * kW64 + tid % kW64;
+    double l[kPer64];
+#pragma unroll
+    for (int q = 0; q < kPer64; ++q) {
+        const int c = kLpr * q + h;
+        l[q] = (r < m && c < wb) ? P[r + (int64_t)(cb + c) * m] : 0.0;
+    }
+    double xv[kPer64];
+    wide_load64(wa, band, s, b, k, wb, false, xv);
+    const int32_t row = r < m ? rows[r] : 0;
+    chain_wait();
+    chain_next();
+    if (tid < kW64) wv[tid] = tid < wb ? __ldcg(w + f + cb + tid) : 0.0;
+    __syncthreads();
+    wide_apply64(xv, wb, wv, xb, part);
+    if (chunk == 0 && tid < wb) z[f + cb + tid] = xb[tid];
+    double acc = 0.0;
+#pragma unroll
+    for (int q = 0; q < kPer64; ++q) {
+        if (kLpr * q >= wb) break;
+        acc = fma(l[q], xb[kLpr * q + h], acc);
+    }
+    part[h][tid % kW64] = acc;
+    __syncthreads();
+    if (tid < kW64 && r < m) {
+        const double sum = (part[0][tid] + part[1][tid]) + (part[2][tid] + part[3][tid]);
+        if (r < k) w[f + r] = __ldcg(w + f + r) - sum;
+        else atomicAdd(w + row, -sum);
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, 2) k_bwd_wide64(DevSym d, const int32_t* __restrict__ items, int b,
+                                                            const double* __restrict__ L, WideArgs wa,
+                                                            double* w, double* x, Strides bs) {
+    const int band = blockIdx.y;
+    L += band * bs.L;
+    w += band * bs.n;
+    x += band * bs.n;
+    __shared__ double yv[kW64], xb[kW64], part[kLpr][kW64];
+    __shared__ double T[kW64][kW64 + 1];  // T[a][r] = L[cb + r][column a of the chunk]
+    const int s = items[2 * blockIdx.x], chunk = items[2 * blockIdx.x + 1];
+    const int f = d.sfirst[s], k = d.sfirst[s + 1] - f;
+    const int64_t m = d.srowptr[s + 1] - d.srowptr[s];
+    const double* P = L + d.lptr[s];
+    const int cb = b * kW64, wb = min(kW64, k - cb);
+    const int tid = threadIdx.x, q0 = tid % kW64, h = tid / kW64;
+    const int a0 = chunk * kW64, na = min(kW64, cb - a0);
+    double xv[kPer64];
+    wide_load64(wa, band, s, b, k, wb, true, xv);
+    if (na > 0) {  // coalesced down the rows, read back by columns
+        double l[kPer64];
+#pragma unroll
+        for (int q = 0; q < kPer64; ++q) {
+            const int a = kLpr * q + h;
+            l[q] = (q0 < wb && a < na) ? P[(cb + q0) + (int64_t)(a0 + a) * m] : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < kPer64; ++q) T[kLpr * q + h][q0] = l[q];
+    }
+    chain_wait();
+    chain_next();
+    if (tid < kW64) yv[tid] = tid < wb ? __ldcg(w + f + cb + tid) : 0.0;
+    __syncthreads();
+    wide_apply64(xv, wb, yv, xb, part);
+    if (chunk == 0 && tid < wb) x[f + cb + tid] = xb[tid];
+    if (na <= 0) return;
+    double acc = 0.0;
+#pragma unroll
+    for (int q = 0; q < kPer64; ++q) {
+        if (kLpr * q >= wb) break;
+        acc = fma(T[q0][kLpr * q + h], xb[kLpr * q + h], acc);
+    }
+    part[h][q0] = acc;
+    __syncthreads();
+    if (tid < na) {
+        double* py = w + f + a0 + tid;
+        *py = __ldcg(py) - ((part[0][tid] + part[1][tid]) + (part[2][tid] + part[3][tid]));
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -839,6 +1050,7 @@ cudaError_t solve_kernel_setup() {
         (const void*)k_bwd_init<double>, (const void*)k_bwd_step<float>,  (const void*)k_bwd_step<double>,
         (const void*)k_fwd_level<float>, (const void*)k_fwd_level<double>, (const void*)k_bwd_level<float>,
         (const void*)k_bwd_level<double>, (const void*)k_fwd_wide,       (const void*)k_bwd_wide,
+        (const void*)k_fwd_wide64,     (const void*)k_bwd_wide64,
         (const void*)k_solve_dag<float>, (const void*)k_solve_dag<double>, (const void*)k_sym_residual,
         (const void*)k_norms2,           (const void*)k_axpy,             (const void*)k_permute_in,
         (const void*)k_permute_out};
@@ -906,18 +1118,12 @@ void launch_permute_out(int32_t n, const int32_t* perm, const double* w, double*
     k_permute_out<<<dim3(std::min(1024, (n + 255) / 256), nb), 256, 0, st>>>(n, perm, w, x);
 }
 
-void build_solve_plan(const Symbolic& S, SolvePlan& P, int batch, const uint8_t* wide) {
+void build_solve_plan(const Symbolic& S, SolvePlan& P, int batch, const uint8_t* wide, bool fp64) {
     P = SolvePlan();
     for (int32_t l = 0; l < S.nlevels; ++l) {
         int32_t kmax = 0;
-        int64_t work = 0;
-        for (int32_t p = S.level_ptr[l]; p < S.level_ptr[l + 1]; ++p) {
-            const int32_t s = S.level_list[p];
-            const int64_t k = S.k_of(s), m = S.m_of(s);
-            kmax = std::max<int32_t>(kmax, (int32_t)k);
-            work = std::max(work, k * m - k * k / 2);
-        }
-        if (batch > 1 && work <= (int64_t)((kmax + kT - 1) / kT) * kFuseFmaPerStep) {  // one launch per sweep
+        for (int32_t p = S.level_ptr[l]; p < S.level_ptr[l + 1]; ++p) kmax = std::max(kmax, S.k_of(S.level_list[p]));
+        if (batch > 1 && kmax <= kFuseCols) {  // one launch per sweep
             Launch lf{10, 0, (int64_t)P.fwd_items.size() / 2, 0};
             Launch lb{11, 0, (int64_t)P.bwd_items.size() / 2, 0};
             for (int32_t p = S.level_ptr[l]; p < S.level_ptr[l + 1]; ++p) {
@@ -932,18 +1138,19 @@ void build_solve_plan(const Symbolic& S, SolvePlan& P, int batch, const uint8_t*
         }
         const int32_t nsteps = (kmax + kT - 1) / kT;
         std::vector<Launch> fw, bw;
-        // wide steps of 128 columns for the flagged supernodes (kinds 15 and 16)
-        for (int32_t b = 0; wide && b * kW < kmax; ++b) {
+        // wide steps of 128 (64 in FP64) columns for the flagged supernodes (kinds 15 and 16)
+        const int32_t ww = fp64 ? kW64 : kW, rpc = fp64 ? kW64 : kFwdRowsW, cpc = fp64 ? kW64 : kBwdColsW;
+        for (int32_t b = 0; wide && b * ww < kmax; ++b) {
             Launch lf{15, b, (int64_t)P.fwd_items.size() / 2, 0};
             Launch lb{16, b, (int64_t)P.bwd_items.size() / 2, 0};
             for (int32_t p = S.level_ptr[l]; p < S.level_ptr[l + 1]; ++p) {
                 const int32_t s = S.level_list[p], k = S.k_of(s), m = S.m_of(s);
-                if (!wide[s] || k <= b * kW) continue;
-                const int32_t wb = std::min(kW, k - b * kW);
-                const int64_t below = (int64_t)m - b * kW - wb;
-                const int32_t nch = std::max<int32_t>(1, (int32_t)((below + kFwdRowsW - 1) / kFwdRowsW));
+                if (!wide[s] || k <= b * ww) continue;
+                const int32_t wb = std::min(ww, k - b * ww);
+                const int64_t below = (int64_t)m - b * ww - wb;
+                const int32_t nch = std::max<int32_t>(1, (int32_t)((below + rpc - 1) / rpc));
                 for (int32_t c = 0; c < nch; ++c) { P.fwd_items.push_back(s); P.fwd_items.push_back(c); lf.count++; }
-                const int32_t ncb = std::max<int32_t>(1, (b * kW + kBwdColsW - 1) / kBwdColsW);
+                const int32_t ncb = std::max<int32_t>(1, (b * ww + cpc - 1) / cpc);
                 for (int32_t c = 0; c < ncb; ++c) { P.bwd_items.push_back(s); P.bwd_items.push_back(c); lb.count++; }
             }
             if (lf.count) fw.push_back(lf);
@@ -957,7 +1164,7 @@ void build_solve_plan(const Symbolic& S, SolvePlan& P, int batch, const uint8_t*
                 if (k <= b * kT || (wide && wide[s])) continue;
                 const int32_t wb = std::min(kT, k - b * kT);
                 const int64_t below = (int64_t)m - b * kT - wb;
-                const int32_t nch = std::max<int32_t>(1, (int32_t)((below + kFwdRows - 1) / kFwdRows));
+                const int32_t nch = std::max<int32_t>(1, (int32_t)((below + kStepRows - 1) / kStepRows));
                 for (int32_t c = 0; c < nch; ++c) { P.fwd_items.push_back(s); P.fwd_items.push_back(c); lf.count++; }
                 const int32_t ncb = std::max<int32_t>(1, (b * kT + kBwdCols - 1) / kBwdCols);
                 for (int32_t c = 0; c < ncb; ++c) { P.bwd_items.push_back(s); P.bwd_items.push_back(c); lb.count++; }
@@ -968,7 +1175,7 @@ void build_solve_plan(const Symbolic& S, SolvePlan& P, int batch, const uint8_t*
         Launch li{5, 0, (int64_t)P.bwd_items.size() / 2, 0};
         for (int32_t p = S.level_ptr[l]; p < S.level_ptr[l + 1]; ++p) {
             const int32_t s = S.level_list[p], k = S.k_of(s);
-            const int32_t nch = std::max<int32_t>(1, (k + kT - 1) / kT);
+            const int32_t nch = std::max<int32_t>(1, (k + kInitCols - 1) / kInitCols);
             for (int32_t c = 0; c < nch; ++c) { P.bwd_items.push_back(s); P.bwd_items.push_back(c); li.count++; }
         }
         P.fwd_launches.insert(P.fwd_launches.end(), fw.begin(), fw.end());
@@ -991,20 +1198,29 @@ void launch_solve_step_t(const DevSym& d, const Launch& l, const int32_t* fwd_it
     const dim3 g(l.count, nb);
     if constexpr (std::is_same<TL, float>::value) {
         if (l.kind == 15 && wa) {
-            k_fwd_wide<<<g, kThreads, 0, st>>>(d, fwd_items + 2 * l.off, l.step, L, *wa, w, z, bs);
+            launch_chained(k_fwd_wide, g, kThreads, st, d, fwd_items + 2 * l.off, l.step, L, *wa, w, z, bs);
             return;
         }
         if (l.kind == 16 && wa) {
-            k_bwd_wide<<<g, kThreads, 0, st>>>(d, bwd_items + 2 * l.off, l.step, L, *wa, w, x, bs);
+            launch_chained(k_bwd_wide, g, kThreads, st, d, bwd_items + 2 * l.off, l.step, L, *wa, w, x, bs);
+            return;
+        }
+    } else {
+        if (l.kind == 15 && wa) {
+            launch_chained(k_fwd_wide64, g, kThreads, st, d, fwd_items + 2 * l.off, l.step, L, *wa, w, z, bs);
+            return;
+        }
+        if (l.kind == 16 && wa) {
+            launch_chained(k_bwd_wide64, g, kThreads, st, d, bwd_items + 2 * l.off, l.step, L, *wa, w, x, bs);
             return;
         }
     }
     switch (l.kind) {
-        case 4: k_fwd_step<TL><<<g, kThreads, 0, st>>>(d, fwd_items + 2 * l.off, l.step, L, w, z, bs); break;
-        case 5: k_bwd_init<TL><<<g, kThreads, 0, st>>>(d, bwd_items + 2 * l.off, L, D, z, x, w, bs); break;
+        case 4: launch_chained(k_fwd_step<TL>, g, kThreads, st, d, fwd_items + 2 * l.off, l.step, L, w, z, bs); break;
+        case 5: launch_chained(k_bwd_init<TL>, g, kThreads, st, d, bwd_items + 2 * l.off, L, D, z, x, w, bs); break;
         case 10: k_fwd_level<TL><<<g, kThreads, 0, st>>>(d, fwd_items + 2 * l.off, L, w, z, bs); break;
         case 11: k_bwd_level<TL><<<g, kThreads, 0, st>>>(d, bwd_items + 2 * l.off, L, D, z, x, w, bs); break;
-        default: k_bwd_step<TL><<<g, kThreads, 0, st>>>(d, bwd_items + 2 * l.off, l.step, L, w, x, bs); break;
+        default: launch_chained(k_bwd_step<TL>, g, kThreads, st, d, bwd_items + 2 * l.off, l.step, L, w, x, bs); break;
     }
 }
 

@@ -81,8 +81,8 @@ struct Launch {
                      // 12 persistent per-level kernel: whole panels of small fronts, one CTA
                      // per front at a time; solves: 4 forward step, 5 backward first launch of
                      // a level, 6 backward step, 10 / 11 forward / backward sweep of a whole
-                     // level, 15 / 16 forward / backward step of 128 columns (mixed form,
-                     // inverted diagonal tiles); -1 a timing marker of the autotuner (no
+                     // level, 15 / 16 forward / backward step of 128 columns (inverted
+                     // diagonal tiles); -1 a timing marker of the autotuner (no
                      // launch; `step` = group)
     int step;        // block column b for kinds 0/1
     int64_t off;     // offset into the item array of the kind
@@ -171,9 +171,9 @@ struct SolvePlan {
 };
 
 // batch: bands per launch (the fused per-level sweeps are used for batches only);
-// wide: per supernode, 1 = steps of 128 columns with the inverted diagonal tiles of
-// the mixed form (launch kinds 15 and 16; such a plan is run with FP32 panels)
-void build_solve_plan(const Symbolic& S, SolvePlan& P, int batch, const uint8_t* wide = nullptr);
+// wide: per supernode, 1 = steps of 128 columns (64 with fp64) with the inverted diagonal tiles
+// (launch kinds 15 and 16)
+void build_solve_plan(const Symbolic& S, SolvePlan& P, int batch, const uint8_t* wide = nullptr, bool fp64 = false);
 void build_solve_dag(const Symbolic& S, SolvePlan& P);
 // both sweeps in one dependency-driven launch; counters: nb * cstride + 1 ints, zeroed before
 void launch_solve_dag(const DevSym& d, const DagTask* tasks, int ntasks, int* counters, int cstride, const double* L,
@@ -205,8 +205,8 @@ struct DevDiagPlan {
     double tc_flops = 0;  // TF32 MMA flops of the tensor-core variance kernel on this plan
     bool fx = false;      // FP64 form: on the tensor cores (diag_fx.cu), with the operand tiles of the
                           //   plan's supernodes
-    int32_t *fx_tiles = nullptr, *fx_dts = nullptr;
-    int64_t fx_ntiles = 0, fx_ndt = 0;
+    int32_t* fx_tiles = nullptr;
+    int64_t fx_ntiles = 0;
     std::vector<void*> allocs;
 };
 
@@ -228,12 +228,16 @@ void launch_factor_dag(const DevSym& d, const DagTask* tasks, int ntasks, int* c
 void launch_permute_in(int32_t n, const int32_t* perm, const double* b, double* w, int nb, cudaStream_t st);
 void launch_permute_out(int32_t n, const int32_t* perm, const double* w, double* x, int nb, cudaStream_t st);
 // L32: the mixed form's FP32 panels (read instead of L, the same values), or null
-// The inverted 128 x 128 diagonal tiles of the mixed form's tensor-core supernodes, for the
-// solve's wide steps (launch kinds 15 and 16).
+// The inverted diagonal tiles for the solve's wide steps (launch kinds 15 and 16): the
+// mixed form's tensor-core supernodes', or every supernode's of the FP64 form.
 struct WideArgs {
-    const float* xinv = nullptr;   // [bands][tiles][128 x 128], row-major
-    const int32_t* xptr = nullptr; // [ns] first tile of each supernode
-    int64_t xband = 0;             // floats per band
+    const float* xinv = nullptr;    // mixed: [bands][tiles][128 x 128], row-major
+    const int32_t* xptr = nullptr;  // [ns] first tile of each supernode
+    int64_t xband = 0;              // floats per band
+    const double* xinv64 = nullptr; // FP64: [bands][xband64], tile t w x w column-major from xoff64[t]
+    const double* xinvt64 = nullptr;// its transposes
+    const int64_t* xoff64 = nullptr;
+    int64_t xband64 = 0;
 };
 void launch_solve_step(const DevSym& d, const Launch& l, const int32_t* fwd_items, const int32_t* bwd_items,
                        const double* L, const double* D, double* w, double* z, double* x, int nb,
@@ -280,13 +284,24 @@ void launch_diag_inv_tc(const DevSym& d, const DevDiagPlan& dp, const DevDiagTc&
                         int nb, const Strides& bs, DevStatus* status, int wait_limit, cudaStream_t st);
 
 // ---- diag_fx.cu: the FP64 form's variances on the tensor cores (exact integer pieces)
+// Inverses of the FP64 form's unit-lower diagonal tiles (w x w, w <= 128, column-major, one
+// after another), for the solves and the variances.
+struct DevTileInv {
+    int64_t ncta = 0, nx = 0;        // CTAs of the launch; doubles per band
+    int32_t* dtiles = nullptr;       // [ncta][4] supernode, chunk, tile, first column
+    int32_t* xptr = nullptr;         // [ns] first tile of each supernode
+    int64_t* xoff = nullptr;         // [tiles]
+    double* xinv = nullptr;          // [bands][nx]
+    double* xinvt = nullptr;         // [bands][nx] their transposes
+};
+void launch_tile_inverses(const DevSym& d, const DevTileInv& x, const double* L, int nb, const Strides& bs,
+                          cudaStream_t st);
 struct DevDiagFx {
-    int64_t npieces = 0, ntiles = 0, ndt = 0;
+    int64_t npieces = 0, ntiles = 0;
     int64_t* pptr = nullptr;
-    int32_t *tptr = nullptr, *tiles = nullptr, *tdiag = nullptr, *dtiles = nullptr;
+    int32_t *tptr = nullptr, *tiles = nullptr, *tdiag = nullptr;
     unsigned char* pack = nullptr;  // [bands][npieces] packed 128 x 16 pieces, seven digit planes each
     int32_t* rexp = nullptr;        // [bands][ntiles][128] row exponents
-    double* xinv = nullptr;         // [bands][ndt][128 x 128] inverted diagonal tiles
     double* fr = nullptr;           // [bands][n] s^2 / d, s the power of two next to sqrt(d)
     std::vector<void*> allocs;
 };
@@ -294,14 +309,14 @@ cudaError_t diag_fx_setup();
 size_t diag_fx_pack_bytes(int64_t npieces);
 // prepares the operands from the factor, then the variances of plan dp (dp.B
 // 16, 32 or 64)
-void launch_diag_fx(const DevSym& d, const DevDiagPlan& dp, const DevDiagFx& p, const double* L, const double* D,
+void launch_diag_fx(const DevSym& d, const DevDiagPlan& dp, const DevDiagFx& p, const DevTileInv& x, const double* L, const double* D,
                     double* out, int nb, const Strides& bs, DevStatus* status, cudaStream_t st);
 
 // (N^-1)(I, I) for the pivots of a plan with zpiv/rowmap: the blocks' forward
 // solves (variances to var_scratch; on the tensor cores with fx, when the plan has fx
 // set), their vectors gathered into Zg (R rows x nrhs), then the Gram product into
 // out (ldo = leading dimension, positions from the plan's rhs_out).
-void launch_inverse_block(const DevSym& d, const DevDiagPlan& p, const DevDiagFx* fx, const double* L, const double* D,
+void launch_inverse_block(const DevSym& d, const DevDiagPlan& p, const DevDiagFx* fx, const DevTileInv& x, const double* L, const double* D,
                           double* var_scratch, double* Zg, int64_t R, double* out, int64_t ldo, DevStatus* status,
                           cudaStream_t st);
 
@@ -339,6 +354,32 @@ void launch_bg_sums(bool mle, int64_t nrows, const int64_t* rowptr, const int32_
                     const double* x, int32_t k0, const int64_t* bgpos, const int32_t* upat, const double* t,
                     const double* y, const double* w, int32_t npat, double* sums, double* acc, cudaStream_t st);
 void launch_bg_pattern(int32_t npat, const double* sums, double* U, cudaStream_t st);
+
+// Programmatic dependent launch of chained kernels (launch_chained below).  chain_wait
+// waits for the previous kernel's results; before it a kernel reads only data that no
+// kernel of the chain writes (indices, L, inverted tiles), so that its launch and those
+// reads overlap the previous kernel.  chain_next, after it, lets the next kernel start.
+// Every CTA of a chained kernel calls both, so each kernel's end implies all earlier
+// ones', and at most one kernel is started ahead.  Vectors written within the chain are
+// read through L2 (__ldcg): a read-only or L1 load could return what an earlier kernel's
+// CTA left in this SM's L1, or be moved above the wait.  Both calls are no-ops in a
+// kernel launched the ordinary way.
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, int threads, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
 
 // Sums over the 32 lanes of a warp of each of v[0..31]: lane j returns the sum of v[j].
 // Recursive halving: at distance h every lane keeps the half of its values whose index

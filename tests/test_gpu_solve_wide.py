@@ -1,0 +1,64 @@
+"""The FP64 solve in 64-column steps through the inverted diagonal tiles (launch kinds 15
+and 16), against the oracle, at the edges of a step, of a 128-column tile and of the 64
+rows or columns a CTA takes.  Bound: x of a well-conditioned matrix (random_spd with a
+unit shift) to 64 n 2^-53, n rounding errors of a few units each way; the SPI members to
+the 1e-10 of the parity tests."""
+import numpy as np
+import pytest
+
+import oracle
+from spigen import SCALE, BAND, generate, generate_bands, random_spd, scaled
+
+pytestmark = pytest.mark.gpu
+EPS = 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def P():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1305_5683_gb300 as P
+    P.build.build()
+    return P
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 63, 64, 65, 127, 128, 129, 191, 193, 256, 257, 330])
+def test_one_dense_front(P, n):
+    pb = random_spd(n, 1.0, n, dominance=float(n))
+    s = P.Solver.for_problem(pb, dag=1)
+    s.factor(pb.values)
+    x, ref = s.solve(pb.b), oracle.OracleFactor.from_problem(pb).solve(pb.b)
+    assert np.abs(x - ref).max() <= 64 * max(n, 16) * EPS * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("points", [300, 1501, 2600])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_spi_members_repeat_and_alias(P, points, precision):
+    """Several solves on one factor, a new factorization, and x aliasing b."""
+    pb = generate(scaled(SCALE, points, seed=points))
+    f = oracle.OracleFactor.from_problem(pb)
+    s = P.Solver.for_problem(pb, precision=precision, dag=1)
+    tol = 1e-10 if precision == 0 else 1e-8
+    rng = np.random.default_rng(points)
+    for scale in (1.0, 1.0, 3.0):
+        s.factor(pb.values * scale)
+        for _ in range(2):
+            b = rng.standard_normal(pb.n)
+            ref = f.solve(b) / scale
+            assert np.abs(s.solve(b) - ref).max() <= tol * np.abs(ref).max()
+            x = b.copy()
+            s.solve(x, x)
+            assert np.abs(x - ref).max() <= tol * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_bands_with_fused_and_stepped_levels(P, precision):
+    bands = generate_bands(scaled(BAND, 900, seed=4), 3)
+    s = P.Solver(bands.n, bands.colptr, bands.rowind, batch=3, precision=precision, dag=1)
+    s.factor_batch(bands.values)
+    x = s.solve_batch(bands.b).reshape(3, -1)
+    for k in range(3):
+        pb = bands.band(k)
+        ref = oracle.OracleFactor.from_problem(pb).solve(pb.b)
+        assert np.abs(x[k] - ref).max() <= (1e-10 if precision == 0 else 1e-8) * np.abs(ref).max()
