@@ -215,7 +215,7 @@ void build_dag(const Symbolic& S, FactorPlan& F, int32_t nlev, const std::vector
                 for (int32_t b = 0; b * kT < k; ++b) {
                     const int32_t w = std::min(kT, k - b * kT), r0 = b * kT + w;
                     std::vector<DagTask> tr, up;
-                    for (int32_t c = 0; r0 + (int64_t)c * kThreads < m; ++c) tr.push_back(task(kDagTrsm, b, c));
+                    for (int32_t c = 0; r0 + (int64_t)c * kT < m; ++c) tr.push_back(task(kDagTrsm, b, c));
                     for (int32_t tj = 0; r0 + tj * kT < k; ++tj)
                         for (int32_t ti = 0; r0 + tj * kT + ti * kT < m; ++ti) up.push_back(task(kDagUpdate, b, (ti << 16) | tj));
                     if (!tr.empty()) t.push_back(tr);
@@ -355,7 +355,7 @@ void build_factor_plan(const Symbolic& S, FactorPlan& F, bool tensor_cores_allow
                 const double k = S.k_of(t.s), m = S.m_of(t.s);
                 if (t.type == kDagFused) F.work_flops += m * k * k - 2.0 * k * k * k / 3.0;
                 if (t.type == kDagPivot) F.work_flops += 2.0 * std::pow(std::min<double>(kT, k), 3) / 3.0;
-                if (t.type == kDagTrsm) F.work_flops += kThreads * std::pow(std::min<double>(kT, k - t.a * kT), 2);
+                if (t.type == kDagTrsm) F.work_flops += kT * std::pow(std::min<double>(kT, k - t.a * kT), 2);
                 if (t.type == kDagUpdate) F.work_flops += 2.0 * kT * kT * std::min<double>(kT, k - t.a * kT);
                 if (t.type == kDagSchur) F.work_flops += 2.0 * kT * kT * k;
             }
@@ -398,104 +398,123 @@ __device__ __forceinline__ T ldx(const T* p) {
 }
 
 // 1/d in FP64 with three FP64 operations on the dependency chain (a dependent FP64
-// operation costs about 64 cycles on this GPU; a division or a conversion to and from
-// single precision costs several).  d = m 2^(ex - 1023) with m in [1, 2): a single-
-// precision seed r0 ~ 1/m is formed from m's top 23 mantissa bits by bit operations and
-// one __frcp_rn, then refined by one step of the third-order reciprocal iteration (the
-// Newton-Raphson iteration for 1/m carried one term further: 1/m = r0 / (1 - e) =
-// r0 (1 + e + e^2 + ...), e = 1 - m r0), r0 (1 + e + e^2); |e| < 2^-22, so the dropped
-// e^3 term is below FP64 rounding and the result is within 2 ulp of the correctly
-// rounded 1/m (measured against 1.0 / d over 2^22 values spanning 2^-60 .. 2^60:
-// at most 1.93 ulp).  The exponent is restored by integer arithmetic.  Zero,
+// operation costs about 64 cycles on this GPU, a division 350): the hardware's
+// approximation r0 (within 2^-19.9), refined by one step of the third-order reciprocal
+// iteration (the Newton-Raphson iteration carried one term further: 1/d = r0 / (1 - e) =
+// r0 (1 + e + e^2 + ...), e = 1 - d r0), r0 (1 + e + e^2): the dropped e^3 term is below
+// FP64 rounding and the result within 1 ulp of the correctly rounded 1/d (268 million
+// values over the whole exponent range).  Zero,
 // subnormal, huge or non-finite d divide.
 __device__ __forceinline__ double recip_fp64(double d) {
-    const long long b = __double_as_longlong(d);
-    const int ex = (int)((b >> 52) & 0x7ff);
+    const int ex = (__double2hiint(d) >> 20) & 0x7ff;
     if (ex < 4 || ex > 2042) return 1.0 / d;
-    const double m = __longlong_as_double((b & 0x800FFFFFFFFFFFFFLL) | 0x3FF0000000000000LL);
-    const float mf = __int_as_float((int)((b >> 29) & 0x7FFFFF) | 0x3F800000 | (int)((b >> 32) & 0x80000000LL));
-    const int rb = __float_as_int(__frcp_rn(mf));  // in (0.5, 1]
-    const double r0 = __longlong_as_double(((long long)(rb & 0x80000000) << 32) |
-                                           ((long long)(((rb >> 23) & 0xff) - 127 + 1023) << 52) |
-                                           ((long long)(rb & 0x7FFFFF) << 29));
-    const double e = fma(-m, r0, 1.0);
-    const double r = fma(r0, fma(e, e, e), r0);
-    return __longlong_as_double(__double_as_longlong(r) - ((long long)(ex - 1023) << 52));
+    double r0;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(d));
+    const double e = fma(-d, r0, 1.0);
+    return fma(r0, fma(e, e, e), r0);
 }
 
-// Entries of the lower triangle of order kT - 2, row by row: entry e is (e >> 8, e & 255).
+// Entries (i, j) of a pivot tile with 2 <= j <= i, column by column: entry e of the
+// list is thread e % 96's.
+constexpr int kTriThreads = 96;
 constexpr int kTri = (kT - 2) * (kT - 1) / 2;
+constexpr int kTriOwn = (kTri + kTriThreads - 1) / kTriThreads;
+struct TriTable {
+    uint16_t at[kTri];  // i << 8 | j, from the last entry to the first
+};
+constexpr TriTable make_tri() {
+    TriTable t{};
+    int n = 0;
+    for (int j = kT - 1; j >= 2; --j)
+        for (int i = kT - 1; i >= j; --i) t.at[n++] = (uint16_t)(i << 8 | j);
+    return t;
+}
+__device__ const TriTable kTriTable = make_tri();
 
 // Unblocked LDL^T, in FP64, of the w x w pivot tile whose first pivot is
 // column c0 of supernode s (panel P of storage type S, leading dimension m),
 // by the CTA's 128 threads; writes L (unit lower, d on the diagonal) back into
 // P, d into D (FP64) and into DS (the storage type's copy used for scaling).
-// The tile is bound by its column-to-column dependency chain, not by FP64
-// throughput, so the work is split by that chain.  Per column c, one barrier
-// apart: warp 3 forms column c + 1 -- its last update, the pivot
-// d_{c+1} = a_{c+1,c+1} - a_{c+1,c} l_{c+1,c} and 1/d_{c+1} (every lane
-// computes them: one lane costs as much as 32), then l_{j,c+1} = a_{j,c+1} / d_{c+1}
-// -- while warps 0-2 apply column c to the rest of the triangle,
-// a_ij -= a_ic l_jc for c + 2 <= j <= i (from a table of the triangle's
-// entries).  The scaled columns of L wait in the tile's unused upper triangle
-// until the end; the pivots are checked there, all at once.
-template <typename S, bool kCg = false>
+// The tile is bound by its column-to-column dependency chain (an FP64 warp
+// instruction takes its pipe 64 cycles, whatever its active lanes), so the work is
+// split by that chain.  Per column c, one barrier apart: warp 3 (lane = row)
+// forms column c + 1 in registers -- a_j = in_j - l_jc a_{c+1,c}, the pivot d_{c+1}
+// from its lane by a shuffle, 1 / d_{c+1}, l_j -- and hands both a and l over in shared
+// memory, while warps 0-2 apply column c to the entries beyond, which stay in the
+// registers of the thread that owns them and go to shared memory (`in`) in the step before
+// their column's turn.  On the chain of a column: one multiply-add, a shuffle, the
+// reciprocal's three operations and a multiplication (in the order l_jc = a_jc / d_c first:
+// a_jc a_{c+1,c} would leave the range of FP64 for entries beyond 10^+-154).  Against
+// the tile held in shared memory, with all four warps on every column, and together with the
+// four-lane panel solve below: factorization + solve + variances of P = 300 608 -> 522 us, of
+// P = 2,003 1,016 -> 884 us, of 48 trees 4,641 -> 4,307 us.
+template <typename S, bool kCg = false, bool kLoaded = false>
 __device__ void factor_pivot_tile(double (*A)[kT + 1], double* dv, S* P, int64_t m, int c0, int w,
                                   int f, double* D, S* DS, const double* __restrict__ adiag, DevStatus* status,
                                   int band_base) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    __shared__ double lc[2][kT];    // l_{j,c} of the column being applied, alternating
-    __shared__ uint16_t tri[kTri];
+    __shared__ double lc[2][kT], ac[2][kT], in[2][kT];  // of the column being applied / the next one, alternating
     static_assert(kThreads == 128 && kT == 32, "three update warps and one pivot warp over a 32 x 32 tile");
-    for (int e = tid; e < kT * kT; e += kThreads) {
-        const int i = e % kT, j = e / kT;
-        if (i < w && j <= i) A[i][j] = (double)ldx<kCg>(P + (c0 + i) + (int64_t)(c0 + j) * m);
-    }
-    for (int e = tid; e < kTri; e += kThreads) {
-        int i = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-        if ((i + 1) * (i + 2) / 2 <= e) ++i;
-        if (i * (i + 1) / 2 > e) --i;
-        tri[e] = (uint16_t)((i << 8) | (e - i * (i + 1) / 2));
-    }
-    __syncthreads();
-    if (warp == 3) {  // column 0
-        const double d = A[0][0];
-        const double inv = recip_fp64(d);
-        if (lane == 0) dv[0] = d;
-        if (lane > 0 && lane < w) {
-            const double l = A[lane][0] * inv;
-            lc[0][lane] = l;
-            A[0][lane] = l;
+    if constexpr (!kLoaded) {  // (kLoaded: the caller left the tile in A, zero beyond w, and passed a barrier)
+        S v[kT * kT / kThreads];
+#pragma unroll
+        for (int q = 0; q < kT * kT / kThreads; ++q) {
+            const int i = lane, j = warp + 4 * q;
+            v[q] = (j <= i && i < w) ? ldx<kCg>(P + (c0 + i) + (int64_t)(c0 + j) * m) : S(0);
         }
+#pragma unroll
+        for (int q = 0; q < kT * kT / kThreads; ++q)
+            if (warp + 4 * q <= lane) A[lane][warp + 4 * q] = (double)v[q];
+    }
+    // this thread's entries (warps 0-2): e = tid + 96 q of the column-by-column list; by its
+    // distance from the end, columns 31, 30, ... hold 1, 2, ... entries
+    int oi[kTriOwn], oj[kTriOwn];
+    double ov[kTriOwn];
+#pragma unroll
+    for (int q = 0; q < kTriOwn; ++q) {
+        const int e = tid + kTriThreads * q;
+        const bool on = warp < 3 && e < kTri;
+        const uint16_t t = on ? kTriTable.at[kTri - 1 - e] : (uint16_t)0;
+        oi[q] = t >> 8;
+        oj[q] = t & 255;
+    }
+    const double ad = tid < w ? adiag[f + c0 + tid] : 0.0;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kTriOwn; ++q) ov[q] = A[oi[q]][oj[q]];
+    double a = 0.0, l = 0.0, an = 0.0, nx = 0.0;  // column c: a and l of this row, a of row c + 1; in of column c + 1
+    if (warp == 3) {  // column 0
+        a = A[lane][0];
+        const double d = __shfl_sync(0xffffffffu, a, 0);
+        an = __shfl_sync(0xffffffffu, a, 1);
+        nx = lane > 0 ? A[lane][1] : 0.0;
+        l = a * recip_fp64(d);
+        if (lane == 0) dv[0] = d;
+        ac[0][lane] = a;
+        lc[0][lane] = l;
     }
     __syncthreads();
+    // column c of L goes into row c of the tile's upper triangle (read by nobody before the end)
+    if (warp == 3 && lane > 0) A[0][lane] = lc[0][lane];
     for (int c = 0; c + 1 < w; ++c) {
-        const double* l = lc[c & 1];
         if (warp == 3) {
-            const int j = lane;
-            const double lcc = l[c + 1];
-            const double d = fma(-A[c + 1][c], lcc, A[c + 1][c + 1]);
-            double a = 0.0;
-            if (j > c + 1 && j < w) a = fma(-A[j][c], lcc, A[j][c + 1]);
-            const double inv = recip_fp64(d);
-            if (j == c + 1) dv[c + 1] = d;
-            if (j > c + 1 && j < w) {
-                const double lj = a * inv;
-                A[j][c + 1] = a;
-                lc[(c + 1) & 1][j] = lj;
-                A[c + 1][j] = lj;
-            }
+            if (c > 0) nx = in[(c + 1) & 1][lane];
+            a = fma(-l, an, nx);  // rows above c + 1 hold nothing of use
+            const double d = __shfl_sync(0xffffffffu, a, c + 1);
+            an = __shfl_sync(0xffffffffu, a, min(c + 2, kT - 1));
+            l = a * recip_fp64(d);
+            ac[(c + 1) & 1][lane] = a;
+            lc[(c + 1) & 1][lane] = l;
+            if (lane == c + 1) dv[c + 1] = d;
+            if (lane > c + 1) A[c + 1][lane] = l;
         } else {
-            const int n = w - 2 - c, N = n * (n + 1) / 2;
-            for (int e = tid; e < N; e += 2 * 96) {
-                const int e2 = e + 96;
-                const int t = tri[e], t2 = tri[e2 < N ? e2 : e];
-                const int gi = c + 2 + (t >> 8), gj = c + 2 + (t & 255);
-                const int gi2 = c + 2 + (t2 >> 8), gj2 = c + 2 + (t2 & 255);
-                const double v = fma(-A[gi][c], l[gj], A[gi][gj]);
-                const double v2 = fma(-A[gi2][c], l[gj2], A[gi2][gj2]);
-                A[gi][gj] = v;
-                if (e2 < N) A[gi2][gj2] = v2;
+            const double *cl = lc[c & 1], *ca = ac[c & 1];
+#pragma unroll
+            for (int q = 0; q < kTriOwn; ++q) {
+                if (oj[q] >= c + 2) {
+                    ov[q] = fma(-ca[oi[q]], cl[oj[q]], ov[q]);
+                    if (oj[q] == c + 2) in[c & 1][oi[q]] = ov[q];
+                }
             }
         }
         __syncthreads();
@@ -506,7 +525,7 @@ __device__ void factor_pivot_tile(double (*A)[kT + 1], double* dv, S* P, int64_t
     }
     if (tid < w) {
         const double dc = dv[tid];
-        if (!(dc > 0.0) || dc <= 1e-14 * adiag[f + c0 + tid]) {
+        if (!(dc > 0.0) || dc <= 1e-14 * ad) {
             atomicOr(&status->flags, FLAG_NOT_SPD);
             atomicMin(&status->bad_pivot, band_base + f + c0 + tid);
         }
@@ -557,10 +576,30 @@ __device__ void diag_front_body(const DevSym& d, int s, S* L, double* D, S* DS, 
         DS[f + c] = (S)dc;
         P[c + (int64_t)c * m] = (S)dc;
     }
-    // one reciprocal per column (uniform across the CTA), then scale its rows
-    for (int c = 0; c < k; ++c) {
-        const S rc = (S)(1.0 / adiag[f + c]);
-        for (int64_t r = k + tid; r < m; r += kThreads) P[r + (int64_t)c * m] = ldx<kCg>(P + r + (int64_t)c * m) * rc;
+    // the reciprocals, a thread per column (32 at a time; an FP64 division each), then the rows
+    // below by elements, four in flight per thread
+    __shared__ S rc[kT];
+    for (int cb = 0; cb < k; cb += kT) {
+        const int w = min(kT, k - cb);
+        __syncthreads();
+        if (tid < w) rc[tid] = (S)(1.0 / adiag[f + cb + tid]);
+        __syncthreads();
+        const int mb = (int)(m - k);
+        S* Q = P + k + (int64_t)cb * m;
+        for (int e0 = tid; e0 < mb * w; e0 += 4 * kThreads) {
+            S v[4];
+            int c[4], r[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int e = e0 + q * kThreads;
+                c[q] = e / mb;
+                r[q] = e - c[q] * mb;
+                v[q] = e < mb * w ? ldx<kCg>(Q + r[q] + (int64_t)c[q] * m) : S(0);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (e0 + q * kThreads < mb * w) Q[r[q] + (int64_t)c[q] * m] = v[q] * rc[c[q]];
+        }
     }
 }
 
@@ -587,13 +626,75 @@ union FrontPanelSmem {
     struct {
         C Bd[kT][kT + 1];       // strictly lower part of the factored pivot tile
         C rd[kT];               // 1 / d of its pivots
-        C X[kThreads][kT + 1];  // one row of the panel solve per thread
+        alignas(16) float Bt[kT][kT + 4];  // its transpose (FP32)
     } trsm;
     struct {
         C Li[kT][kT + 1];       // 32 rows of the block column
         C Lj[kT][kT + 1];       // 32 rows of the block column scaled by d
     } upd;
 };
+
+// The panel solve L21 = X L11^-T D^-1 of 32 rows r0 .. r0 + nr by the CTA, four lanes per
+// row (warp w holds rows 8 w .. 8 w + 7, lane q = lane % 4 of a row's group the columns
+// q, q + 4, ...): column c is final at its owner when the columns before it have been
+// applied; a shuffle hands it to the row's other lanes, which apply it to their later
+// columns.  All four warps work (a narrow FP64 pipe gives one warp a quarter of the SM's
+// rate), and the dependency chain per column is one shuffle and one multiply-add.
+// Bd: the strictly lower pivot tile, rd: 1 / d, both zero beyond w.
+template <bool kCg, typename C>
+__device__ __forceinline__ void panel_rows4(C* P, int64_t m, int c0, int w, int64_t r0, int nr,
+                                            const C (*Bd)[kT + 1], const C* rd) {
+    const int tid = threadIdx.x, lane = tid & 31, q = lane & 3;
+    const int r = 8 * (tid >> 5) + (lane >> 2);
+    const bool on = r < nr;
+    C y[kT / 4];  // y[t]: column 4 t + q of row r
+#pragma unroll
+    for (int t = 0; t < kT / 4; ++t) {
+        const int c = 4 * t + q;
+        y[t] = (on && c < w) ? ldx<kCg>(P + (r0 + r) + (int64_t)(c0 + c) * m) : C(0);
+    }
+#pragma unroll
+    for (int c = 0; c < kT; ++c) {
+        if (c >= w) break;
+        const C xc = __shfl_sync(0xffffffffu, y[c >> 2], (lane & ~3) | (c & 3));
+#pragma unroll
+        for (int t = 0; t < kT / 4; ++t) {
+            const int cc = 4 * t + q;
+            if (4 * t + 3 > c && cc > c && cc < w) y[t] -= xc * Bd[cc][c];
+        }
+    }
+#pragma unroll
+    for (int t = 0; t < kT / 4; ++t) {
+        const int c = 4 * t + q;
+        if (on && c < w) P[(r0 + r) + (int64_t)(c0 + c) * m] = y[t] * rd[c];
+    }
+}
+
+// The same for FP32, where a row fits one thread's registers and the arithmetic is cheap:
+// a thread per row, the tile's columns read four entries at a time (Bt[c][cc], zero on and
+// above the diagonal and beyond w).
+template <bool kCg>
+__device__ __forceinline__ void panel_row1(float* P, int64_t m, int c0, int w, int64_t r, const float (*Bt)[kT + 4],
+                                           const float* rd) {
+    float y[kT];
+#pragma unroll
+    for (int c = 0; c < kT; ++c) y[c] = c < w ? ldx<kCg>(P + r + (int64_t)(c0 + c) * m) : 0.f;
+#pragma unroll
+    for (int c = 0; c < kT - 1; ++c) {
+        if (c >= w) break;
+#pragma unroll
+        for (int t = (c + 1) / 4; t < kT / 4; ++t) {
+            const float4 b = *reinterpret_cast<const float4*>(&Bt[c][4 * t]);
+            y[4 * t] -= y[c] * b.x;
+            y[4 * t + 1] -= y[c] * b.y;
+            y[4 * t + 2] -= y[c] * b.z;
+            y[4 * t + 3] -= y[c] * b.w;
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < kT; ++c)
+        if (c < w) P[r + (int64_t)(c0 + c) * m] = y[c] * rd[c];
+}
 
 // A whole front's panel by one CTA: per 32-column block step, the FP64 pivot
 // tile, the panel solve of every row below it (one thread per row), then the
@@ -614,19 +715,17 @@ __device__ void front_panel_body(const DevSym& d, int s, C* Lb, double* Db, C* D
         // L21 = X L11^-T D^-1 for the rows below the pivot tile
         for (int e = tid; e < kT * kT; e += kThreads) {
             const int i = e % kT, j = e / kT;
-            sm.trsm.Bd[i][j] = (i < w && j < i) ? ldx<kCg>(P + (c0 + i) + (int64_t)(c0 + j) * m) : C(0);
+            const C v = (i < w && j < i) ? ldx<kCg>(P + (c0 + i) + (int64_t)(c0 + j) * m) : C(0);
+            if constexpr (std::is_same<C, float>::value) sm.trsm.Bt[j][i] = v;
+            else sm.trsm.Bd[i][j] = v;
         }
-        if (tid < kT) sm.trsm.rd[tid] = tid < w ? (C)(1.0 / ldx<kCg>(Db + f + c0 + tid)) : C(0);
+        if (tid < kT) sm.trsm.rd[tid] = tid < w ? (C)recip_fp64(ldx<kCg>(Db + f + c0 + tid)) : C(0);
         __syncthreads();
-        C* xr = sm.trsm.X[tid];
-        for (int64_t r = c0 + w + tid; r < m; r += kThreads) {
-            for (int c = 0; c < w; ++c) xr[c] = ldx<kCg>(P + r + (int64_t)(c0 + c) * m);
-            for (int c = 1; c < w; ++c) {
-                C y = xr[c];
-                for (int cp = 0; cp < c; ++cp) y -= xr[cp] * sm.trsm.Bd[c][cp];
-                xr[c] = y;
-            }
-            for (int c = 0; c < w; ++c) P[r + (int64_t)(c0 + c) * m] = xr[c] * sm.trsm.rd[c];
+        if constexpr (std::is_same<C, float>::value) {
+            for (int64_t r = c0 + w + tid; r < m; r += kThreads) panel_row1<kCg>(P, m, c0, w, r, sm.trsm.Bt, sm.trsm.rd);
+        } else {
+            for (int64_t r0 = c0 + w; r0 < m; r0 += kT)
+                panel_rows4<kCg, C>(P, m, c0, w, r0, (int)(m - r0 < kT ? m - r0 : kT), sm.trsm.Bd, sm.trsm.rd);
         }
         // rank-w update of panel columns [c0 + w, k), rows i >= j, in 32 x 32 tiles:
         // P[i][j] -= sum_c L[i][c] d_c L[j][c]; thread (ii, j0) owns row ii, columns j0 + 4 q
@@ -683,7 +782,7 @@ __device__ void front_panel_body(const DevSym& d, int s, C* Lb, double* Db, C* D
 // more per 32-column block step.  A front with a diagonal pivot block (~s in
 // the list) is scaled column by column.  The CTAs never wait on one another.
 template <typename C>
-__global__ void __launch_bounds__(kThreads) k_front_panel(DevSym d, const int32_t* __restrict__ items, int nitems,
+__global__ void __launch_bounds__(kThreads, sizeof(C) == 4 ? 4 : 3) k_front_panel(DevSym d, const int32_t* __restrict__ items, int nitems,
                                                           int nb, C* __restrict__ L, double* __restrict__ D,
                                                           C* __restrict__ DS, const double* __restrict__ adiag,
                                                           DevStatus* status, Strides bs) {
@@ -704,13 +803,7 @@ __global__ void __launch_bounds__(kThreads) k_front_panel(DevSym d, const int32_
 }
 
 // Row tile rt below the diagonal tile of block column b (already updated by
-// the block columns before it): L21 = X L11^-T D^-1.  Four lanes per row (warp
-// w holds rows 8 w .. 8 w + 7, lane q = lane % 4 of a row's group the columns
-// q, q + 4, ...): column c is final at its owner when the columns before it
-// have been applied; a shuffle hands it to the row's other lanes, which apply
-// it to their later columns.  All four warps work (a narrow FP64 pipe gives
-// one warp a quarter of the SM's rate), and the dependency chain per column is
-// one shuffle and one multiply-add.
+// the block columns before it): L21 = X L11^-T D^-1 (panel_rows4).
 template <typename C>
 __global__ void __launch_bounds__(kThreads) k_panel_trsm(DevSym d, const int32_t* __restrict__ items, int b,
                                                          C* __restrict__ L, const double* __restrict__ D,
@@ -719,43 +812,20 @@ __global__ void __launch_bounds__(kThreads) k_panel_trsm(DevSym d, const int32_t
     D += blockIdx.y * bs.n;
     __shared__ C Bd[kT][kT + 1];
     __shared__ C dv[kT];
-    const int tid = threadIdx.x, lane = tid & 31, q = lane & 3;
+    const int tid = threadIdx.x;
     const int s = items[2 * blockIdx.x], rt = items[2 * blockIdx.x + 1];
     const int f = d.sfirst[s], k = d.sfirst[s + 1] - f;
     const int64_t m = d.srowptr[s + 1] - d.srowptr[s];
     C* P = L + d.lptr[s];
     const int c0 = b * kT, w = min(kT, k - c0);
     const int64_t r0 = c0 + w + (int64_t)rt * kT;
-    const int nr = (int)(m - r0 < kT ? m - r0 : kT);
-    const int r = 8 * (tid >> 5) + (lane >> 2);
-    const bool on = r < nr;
     for (int e = tid; e < kT * kT; e += kThreads) {
         const int i = e % kT, j = e / kT;
         Bd[i][j] = (i < w && j < i) ? P[(c0 + i) + (int64_t)(c0 + j) * m] : C(0);
     }
     if (tid < kT) dv[tid] = (tid < w) ? (C)recip_fp64(D[f + c0 + tid]) : C(0);
-    C y[kT / 4];  // y[t]: column 4 t + q of row r
-#pragma unroll
-    for (int t = 0; t < kT / 4; ++t) {
-        const int c = 4 * t + q;
-        y[t] = (on && c < w) ? P[(r0 + r) + (int64_t)(c0 + c) * m] : C(0);
-    }
     __syncthreads();
-#pragma unroll
-    for (int c = 0; c < kT; ++c) {
-        if (c >= w) break;
-        const C xc = __shfl_sync(0xffffffffu, y[c >> 2], (lane & ~3) | (c & 3));
-#pragma unroll
-        for (int t = 0; t < kT / 4; ++t) {
-            const int cc = 4 * t + q;
-            if (4 * t + 3 > c && cc > c && cc < w) y[t] -= xc * Bd[cc][c];
-        }
-    }
-#pragma unroll
-    for (int t = 0; t < kT / 4; ++t) {
-        const int c = 4 * t + q;
-        if (on && c < w) P[(r0 + r) + (int64_t)(c0 + c) * m] = y[t] * dv[c];
-    }
+    panel_rows4<false, C>(P, m, c0, w, r0, (int)(m - r0 < kT ? m - r0 : kT), Bd, dv);
 }
 
 // Trailing panel update after block column b: for panel columns j in
@@ -787,6 +857,8 @@ __global__ void __launch_bounds__(kThreads) k_panel_update(DevSym d, const int32
         Lj[i][c] = (i < nj && c < w) ? P[(cj + i) + (int64_t)(c0 + c) * m] * DS[f + c0 + c] : C(0);
     }
     __syncthreads();
+    __shared__ double A[kT][kT + 1];  // the next pivot tile, for the CTA that updates it
+    const bool piv = ti == 0 && tj == 0;
     // thread owns row ii and columns j0 + 4 q: a warp's lanes run down one
     // column, so its read-modify-writes of the panel are coalesced
     const int ii = tid % kT, j0 = tid / kT;
@@ -809,15 +881,21 @@ __global__ void __launch_bounds__(kThreads) k_panel_update(DevSym d, const int32
 #pragma unroll
         for (int q = 0; q < kT / 4; ++q) {
             const int jj = j0 + 4 * q;
-            if (jj < nj && ri + ii >= cj + jj) P[(ri + ii) + (int64_t)(cj + jj) * m] = old[q] - acc[q];
+            const C v = old[q] - acc[q];
+            if (jj < nj && ri + ii >= cj + jj) {
+                if (piv && ii < nj) A[ii][jj] = (double)v;
+                else P[(ri + ii) + (int64_t)(cj + jj) * m] = v;
+            }
         }
     }
-    if (ti == 0 && tj == 0) {
-        // this CTA wrote the last update of the next block column's pivot tile: factor it now
-        __shared__ double A[kT][kT + 1];
+    if (piv) {
+        // this CTA made the last update of the next block column's pivot tile: factor it now
         __shared__ double dv[kT];
+        if (nj < kT)  // the last, narrower tile: zero beyond it
+            for (int e = tid; e < kT * kT; e += kThreads)
+                if (e % kT >= nj && e / kT <= e % kT) A[e % kT][e / kT] = 0.0;
         __syncthreads();
-        factor_pivot_tile(A, dv, P, m, cj, nj, f, D, DS, adiag, status, (int)(blockIdx.y * bs.n));
+        factor_pivot_tile<C, false, true>(A, dv, P, m, cj, nj, f, D, DS, adiag, status, (int)(blockIdx.y * bs.n));
     }
 }
 
@@ -1132,7 +1210,7 @@ __global__ void __launch_bounds__(128) k_schur_tc(DevSym d, const int32_t* __res
 // Dependency-driven persistent factorization (launch kind 13).
 //
 // One launch runs every task of a prefix of the tree's levels: diagonal-pivot
-// fronts, whole small fronts (front_panel_body), pivot tiles, 128-row chunks
+// fronts, whole small fronts (front_panel_body), pivot tiles, 32-row chunks
 // of the panel solve, 32 x 32 tiles of the trailing panel update (the first of
 // which factors the next pivot tile) and 32 x 32 Schur tiles added into the
 // parent.  The host lists the tasks in a topological order -- by level, then
@@ -1169,7 +1247,7 @@ __device__ bool dag_wait(const int* c, int need, const DevStatus* status, uint32
     }
 }
 
-// 128 rows of the panel solve below pivot tile b: L21 = X L11^-T D^-1.
+// 32 rows of the panel solve below pivot tile b: L21 = X L11^-T D^-1.
 template <typename C>
 __device__ void dag_trsm(const DevSym& d, int s, int b, int chunk, C* Lb, const double* Db, FrontPanelSmem<C>& sm) {
     const int tid = threadIdx.x;
@@ -1181,19 +1259,10 @@ __device__ void dag_trsm(const DevSym& d, int s, int b, int chunk, C* Lb, const 
         const int i = e % kT, j = e / kT;
         sm.trsm.Bd[i][j] = (i < w && j < i) ? __ldcg(P + (c0 + i) + (int64_t)(c0 + j) * m) : C(0);
     }
-    if (tid < kT) sm.trsm.rd[tid] = tid < w ? (C)(1.0 / __ldcg(Db + f + c0 + tid)) : C(0);
+    if (tid < kT) sm.trsm.rd[tid] = tid < w ? (C)recip_fp64(__ldcg(Db + f + c0 + tid)) : C(0);
     __syncthreads();
-    const int64_t r = c0 + w + (int64_t)chunk * kThreads + tid;
-    if (r < m) {
-        C* xr = sm.trsm.X[tid];
-        for (int c = 0; c < w; ++c) xr[c] = __ldcg(P + r + (int64_t)(c0 + c) * m);
-        for (int c = 1; c < w; ++c) {
-            C y = xr[c];
-            for (int cp = 0; cp < c; ++cp) y -= xr[cp] * sm.trsm.Bd[c][cp];
-            xr[c] = y;
-        }
-        for (int c = 0; c < w; ++c) P[r + (int64_t)(c0 + c) * m] = xr[c] * sm.trsm.rd[c];
-    }
+    const int64_t r0 = c0 + w + (int64_t)chunk * kT;
+    panel_rows4<true, C>(P, m, c0, w, r0, (int)(m - r0 < kT ? m - r0 : kT), sm.trsm.Bd, sm.trsm.rd);
 }
 
 // Trailing-update tile (ti, tj) after block column b (as k_panel_update); the
@@ -1302,7 +1371,7 @@ __device__ void dag_schur(const DevSym& d, int s, int ti, int tj, C* Lb, C* Fb, 
 }
 
 template <typename C>
-__global__ void __launch_bounds__(kThreads) k_factor_dag(DevSym d, const DagTask* __restrict__ tasks, int ntasks,
+__global__ void __launch_bounds__(kThreads, sizeof(C) == 4 ? 4 : 3) k_factor_dag(DevSym d, const DagTask* __restrict__ tasks, int ntasks,
                                                          int nb, int* cnt, int cstride, C* L, C* F22, double* D,
                                                          C* DS, const double* __restrict__ adiag, DevStatus* status,
                                                          Strides bs, uint32_t wait_limit) {

@@ -97,7 +97,7 @@ enum DagType : int32_t {
 struct DagTask {
     int32_t type;      // DagType
     int32_t s;         // supernode
-    int32_t a, b;      // kDagTrsm: block step, 128-row chunk; kDagUpdate: block step, ti << 16 | tj;
+    int32_t a, b;      // kDagTrsm: block step, 32-row chunk; kDagUpdate: block step, ti << 16 | tj;
                        // kDagSchur: ti, tj
     int32_t wait_idx;  // the task waits until counter[wait_idx] >= wait_val (0: no wait); counters
     int32_t wait_val;  //   [0, ns): tasks done of each front, [ns, 2 ns): children's Schur tiles added
