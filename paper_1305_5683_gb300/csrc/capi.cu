@@ -119,7 +119,7 @@ struct spi_ctx {
         bool ready = false;
         int64_t nrows = 0, nnzh = 0;
         int32_t ngroups = 0;
-        size_t smem = 0;
+        size_t smem = 0, smem_full = 0;
         std::vector<int64_t> grp_row;
         std::vector<int32_t> row_grp;
         std::vector<int64_t> hcp;  // H's pattern by columns: rows of each column
@@ -2072,7 +2072,8 @@ int spi_normal_setup(spi_ctx* c, int64_t nrows, const int64_t* rowptr, const int
         max_cols = std::max<int32_t>(max_cols, (int32_t)(gcolptr[(size_t)g + 1] - gcolptr[(size_t)g]));
     N.smem = normal_smem_bytes(max_dense, max_rows, max_cols);
     if (N.smem > 200 * 1024) return SPI_ERR_ARG;  // a row with too many entries for one CTA's list
-    CK(normal_kernel_setup(N.smem));
+    N.smem_full = normal_full_smem_bytes(max_dense, max_rows);
+    CK(normal_kernel_setup(N.smem, N.smem_full));
     N.ready = true;
     return SPI_OK;
 }
@@ -2122,7 +2123,7 @@ int spi_normal_assemble(spi_ctx* c, const double* hvals, const double* w, const 
     CK(cudaMemsetAsync(nv, 0, (size_t)c->S.nnz_a * sizeof(double), st));
     CK(cudaMemsetAsync(bv, 0, (size_t)c->S.n * sizeof(double), st));
     CK(cudaMemsetAsync(N.d_flag, 0, sizeof(int), st));
-    launch_normal(N.args, N.d_groups, N.ngroups, hv, wd, yd, nullptr, nullptr, false, nv, bv, N.d_flag, N.smem, st);
+    launch_normal(N.args, N.d_groups, N.ngroups, hv, wd, yd, nullptr, nv, bv, N.d_flag, N.smem_full, st);
     return normal_finish(c, nvals, b, on_device, st);
 }
 
@@ -2161,9 +2162,9 @@ int spi_normal_update(spi_ctx* c, int64_t ncols, const int32_t* cols, const doub
     if (!sel.empty()) {
         CK(cudaMemcpyAsync(N.d_mark, mark.data(), (size_t)n, cudaMemcpyHostToDevice, st));
         CK(cudaMemcpyAsync(N.d_sel, sel.data(), sel.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-        launch_normal(N.args, N.d_sel, (int32_t)sel.size(), hv, wd, yd, nullptr, N.d_mark, true, nv, bv, N.d_flag,
+        launch_normal_update(N.args, N.d_sel, (int32_t)sel.size(), hv, wd, yd, N.d_mark, true, nv, bv, N.d_flag,
                       N.smem, st);
-        launch_normal(N.args, N.d_sel, (int32_t)sel.size(), hv, wd, yd, nullptr, N.d_mark, false, nv, bv, N.d_flag,
+        launch_normal_update(N.args, N.d_sel, (int32_t)sel.size(), hv, wd, yd, N.d_mark, false, nv, bv, N.d_flag,
                       N.smem, st);
     }
     return normal_finish(c, nvals, b, on_device, st);
@@ -2207,7 +2208,7 @@ int mle_hessian(spi_ctx* c, const MleWork& W, const double* hv, const double* yd
     CK(cudaMemsetAsync(N.d_nv, 0, (size_t)c->S.nnz_a * sizeof(double), st));
     CK(cudaMemsetAsync(W.gx, 0, (size_t)c->S.n * sizeof(double), st));
     CK(cudaMemsetAsync(N.d_flag, 0, sizeof(int), st));
-    launch_normal(N.args, N.d_groups, N.ngroups, hv, W.w, yd, W.v, nullptr, false, N.d_nv, W.gx, N.d_flag, N.smem, st);
+    launch_normal(N.args, N.d_groups, N.ngroups, hv, W.w, yd, W.v, N.d_nv, W.gx, N.d_flag, N.smem_full, st);
     int flag = 0;
     CK(cudaMemcpyAsync(&flag, N.d_flag, sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -2381,12 +2382,12 @@ int spi_background_fit(spi_ctx* c, int64_t k0, const int32_t* upat, const double
         if (full) {
             CK(cudaMemsetAsync(N.d_nv, 0, nvb, st));
             CK(cudaMemsetAsync(N.d_b, 0, nb8, st));
-            launch_normal(N.args, N.d_groups, N.ngroups, hv, wd, yd, nullptr, nullptr, false, N.d_nv, N.d_b,
-                          N.d_flag, N.smem, st);
+            launch_normal(N.args, N.d_groups, N.ngroups, hv, wd, yd, nullptr, N.d_nv, N.d_b,
+                          N.d_flag, N.smem_full, st);
         } else if (!sel.empty()) {
-            launch_normal(N.args, N.d_sel, (int32_t)sel.size(), hv, wd, yd, nullptr, N.d_mark, true, N.d_nv, N.d_b,
+            launch_normal_update(N.args, N.d_sel, (int32_t)sel.size(), hv, wd, yd, N.d_mark, true, N.d_nv, N.d_b,
                           N.d_flag, N.smem, st);
-            launch_normal(N.args, N.d_sel, (int32_t)sel.size(), hv, wd, yd, nullptr, N.d_mark, false, N.d_nv,
+            launch_normal_update(N.args, N.d_sel, (int32_t)sel.size(), hv, wd, yd, N.d_mark, false, N.d_nv,
                           N.d_b, N.d_flag, N.smem, st);
         }
         int fl = 0;

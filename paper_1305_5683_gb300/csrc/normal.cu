@@ -7,11 +7,11 @@
 // Rows are grouped on the host into runs of consecutive rows whose column
 // sets nearly coincide (for SPI: the detectors of one pointing).  One CTA per
 // group stages the group's rows densely over the union of their columns C
-// (R rows x c columns in shared memory; a single long row is read in place),
-// then takes the columns b of the union one at a time (u_r = w_r h_rb in
-// shared memory) and spreads a = b .. c-1 over its threads, each forming
-// g_ab = sum_r u_r h_ra and adding it to N's entry
-// (C[a], C[b]).  That entry's position comes from a table the host builds at
+// (R rows x c columns in shared memory; a single long row is read in place) and
+// forms g_ab = sum_r (w_r h_rb) h_ra for its column pairs a >= b, adding each to N's
+// entry (C[a], C[b]): the whole product (k_normal_full) spreads all pairs over the
+// CTA's threads, the update (k_normal_group) takes the columns b one at a time and
+// of each only what the marked columns touch.  That entry's position comes from a table the host builds at
 // setup (pair (a, b) of group g at pairptr[g] + b c - b (b - 1) / 2 + a - b,
 // -1 when the pattern has no such entry); when the table would be too large
 // it is found by binary search in column C[b] of the pattern.  Groups share entries of N, so
@@ -28,14 +28,13 @@ namespace {
 
 constexpr int kNThreads = 256;
 
-// kPass 0: the update's zero pass (entries and b of the marked columns set to
-// 0); kPass 1: accumulate.  With mark == nullptr every pair is taken.
+// The update after a change of the marked columns.  kPass 0: the zero pass (entries and b
+// of the marked columns set to 0); kPass 1: accumulate.
 template <int kPass>
 __global__ void __launch_bounds__(kNThreads) k_normal_group(NormalArgs a, const int32_t* __restrict__ groups,
                                                              const double* __restrict__ hv,
                                                              const double* __restrict__ w,
                                                              const double* __restrict__ y,
-                                                             const double* __restrict__ bw,
                                                              const uint8_t* __restrict__ mark,
                                                              double* __restrict__ nv, double* __restrict__ bv,
                                                              int* __restrict__ flag) {
@@ -65,17 +64,16 @@ __global__ void __launch_bounds__(kNThreads) k_normal_group(NormalArgs a, const 
     }
     for (int r = tid; r < R; r += kNThreads) {
         ws[2 * r] = w[r0 + r];
-        ws[2 * r + 1] = bw ? bw[r0 + r] : w[r0 + r] * y[r0 + r];  // b_j = sum_r (w_r y_r or bw_r) h_rj
+        ws[2 * r + 1] = w[r0 + r] * y[r0 + r];
     }
-    // update: the group's marked columns, as a list of union indices (ascending)
+    // the group's marked columns, as a list of union indices (ascending)
     int32_t* ml = reinterpret_cast<int32_t*>(ws + 2 * R);
     double* us = ws + 2 * R;  // u_r = w_r h_rb of the current column b (after ml's space)
     __shared__ int nml;
     if (tid == 0) {
         int k = 0;
-        if (mark)
-            for (int aa = 0; aa < c; ++aa)
-                if (mark[C[aa]]) ml[k++] = aa;
+        for (int aa = 0; aa < c; ++aa)
+            if (mark[C[aa]]) ml[k++] = aa;
         nml = k;
     }
     __syncthreads();
@@ -83,10 +81,10 @@ __global__ void __launch_bounds__(kNThreads) k_normal_group(NormalArgs a, const 
     const double* h1 = hv + a.rowptr[r0];  // the single row's values, in union order
     auto H = [&](int r, int col) { return dense ? Hs[(size_t)r * c + col] : h1[col]; };
     // columns b one at a time across the CTA: g_ab = sum_r u_r h_ra for a = b .. c-1
-    // (with a mark and an unmarked b: only the marked a)
+    // (an unmarked b: only the marked a)
     for (int b = 0; b < c; ++b) {
         const int32_t j = C[b];
-        const bool mb = mark ? mark[j] != 0 : true;
+        const bool mb = mark[j] != 0;
         if (kPass == 1 && tid < R) us[tid] = ws[2 * tid] * H(tid, b);
         if (tid == kNThreads - 1 && mb) {  // b_j = sum_r w_r y_r h_rj
             if (kPass == 0) {
@@ -140,6 +138,93 @@ __global__ void __launch_bounds__(kNThreads) k_normal_group(NormalArgs a, const 
     }
 }
 
+// The whole product: pair t of the group (b-major, the order of the position table) is
+// thread t % 256's, so that a warp's 32 lanes are all at work and its table reads are
+// consecutive; w_r h_rb comes from a second dense copy of the rows, and b_j = sum_r w_r y_r
+// h_rj are c more sums behind the pairs.  Bound by the FP64 pipe (1.26 TFLOP/s).
+// Column by column, with two barriers and a half-empty CTA per column and b_j on one lane, N of
+// P = 5,000 (95,000 rows, 115 columns and 19 rows a group) took 2.51 ms; so 1.10 ms.
+__global__ void __launch_bounds__(kNThreads) k_normal_full(NormalArgs a, const int32_t* __restrict__ groups,
+                                                            const double* __restrict__ hv,
+                                                            const double* __restrict__ w,
+                                                            const double* __restrict__ y,
+                                                            const double* __restrict__ bw, double* __restrict__ nv,
+                                                            double* __restrict__ bv, int* __restrict__ flag) {
+    extern __shared__ __align__(16) double nsm[];
+    const int g = groups[blockIdx.x];
+    const int64_t r0 = a.grp_row[g], r1 = a.grp_row[g + 1];
+    const int R = (int)(r1 - r0);
+    const int64_t c0 = a.grp_colptr[g];
+    const int c = (int)(a.grp_colptr[g + 1] - c0);
+    const int32_t* C = a.grp_cols + c0;
+    const int tid = threadIdx.x;
+    const int64_t e0 = a.rowptr[r0];
+    // position of the pair (C[aa], C[b]) in N, -1 if the pattern has none
+    auto search = [&](int32_t i, int32_t j) -> int64_t {
+        int64_t lo = a.cp[j], hi = a.cp[j + 1];
+        while (lo < hi) { const int64_t mid = (lo + hi) >> 1; if (a.ri[mid] < i) lo = mid + 1; else hi = mid; }
+        return lo < a.cp[j + 1] && a.ri[lo] == i ? lo : -1;
+    };
+    auto add = [&](int64_t q, double v) {
+        if (q >= 0) atomicAdd(nv + q, v);
+        else if (v != 0.0) atomicOr(flag, 1);
+    };
+    const int32_t* pos = a.pairpos ? a.pairpos + a.pairptr[g] : nullptr;
+    if (R == 1) {  // a row on its own (it may be long): a column per warp at a time, read in place
+        const double* h1 = hv + e0;
+        const double wr = w[r0], wy = bw ? bw[r0] : w[r0] * y[r0];
+        const int lane = tid & 31;
+        for (int b = tid >> 5; b < c; b += kNThreads / 32) {
+            const int32_t j = C[b];
+            const double u = wr * h1[b];
+            if (lane == 0) atomicAdd(bv + j, wy * h1[b]);
+            const int64_t o = (int64_t)b * c - (int64_t)b * (b - 1) / 2 - b;
+            for (int aa = b + lane; aa < c; aa += 32)
+                add(pos ? (int64_t)pos[o + aa] : search(C[aa], j), u * h1[aa]);
+        }
+        return;
+    }
+    double* Hs = nsm;                     // [R][c] the rows
+    double* Us = Hs + (size_t)R * c;      // [R][c] the rows times w_r
+    double* wy = Us + (size_t)R * c;      // [R]
+    for (int e = tid; e < 2 * R * c; e += kNThreads) Hs[e] = 0.0;
+    for (int r = tid; r < R; r += kNThreads) wy[r] = bw ? bw[r0 + r] : w[r0 + r] * y[r0 + r];
+    __syncthreads();
+    for (int64_t e = e0 + tid; e < a.rowptr[r1]; e += kNThreads) {
+        int lo = 0, hi = R;  // the row of entry e
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (a.rowptr[r0 + mid] <= e) lo = mid; else hi = mid;
+        }
+        const size_t o = (size_t)lo * c + a.ent_pos[e];
+        const double h = hv[e];
+        Hs[o] = h;
+        Us[o] = w[r0 + lo] * h;
+    }
+    __syncthreads();
+    const int np = c * (c + 1) / 2;  // at most 4,096 x 4,097 / 2 (two rows of 8,192 dense entries)
+    for (int t = tid; t < np + c; t += kNThreads) {
+        if (t >= np) {
+            const int b = t - np;
+            double sb = 0.0;
+            for (int r = 0; r < R; ++r) sb += wy[r] * Hs[r * c + b];
+            atomicAdd(bv + C[b], sb);
+            continue;
+        }
+        // counted from the end the columns hold 1, 2, 3, ... pairs: the k-th from the end, q-th pair
+        const int u = np - 1 - t;
+        int k = (int)((sqrtf(8.0f * (float)u + 1.0f) - 1.0f) * 0.5f);
+        if ((k + 1) * (k + 2) / 2 <= u) ++k;
+        if (k * (k + 1) / 2 > u) --k;
+        const int b = c - 1 - k, aa = c - 1 - (u - k * (k + 1) / 2);
+        const int64_t q = pos ? (int64_t)pos[t] : search(C[aa], C[b]);
+        const double *hp = Hs + aa, *up = Us + b;
+        double sv = 0.0;
+        for (int r = 0; r < R; ++r) sv += up[r * c] * hp[r * c];
+        add(q, sv);
+    }
+}
+
 }  // namespace
 
 size_t normal_smem_bytes(int32_t max_dense_entries, int32_t max_rows, int32_t max_cols) {
@@ -147,20 +232,34 @@ size_t normal_smem_bytes(int32_t max_dense_entries, int32_t max_rows, int32_t ma
            sizeof(int32_t) * (size_t)max_cols;
 }
 
-cudaError_t normal_kernel_setup(size_t smem) {
-    cudaError_t e = cudaFuncSetAttribute(k_normal_group<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+size_t normal_full_smem_bytes(int32_t max_dense_entries, int32_t max_rows) {
+    return sizeof(double) * (2 * (size_t)max_dense_entries + (size_t)max_rows);
+}
+
+cudaError_t normal_kernel_setup(size_t smem, size_t smem_full) {
+    cudaError_t e =
+        cudaFuncSetAttribute(k_normal_full, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_full);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_normal_group<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(k_normal_group<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
 void launch_normal(const NormalArgs& a, const int32_t* groups, int32_t ngroups, const double* hv, const double* w,
-                   const double* y, const double* bw, const uint8_t* mark, bool zero_pass, double* nv, double* bv,
-                   int* flag, size_t smem, cudaStream_t st) {
+                   const double* y, const double* bw, double* nv, double* bv, int* flag, size_t smem_full,
+                   cudaStream_t st) {
+    if (ngroups == 0) return;
+    k_normal_full<<<ngroups, kNThreads, smem_full, st>>>(a, groups, hv, w, y, bw, nv, bv, flag);
+}
+
+void launch_normal_update(const NormalArgs& a, const int32_t* groups, int32_t ngroups, const double* hv,
+                          const double* w, const double* y, const uint8_t* mark, bool zero_pass, double* nv,
+                          double* bv, int* flag, size_t smem, cudaStream_t st) {
     if (ngroups == 0) return;
     if (zero_pass)
-        k_normal_group<0><<<ngroups, kNThreads, smem, st>>>(a, groups, hv, w, y, bw, mark, nv, bv, flag);
+        k_normal_group<0><<<ngroups, kNThreads, smem, st>>>(a, groups, hv, w, y, mark, nv, bv, flag);
     else
-        k_normal_group<1><<<ngroups, kNThreads, smem, st>>>(a, groups, hv, w, y, bw, mark, nv, bv, flag);
+        k_normal_group<1><<<ngroups, kNThreads, smem, st>>>(a, groups, hv, w, y, mark, nv, bv, flag);
 }
 
 // ---- Poisson maximum likelihood (the appendix on low-count fitting): the model

@@ -334,11 +334,16 @@ struct NormalArgs {
     const int32_t* pairpos;     // position in N of pair (a, b), b-major, -1 if absent; or null
 };
 size_t normal_smem_bytes(int32_t max_dense_entries, int32_t max_rows, int32_t max_cols);
-cudaError_t normal_kernel_setup(size_t smem);
-// bw: per-row coefficients of b = H^T bw (null: w * y)
+size_t normal_full_smem_bytes(int32_t max_dense_entries, int32_t max_rows);
+cudaError_t normal_kernel_setup(size_t smem, size_t smem_full);
+// The whole product.  bw: per-row coefficients of b = H^T bw (null: w * y)
 void launch_normal(const NormalArgs& a, const int32_t* groups, int32_t ngroups, const double* hv, const double* w,
-                   const double* y, const double* bw, const uint8_t* mark, bool zero_pass, double* nv, double* bv,
-                   int* flag, size_t smem, cudaStream_t st);
+                   const double* y, const double* bw, double* nv, double* bv, int* flag, size_t smem_full,
+                   cudaStream_t st);
+// The entries and b of the marked columns: the zero pass, then the accumulation.
+void launch_normal_update(const NormalArgs& a, const int32_t* groups, int32_t ngroups, const double* hv,
+                          const double* w, const double* y, const uint8_t* mark, bool zero_pass, double* nv,
+                          double* bv, int* flag, size_t smem, cudaStream_t st);
 void launch_spmv_rows(int64_t nrows, const int64_t* rowptr, const int32_t* colind, const double* hv, const double* x,
                       double* e, cudaStream_t st);
 void launch_mle_rows(int64_t nrows, const double* e, const double* y, double* w, double* v, double* acc,
