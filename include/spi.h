@@ -110,10 +110,12 @@ typedef struct spi_options {
                         factorizations, once per context */
     int force_panel; /* 0 = as chosen above; 1 = every panel on the block-step chain; 2 = every
                         panel whose work allows it in the persistent per-level kernel */
-    int force_schur; /* 0 = as chosen above; 1 = no tensor-core launch at all (SIMT Schur
-                        complements and panel updates); 2 = Schur complements on the tensor
-                        cores wherever legal (mixed precision, at least 256 trailing rows and
-                        32 pivots) */
+    int force_schur; /* 0 = as chosen above (FP64 form, launches level by level: Schur complements
+                        of at least 64 rows and 4 pivots and the panel updates of more than 128
+                        pivots on the tensor cores, products from exact integer pieces); 1 = no
+                        tensor-core launch at all (SIMT Schur complements and panel updates); 2 =
+                        Schur complements on the tensor cores wherever legal (mixed precision, at
+                        least 256 trailing rows and 32 pivots) */
     int dag;         /* 0 = as chosen by the autotuner (timed: one dependency-driven launch against
                         launches level by level, for spi_factor at the first factorization and for
                         spi_solve at the first solve), else on for spi_factor and launches level by
@@ -202,7 +204,8 @@ typedef struct spi_stats {
     double factor_tc_flops;      /* TF32 flops the tensor cores execute per spi_factor: 2 x 128 x 128 x K
                                     per tile and MMA, 6 MMAs per product (split precision) */
     double factor_work_flops;    /* flops the SIMT kernels of spi_factor execute: whole 32 x 32 tiles
-                                    and explicit zeros included (compare factor_flops) */
+                                    and explicit zeros included (compare factor_flops; the FP64
+                                    form's tensor-core products are not among them) */
     int64_t factor_dag_tasks;    /* tasks of the dependency-driven launch (0: none) ... */
     int64_t factor_dag_levels;   /* ... covering the tree levels [0, factor_dag_levels) */
     double tune_ms_launches;     /* the timed factorization with launches level by level ... */

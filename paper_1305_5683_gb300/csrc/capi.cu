@@ -44,7 +44,7 @@ struct spi_ctx {
     int32_t *d_diag_src = nullptr, *d_fwd_items = nullptr, *d_bwd_items = nullptr;
     // the factorization's launch items on the device (per plan: the autotuner's plans have their own)
     struct DevFactorPlan {
-        int32_t* items[15] = {};  // by launch kind
+        int32_t* items[19] = {};  // by launch kind
         DagTask* dag = nullptr;   // the dependency-driven kernel's tasks
         int* counters = nullptr;  // its counters: opt.batch x 2 ns, then the work counter
         std::vector<void*> allocs;
@@ -477,6 +477,8 @@ int upload_factor_plan(spi_ctx* c, const FactorPlan& F, spi_ctx::DevFactorPlan& 
     CK(dev_upload(c, &d.items[2], F.schur_items, tr));
     CK(dev_upload(c, &d.items[3], F.update_items, tr));
     CK(dev_upload(c, &d.items[7], F.schur_tc_items, tr));
+    CK(dev_upload(c, &d.items[17], F.schur_fx_items, tr));
+    CK(dev_upload(c, &d.items[18], F.panel_fx_items, tr));
     CK(dev_upload(c, &d.items[8], F.dfront_items, tr));
     CK(dev_upload(c, &d.items[9], F.panel_tc_items, tr));
     CK(dev_upload(c, &d.items[12], F.fused_items, tr));

@@ -22,6 +22,7 @@
 #include <cmath>
 #include <type_traits>
 
+#include "fx.cuh"
 #include "spi_internal.cuh"
 #include "tcgen05.cuh"
 
@@ -44,6 +45,9 @@ constexpr int32_t kOuter = 128;
 constexpr int32_t kInner = kOuter / kT;
 // tensor-core output tile (rows x columns) and K chunk; one thread per tile row
 constexpr int kTcM = 128, kTcN = 128, kTcK = 32;
+// FP64 tensor-core Schur tiles: rows x columns, K chunk
+constexpr int kFxTileM = 128, kFxTileN = 32, kFxTileK = 32;
+constexpr int32_t kFxGroup = 4;  // column tiles of one CTA when all pivots fit one chunk
 constexpr int kThreads = 128;  // threads of the SIMT front kernels
 static_assert(kTcM == 128 && kTcN == 128, "the tensor-core kernels give thread t row t of both operand tiles");
 
@@ -70,6 +74,17 @@ bool fused_legal(int64_t m, int64_t k) { return m * k * k <= ((int64_t)1 << 26) 
 // the tensor cores from kTcMinRows trailing rows on.
 bool rule_fused(int64_t m, int64_t k) { return m * k * k <= (int64_t)1 << 22 && k <= 256; }
 bool rule_schur_tc(int64_t m, int64_t k) { return m - k >= kTcMinRows; }
+// FP64 form, launches level by level: Schur complements on the tensor cores from exact
+// integer pieces (k_schur_fx), from 64 rows on (at least half a tile filled) and 4 pivots.
+// Factorization level by level of 48 trees of 50-2,000 pointings / of P = 20,000: 2.70 / 7.80 ms;
+// from 33 rows 2.69 / 7.80, 96 rows 2.82 / 7.81, 128 rows 2.98 / 7.80, 256 rows 3.34 / 7.80; from
+// 1 pivot 2.74 / 7.84, 8 pivots 2.72 / 7.91, 16 pivots 2.80 / 8.66.
+bool rule_schur_fx(int64_t m, int64_t k) { return m - k >= 64 && k >= 4; }
+// FP64 form: the panels blocked twice as in the mixed form, the rank-kOuter updates by
+// k_schur_fx<1>, wherever there is an update (one outer block or less has none).  Factorization
+// of P = 20,000 (when written): 9.67 ms with every such front, 9.84 ms with those of 200,000
+// entries or more only, 10.4 ms without.
+bool rule_wide_fx(int64_t, int64_t k) { return k > kOuter; }
 
 namespace {
 
@@ -95,7 +110,7 @@ void append_fused(const Symbolic& S, FactorPlan& F, std::vector<int32_t> fronts)
 // the panel solve, the trailing panel update (whose first tile factors the
 // next pivot tile) and, for wide fronts in mixed precision, the rank-kOuter
 // tensor-core update at the end of each outer block.
-void append_tiled(const Symbolic& S, FactorPlan& F, const std::vector<int32_t>& fronts, bool tensor_cores) {
+void append_tiled(const Symbolic& S, FactorPlan& F, const std::vector<int32_t>& fronts, bool tensor_cores, bool fx) {
     int32_t kmax = 0;
     for (int32_t s : fronts) kmax = std::max(kmax, S.k_of(s));
     const int32_t nsteps = (kmax + kT - 1) / kT;
@@ -104,10 +119,12 @@ void append_tiled(const Symbolic& S, FactorPlan& F, const std::vector<int32_t>& 
         Launch lt{1, b, (int64_t)F.trsm_items.size() / 2, 0};
         Launch lu{3, b, (int64_t)F.update_items.size() / 3, 0};
         Launch lw{9, b, (int64_t)F.panel_tc_items.size() / 3, 0};
+        Launch lx{18, b, (int64_t)F.panel_fx_items.size() / 4, 0};
         for (int32_t s : fronts) {
             const int32_t k = S.k_of(s), m = S.m_of(s);
             if (k <= b * kT) continue;
-            const bool wide = wide_front(tensor_cores, m, k);
+            const bool wide_fx = fx && rule_wide_fx(m, k);
+            const bool wide = wide_fx || wide_front(tensor_cores, m, k);
             if (b == 0 || (wide && b % kInner == 0)) {
                 F.diag_items.push_back(s);
                 ld.count++;
@@ -130,7 +147,16 @@ void append_tiled(const Symbolic& S, FactorPlan& F, const std::vector<int32_t>& 
                 }
             }
             // end of an outer block: rank-kOuter update of panel columns [r0, k)
-            if (wide && r0 == kend && r0 < k) {
+            if (wide_fx && r0 == kend && r0 < k) {
+                for (int32_t ti = 0; r0 + ti * kFxTileM < m; ++ti)
+                    for (int32_t tj = 0; r0 + tj * kFxTileN < k && tj * kFxTileN <= ti * kFxTileM + kFxTileM - 1; ++tj) {
+                        F.panel_fx_items.push_back(s);
+                        F.panel_fx_items.push_back(ti);
+                        F.panel_fx_items.push_back(tj | 1 << 16);
+                        F.panel_fx_items.push_back(0);
+                        lx.count++;
+                    }
+            } else if (wide && r0 == kend && r0 < k) {
                 for (int32_t ti = 0; r0 + ti * kTcM < m; ++ti)
                     for (int32_t tj = 0; r0 + tj * kTcN < k && tj * kTcN <= ti * kTcM + kTcM - 1; ++tj) {
                         F.panel_tc_items.push_back(s);
@@ -144,12 +170,44 @@ void append_tiled(const Symbolic& S, FactorPlan& F, const std::vector<int32_t>& 
         if (lt.count) F.launches.push_back(lt);
         if (lu.count) F.launches.push_back(lu);
         if (lw.count) F.launches.push_back(lw);
+        if (lx.count) F.launches.push_back(lx);
     }
 }
 
-// Schur complements of `simt` (32 x 32 tiles, kind 2) and `tc` (128 x 128
-// tensor-core tiles, kind 7), each added into its parent's front.
-void append_schur(const Symbolic& S, FactorPlan& F, const std::vector<int32_t>& simt, const std::vector<int32_t>& tc) {
+// Schur complements of `simt` (32 x 32 tiles, kind 2), `tc` (128 x 128 tensor-core
+// tiles of the mixed form, kind 7) and `fx` (128 x 32 tensor-core tiles of the FP64 form,
+// kind 17), each added into its parent's front.
+void append_schur(const Symbolic& S, FactorPlan& F, const std::vector<int32_t>& simt, const std::vector<int32_t>& tc,
+                  std::vector<int32_t> fx = {}) {
+    Launch lx{17, 0, (int64_t)F.schur_fx_items.size() / 4, 0};
+    auto ntj_of = [&](int32_t s, int32_t ti) {  // column tiles of row tile ti
+        return (std::min(S.m_of(s) - S.k_of(s), (ti + 1) * kFxTileM) + kFxTileN - 1) / kFxTileN;
+    };
+    // the heaviest CTAs first, none with more than half an even share of the launch (two CTAs
+    // on each of 152 SMs): the kOuter-pivot groups of a tile may be split over several CTAs
+    // (their sums meet in the parent's entries)
+    std::stable_sort(fx.begin(), fx.end(), [&](int32_t a, int32_t b) { return S.k_of(a) > S.k_of(b); });
+    int64_t work = 0;
+    for (int32_t s : fx)
+        for (int32_t ti = 0; ti * kFxTileM < S.m_of(s) - S.k_of(s); ++ti)
+            work += (int64_t)ntj_of(s, ti) * ((S.k_of(s) + kOuter - 1) / kOuter);
+    const int64_t share = std::max<int64_t>(1, work / 608);
+    for (int32_t s : fx) {
+        const int32_t mb = S.m_of(s) - S.k_of(s), group = S.k_of(s) <= kFxTileK ? kFxGroup : 1;
+        const int32_t groups = (S.k_of(s) + kOuter - 1) / kOuter, span = (int32_t)std::min<int64_t>(groups, share);
+        for (int32_t ti = 0; ti * kFxTileM < mb; ++ti) {
+            const int32_t ntj = ntj_of(s, ti);
+            for (int32_t tj = 0; tj < ntj; tj += group)
+                for (int32_t g = 0; g < groups; g += span) {
+                    F.schur_fx_items.push_back(s);
+                    F.schur_fx_items.push_back(ti);
+                    F.schur_fx_items.push_back(tj | std::min(group, ntj - tj) << 16);
+                    F.schur_fx_items.push_back(g | span << 16);
+                    lx.count++;
+                }
+        }
+    }
+    if (lx.count) F.launches.push_back(lx);
     Launch ls{2, 0, (int64_t)F.schur_items.size() / 3, 0};
     for (int32_t s : simt) {
         const int32_t k = S.k_of(s), m = S.m_of(s);
@@ -257,6 +315,7 @@ void build_factor_plan(const Symbolic& S, FactorPlan& F, bool tensor_cores_allow
                        bool markers) {
     F = FactorPlan();
     const bool tensor_cores = tensor_cores_allowed && ch.force_schur != 1;  // 1: no tensor-core launch at all
+    const bool fx_allowed = !tensor_cores_allowed && ch.force_schur != 1;
     if (ch.dag && !markers) {
         // the levels before the first one with a tensor-core launch run as one dependency-driven launch
         int32_t nlev = S.nlevels;
@@ -285,6 +344,7 @@ void build_factor_plan(const Symbolic& S, FactorPlan& F, bool tensor_cores_allow
         std::map<int32_t, std::vector<int32_t>> fused_by, tiled_by;
         std::vector<int32_t> diag_fronts;
         std::map<int32_t, std::vector<int32_t>> simt_by, tc_by;
+        std::vector<int32_t> fx;
         for (int32_t p = S.level_ptr[l]; p < S.level_ptr[l + 1]; ++p) {
             const int32_t s = S.level_list[p];
             const int32_t k = S.k_of(s), m = S.m_of(s);
@@ -293,7 +353,8 @@ void build_factor_plan(const Symbolic& S, FactorPlan& F, bool tensor_cores_allow
                 fused_by[panel_bucket(m, k)].push_back(s);
             else tiled_by[panel_bucket(m, k)].push_back(s);
             if (S.sparent[s] == -1 || m <= k) continue;
-            if (schur_tc_legal(tensor_cores, m, k) && ch.schur_tc(m, k)) tc_by[schur_bucket(m, k)].push_back(s);
+            if (fx_allowed && rule_schur_fx(m, k)) fx.push_back(s);
+            else if (schur_tc_legal(tensor_cores, m, k) && ch.schur_tc(m, k)) tc_by[schur_bucket(m, k)].push_back(s);
             else simt_by[schur_bucket(m, k)].push_back(s);
         }
         if (ch.force_panel == 1 && !diag_fronts.empty()) {
@@ -307,9 +368,10 @@ void build_factor_plan(const Symbolic& S, FactorPlan& F, bool tensor_cores_allow
             // one timed group per (kind, bucket) of the level, launched on its own
             if (!diag_fronts.empty()) { marker(FactorPlan::kDiagFronts, -1); append_fused(S, F, diag_fronts); }
             for (auto& kv : fused_by) { marker(FactorPlan::kPanel, kv.first); append_fused(S, F, kv.second); }
-            for (auto& kv : tiled_by) { marker(FactorPlan::kPanel, kv.first); append_tiled(S, F, kv.second, tensor_cores); }
+            for (auto& kv : tiled_by) { marker(FactorPlan::kPanel, kv.first); append_tiled(S, F, kv.second, tensor_cores, fx_allowed); }
             for (auto& kv : simt_by) { marker(FactorPlan::kSchur, kv.first); append_schur(S, F, kv.second, {}); }
             for (auto& kv : tc_by) { marker(FactorPlan::kSchur, kv.first); append_schur(S, F, {}, kv.second); }
+            if (!fx.empty()) { marker(FactorPlan::kSchur, -1); append_schur(S, F, {}, {}, fx); }
         } else {
             std::vector<int32_t> fused(diag_fronts), tiled, simt, tc;
             for (auto& kv : fused_by) fused.insert(fused.end(), kv.second.begin(), kv.second.end());
@@ -320,8 +382,8 @@ void build_factor_plan(const Symbolic& S, FactorPlan& F, bool tensor_cores_allow
             std::sort(simt.begin(), simt.end());
             std::sort(tc.begin(), tc.end());
             append_fused(S, F, fused);
-            append_tiled(S, F, tiled, tensor_cores);
-            append_schur(S, F, simt, tc);
+            append_tiled(S, F, tiled, tensor_cores, fx_allowed);
+            append_schur(S, F, simt, tc, fx);
         }
         F.level_launch_ptr.push_back((int32_t)F.launches.size());
     }
@@ -1207,6 +1269,245 @@ __global__ void __launch_bounds__(128) k_schur_tc(DevSym d, const int32_t* __res
 }
 
 // ---------------------------------------------------------------------------
+// FP64 products on the tensor cores from exact integer pieces (fx.cuh), 128 x 32 tiles:
+// C_ij = sum_c (L_ic s_c) (L_jc d_c / s_c), s_c the power of two next to sqrt(d_c), which
+// puts both operands on the scale of N's entries.
+// kMode 0: the Schur complement F22 - C over all k pivots, added into the parent's front;
+// an item is (supernode, row tile, first column tile | number of column tiles << 16, first
+// kOuter pivots | number of them << 16), more than one column tile only for up to
+// kFxTileK pivots: the row tile's digit planes then stay.
+// kMode 1: the rank-kOuter trailing update of a wide front (as k_schur_tc<1>), in place.
+// Per kOuter pivots both operands get one exponent per row (a first pass over them) and
+// the level sums (below 2^24) stay in tensor memory; per kFxTileK of them the CTA cuts its
+// operands into digit planes in shared memory (28 digit pairs in 14 MMAs of up to 224
+// columns, the next pivots loaded meanwhile); then the sums are joined, rounded once and
+// added in.  Two CTAs share an SM (73 KB and half the tensor memory
+// each), one cutting while the other multiplies or reads out.  The SIMT kernels are
+// bound by the FP64 pipe: 79,000 cycles of an SM for the multiply-adds of 128 x 32 x 32.
+// Factorization of P = 20,000: 16.8 -> 8.3 ms; its leaves' Schur complements (41,335 tiles, 13
+// pivots on average) take 1.2 ms, 47 % of the issue slots in use (cutting, joining, scattering).
+// A non-finite operand makes its row or column of C NaN.
+constexpr int kSfThreads = 256;
+constexpr int kSfPlaneA = kFxTileM * kFxTileK * 2;  // bytes of a digit plane of the rows
+constexpr int kSfPlaneB = kFxTileN * kFxTileK * 2;
+constexpr size_t kSfSmem =
+    (size_t)kDig * (kSfPlaneA + kSfPlaneB) + (2 * kFxTileM + kFxTileN + kOuter) * sizeof(int) +
+    kFxTileN * sizeof(double*) + 16;
+template <int kMode>
+__global__ void __launch_bounds__(kSfThreads, 2) k_schur_fx(DevSym d, const int32_t* __restrict__ items, int step,
+                                                            double* L, double* F22, const double* __restrict__ D,
+                                                            DevStatus* status, Strides bs) {
+    L += blockIdx.y * bs.L;
+    F22 += blockIdx.y * bs.F22;
+    D += blockIdx.y * bs.n;
+    extern __shared__ __align__(1024) unsigned char sfm[];
+    unsigned char* As = sfm;
+    unsigned char* Bs = sfm + kDig * kSfPlaneA;
+    int* aexp = reinterpret_cast<int*>(Bs + kDig * kSfPlaneB);  // [128]
+    int* bexp = aexp + kFxTileM;                                // [32]
+    int* sc = bexp + kFxTileN;                                  // [128] exponent of s_c
+    int* rowp = sc + kOuter;                                    // [128] row of the parent's front, -1: none
+    double** colp = reinterpret_cast<double**>(rowp + kFxTileM);  // [32] its column, null: none
+    uint64_t* bar = reinterpret_cast<uint64_t*>(colp + kFxTileN);
+    uint32_t* slot = reinterpret_cast<uint32_t*>(bar + 1);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int4 it = reinterpret_cast<const int4*>(items)[blockIdx.x];
+    const int s = it.x, ti = it.y, tj0 = it.z & 0xffff, ntj = it.z >> 16;
+    const int f = d.sfirst[s], k = d.sfirst[s + 1] - f;
+    const int64_t m = d.srowptr[s + 1] - d.srowptr[s];
+    double* P = L + d.lptr[s];
+    const int c1 = (step + 1) * kT;
+    const int kb0 = kMode == 0 ? (it.w & 0xffff) * kOuter : c1 - kOuter;
+    const int kb1 = kMode == 0 ? min(k, kb0 + (it.w >> 16) * kOuter) : c1;
+    const int64_t ob = kMode == 0 ? k : c1;  // first output row and column
+    const int64_t ib = ob + (int64_t)ti * kFxTileM, jlim = kMode == 0 ? m : k;
+    constexpr uint32_t kCols = 256;  // 7 x 32 used
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(tc_smem_u32(slot)), "r"(kCols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    if (tid == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(tc_smem_u32(bar)), "r"(1));
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t tmem = *slot;
+    const int ra = tid & (kFxTileM - 1), ha = tid / kFxTileM;   // rows: row ra, pivots 16 ha ..
+    const int cn = tid & (kFxTileN - 1), kb = tid / kFxTileN;   // columns: column cn, pivots 4 kb ..
+    const int quad = warp & 3, half = warp >> 2;                // read-out: rows 32 quad .., columns 16 half ..
+    double va[16], vb[4];
+    auto load_a = [&](int cb) {
+        const int cw = min(kFxTileK, kb1 - cb);
+#pragma unroll
+        for (int q = 0; q < 16; ++q)
+            va[q] = (ib + ra < m && 16 * ha + q < cw) ? P[(ib + ra) + (int64_t)(cb + 16 * ha + q) * m] : 0.0;
+    };
+    auto load_b = [&](int cb, int64_t jb) {
+        const int cw = min(kFxTileK, kb1 - cb);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int c = 4 * kb + q;
+            vb[q] = (jb + cn < jlim && c < cw) ? P[(jb + cn) + (int64_t)(cb + c) * m] * D[f + cb + c] : 0.0;
+        }
+    };
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int t = 0; t < ntj && ok; ++t) {
+        const int64_t jb = ob + (int64_t)(tj0 + t) * kFxTileN;
+        const bool keep = t > 0;  // the digit planes of the rows are those of the tile before
+        if (kMode == 0 && tid < kFxTileM + kFxTileN && (!keep || tid >= kFxTileM)) {
+            const int p = d.sparent[s];
+            const int kp = d.sfirst[p + 1] - d.sfirst[p];
+            const int64_t mp = d.srowptr[p + 1] - d.srowptr[p], fp = d.f22ptr[p];
+            const int64_t l = tid < kFxTileM ? ib + tid : jb + tid - kFxTileM;
+            const int q = l < m ? d.relmap[d.srowptr[s] + l] : -1;
+            if (tid < kFxTileM) rowp[tid] = q;
+            else  // the columns of the parent's panel, then those of its update area (rows from kp)
+                colp[tid - kFxTileM] = q < 0 ? nullptr
+                                       : q < kp ? L + d.lptr[p] + q * mp
+                                                : F22 + (fp < 0 ? 0 : fp) + (q - kp) * (mp - kp) - kp;
+        }
+        for (int cg = kb0; cg < kb1 && ok; cg += kOuter) {
+            const int gw = min(kOuter, kb1 - cg);
+            // the exponents; from the last pivots to the first, whose values stay for the first product
+            if (!keep && tid < kFxTileM) aexp[tid] = -16384;
+            if (tid < kFxTileN) bexp[tid] = -16384;
+            if (!keep && tid < kOuter) sc[tid] = tid < gw ? fx_scale_exp(D[f + cg + tid]) : 0;
+            int ea = -16384, eb = -16384;
+            for (int cc = (gw - 1) / kFxTileK * kFxTileK; cc >= 0; cc -= kFxTileK) {
+                if (!keep) load_a(cg + cc);
+                load_b(cg + cc, jb);
+                if (cc == (gw - 1) / kFxTileK * kFxTileK) __syncthreads();  // aexp, bexp and sc are set
+                if (!keep)
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) ea = max(ea, fx_scaled_exp_nf(va[q]) + sc[cc + 16 * ha + q]);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) eb = max(eb, fx_scaled_exp_nf(vb[q]) - sc[cc + 4 * kb + q]);
+            }
+            if (ea > -16384) atomicMax(&aexp[ra], ea);
+            if (eb > -16384) atomicMax(&bexp[cn], eb);
+            __syncthreads();
+            ea = aexp[ra];
+            eb = bexp[cn];
+            for (int cc = 0; cc < gw && ok; cc += kFxTileK) {
+                const int cw = min(kFxTileK, gw - cc);
+                if (!keep) {
+#pragma unroll
+                    for (int g = 0; g < 2; ++g) {
+                        const int c0 = 16 * ha + 8 * g;
+                        if (c0 < ((cw + 15) & ~15)) {
+                            unsigned long long x[8];
+#pragma unroll
+                            for (int q = 0; q < 8; ++q)
+                                x[q] = fx_fix(va[8 * g + q], fx_scaled_exp(va[8 * g + q]) + sc[cc + c0 + q], ea);
+                            fx_store_planes<0>(As + (ra >> 3) * 512 + (c0 >> 3) * 128 + (ra & 7) * 16, kSfPlaneA, x);
+                        }
+                    }
+                }
+                {
+                    unsigned long long x[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) x[q] = fx_fix(vb[q], fx_scaled_exp(vb[q]) - sc[cc + 4 * kb + q], eb);
+                    fx_store_planes4<0>(Bs + (cn >> 3) * 512 + (kb >> 1) * 128 + (cn & 7) * 16 + (kb & 1) * 8, kSfPlaneB, x);
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                asm volatile("tcgen05.fence::before_thread_sync;");
+                __syncthreads();
+                if (tid == 0) {
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    const uint32_t id0 = (1u << 4) | ((uint32_t)(kFxTileM >> 4) << 24);
+                    const uint32_t ab = tc_smem_u32(As), bb = tc_smem_u32(Bs);
+                    const int ks = (cw + 15) / 16;
+                    for (int kk = 0; kk < ks; ++kk)
+#pragma unroll
+                        for (int q = 0; q < kDig; ++q)
+                            fx_mma(tmem + q * kFxTileN, fx_desc(ab + q * kSfPlaneA + kk * 256, 512),
+                                   fx_desc(bb + kk * 256, 512), id0 | ((uint32_t)((kDig - q) * kFxTileN >> 3) << 17),
+                                   (cc > 0 || kk > 0 || q > 0) ? 1u : 0u);
+                    fx_commit(bar);
+                }
+                if (cc + kFxTileK < gw) {  // the next pivots, while these are multiplied
+                    load_a(cg + cc + kFxTileK);
+                    load_b(cg + cc + kFxTileK, jb);
+                }
+                ok = !__syncthreads_or(!tc_wait(bar, phase & 1u));
+                if (ok) ++phase;
+            }
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            // output entry (h, r16, j): row 32 quad + 16 r16 + lane / 4 + 8 (j / 2), column 16 half +
+            // 8 h + 2 (lane % 4) + j % 2
+            const int i0 = 32 * quad + (lane >> 2), j0 = 16 * half + 2 * (lane & 3);
+            const int64_t fo = kMode == 0 && cg == 0 ? d.f22ptr[s] : -1;  // (the children's sums once)
+            double old[kMode == 1 ? 16 : 1];  // the loads first: none waits behind a store
+            if constexpr (kMode == 1) {
+#pragma unroll
+                for (int o = 0; o < 16; ++o) {
+                    const int64_t il = ib + i0 + 16 * (o >> 2 & 1) + 8 * (o >> 1 & 1), jl = jb + j0 + 8 * (o >> 3) + (o & 1);
+                    old[o] = (il < m && jl < k && il >= jl) ? P[il + jl * m] : 0.0;
+                }
+            }
+            // the children's sums of entry group o4, loaded while the group before is read out
+            double f22[4] = {0.0, 0.0, 0.0, 0.0};
+            auto load_f22 = [&](int o4) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int64_t il = ib + i0 + 16 * (o4 & 1) + 8 * (j >> 1), jl = jb + j0 + 8 * (o4 >> 1) + (j & 1);
+                    f22[j] = (il < m && jl < m && il >= jl) ? F22[fo + (il - k) + (jl - k) * (m - k)] : 0.0;
+                }
+            };
+            if (fo >= 0) load_f22(0);
+            constexpr int kUnroll = kMode == 1 ? 4 : 1;  // (kMode 0: one copy; four miss the instruction cache, 1.41 against 1.13 ms)
+#pragma unroll kUnroll
+            for (int o4 = 0; o4 < 4; ++o4) {
+                const int r = i0 + 16 * (o4 & 1), c = j0 + 8 * (o4 >> 1);
+                uint32_t u[kDig][4];
+                const uint32_t ta = tmem + ((uint32_t)(32 * quad + 16 * (o4 & 1)) << 16) + 16 * half + 8 * (o4 >> 1);
+#pragma unroll
+                for (int l = 0; l < kDig; ++l) fx_ld16x8(ta + l * kFxTileN, u[l]);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                double v[4], cf[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) cf[j] = f22[j];
+                if (fo >= 0 && o4 < 3) load_f22(o4 + 1);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint32_t a[kDig] = {u[0][j], u[1][j], u[2][j], u[3][j], u[4][j], u[5][j], u[6][j]};
+                    const int e = aexp[r + 8 * (j >> 1)] + bexp[c + (j & 1)] - 2044;
+                    v[j] = e > kFxNonFinite / 2 ? __longlong_as_double(0x7ff8000000000000LL)
+                                                : fx_value(-(gw <= 32 ? fx_join_small(a) : fx_join(a)), e);
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int64_t il = ib + r + 8 * (j >> 1), jl = jb + c + (j & 1);
+                    if constexpr (kMode == 1) {
+                        if (il < m && jl < k && il >= jl) P[il + jl * m] = old[4 * o4 + j] + v[j];
+                    } else {
+                        const int q = rowp[r + 8 * (j >> 1)];
+                        double* pc = colp[c + (j & 1)];
+                        if (q < 0 || pc == nullptr || il < jl) continue;
+                        if (fo >= 0) v[j] += cf[j];
+                        atomicAdd(pc + q, v[j]);
+                    }
+                }
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;");
+            __syncthreads();  // the exponents, digit planes, accumulators and maps are free
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;");
+    }
+    if (!ok) {
+        tc_wait(bar, phase & 1u);  // drain before release
+        if (tid == 0) atomicOr(&status->flags, FLAG_TIMEOUT);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(kCols));
+}
+
+// ---------------------------------------------------------------------------
 // Dependency-driven persistent factorization (launch kind 13).
 //
 // One launch runs every task of a prefix of the tree's levels: diagonal-pivot
@@ -1640,6 +1941,10 @@ cudaError_t factor_kernel_setup() {
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_schur_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
     if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_schur_fx<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSfSmem);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_schur_fx<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSfSmem);
+    if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, b64 = 0, b32 = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
@@ -1698,6 +2003,14 @@ void launch_step_t(const DevSym& d, const Launch& l, const int32_t* items, C* L,
                 else
                     k_schur_tc<1><<<g, 128, kTcSmem, st>>>(d, items + 3 * l.off, l.step, L, F22, DS, status, bs, lim);
             }
+            break;
+        case 17:
+            if constexpr (std::is_same<C, double>::value)  // the FP64 form's tensor-core items
+                k_schur_fx<0><<<g, kSfThreads, kSfSmem, st>>>(d, items + 4 * l.off, 0, L, F22, D, status, bs);
+            break;
+        case 18:
+            if constexpr (std::is_same<C, double>::value)
+                k_schur_fx<1><<<g, kSfThreads, kSfSmem, st>>>(d, items + 4 * l.off, l.step, L, F22, D, status, bs);
             break;
         case 8: k_diag_front<C><<<g, kThreads, 0, st>>>(d, items + l.off, L, D, DS, adiag, status, bs); break;
         case 12: {

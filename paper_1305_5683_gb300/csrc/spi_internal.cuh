@@ -77,6 +77,7 @@ struct Launch {
     int kind;        // 0 pivot tile, 1 panel TRSM, 2 Schur+scatter, 3 trailing panel update,
                      // 7 tensor-core Schur+scatter (mixed precision), 8 diagonal-pivot front,
                      // 9 tensor-core trailing panel update of a wide front (mixed precision),
+                     // 17 FP64 tensor-core Schur+scatter, 18 rank-128 panel update;
                      // 14 symmetric indefinite fronts with 2x2 pivots (one CTA each);
                      // 12 persistent per-level kernel: whole panels of small fronts, one CTA
                      // per front at a time; solves: 4 forward step, 5 backward first launch of
@@ -111,6 +112,9 @@ struct FactorPlan {
     std::vector<int32_t> schur_items; // triples (supernode, ti, tj)
     std::vector<int32_t> update_items;// triples (supernode, ti, tj) of the trailing panel
     std::vector<int32_t> schur_tc_items; // triples (supernode, 128-row tile, 64-column tile)
+    std::vector<int32_t> schur_fx_items; // FP64 form, quadruples (supernode, 128-row tile,
+                                         // 32-column tile | tiles << 16, 128 pivots | number << 16)
+    std::vector<int32_t> panel_fx_items; // the same of the FP64 form's rank-128 panel updates
     std::vector<int32_t> dfront_items;   // supernodes with a diagonal pivot block
     std::vector<int32_t> panel_tc_items; // triples (supernode, 128-row tile, 64-column tile)
     std::vector<int32_t> fused_items;    // kind 12: supernode, or ~supernode for a diagonal pivot block
