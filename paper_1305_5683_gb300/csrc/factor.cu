@@ -890,6 +890,42 @@ __global__ void __launch_bounds__(kThreads) k_panel_trsm(DevSym d, const int32_t
     panel_rows4<false, C>(P, m, c0, w, r0, (int)(m - r0 < kT ? m - r0 : kT), Bd, dv);
 }
 
+// FP64 update of a 32 x 32 tile on the diagonal of a panel, old - Li Lj^T over w pivots, by
+// the CTA: only the lower triangle, 4 or 5 entries a thread where whole columns take 8 (an
+// FP64 warp instruction costs the same with idle lanes).  The tile that becomes the next
+// pivot tile is on the chain of the steps: a step of k_panel_update with few tiles takes 25
+// us (update and pivot tile) against 31.  store(i, j, value).
+template <typename C, bool kCg, typename Store>
+__device__ __forceinline__ void update_triangle(const C (*Li)[kT + 1], const C (*Lj)[kT + 1], const C* T, int64_t m,
+                                                int ni, int nj, int w, Store store) {
+    const int tid = threadIdx.x;
+    constexpr int kE = kT * (kT + 1) / 2, kQ = kE / kThreads;
+    int ei[kQ + 1], ej[kQ + 1];
+    C acc[kQ + 1], old[kQ + 1];
+#pragma unroll
+    for (int q = 0; q <= kQ; ++q) {
+        const int u = min(tid + kThreads * q, kE - 1);  // columns from the last: 1, 2, ... entries
+        int t = (int)((sqrtf(8.0f * (float)u + 1.0f) - 1.0f) * 0.5f);
+        if ((t + 1) * (t + 2) / 2 <= u) ++t;
+        if (t * (t + 1) / 2 > u) --t;
+        ej[q] = kT - 1 - t;
+        ei[q] = kT - 1 - (u - t * (t + 1) / 2);
+        acc[q] = C(0);
+        old[q] = (ei[q] < ni && ej[q] < nj) ? ldx<kCg>(T + ei[q] + (int64_t)ej[q] * m) : C(0);
+    }
+#pragma unroll 4
+    for (int c = 0; c < w; ++c)
+#pragma unroll
+        for (int q = 0; q < kQ; ++q) acc[q] += Li[ei[q]][c] * Lj[ej[q]][c];
+    const bool more = tid < kE - kQ * kThreads;
+    if (more)
+#pragma unroll 4
+        for (int c = 0; c < w; ++c) acc[kQ] += Li[ei[kQ]][c] * Lj[ej[kQ]][c];
+#pragma unroll
+    for (int q = 0; q <= kQ; ++q)
+        if ((q < kQ || more) && ei[q] < ni && ej[q] < nj) store(ei[q], ej[q], old[q] - acc[q]);
+}
+
 // Trailing panel update after block column b: for panel columns j in
 // [c0+w, k) and rows i >= j, P[i][j] -= sum_{c in block b} L[i][c] d_c L[j][c].
 template <typename C>
@@ -924,7 +960,12 @@ __global__ void __launch_bounds__(kThreads) k_panel_update(DevSym d, const int32
     // thread owns row ii and columns j0 + 4 q: a warp's lanes run down one
     // column, so its read-modify-writes of the panel are coalesced
     const int ii = tid % kT, j0 = tid / kT;
-    if (ii < ni) {
+    if (std::is_same<C, double>::value && ti == 0) {
+        update_triangle<C, false>(Li, Lj, P + ri + (int64_t)cj * m, m, ni, nj, w, [&](int i, int j, C v) {
+            if (piv && i < nj) A[i][j] = (double)v;
+            else P[(ri + i) + (int64_t)(cj + j) * m] = v;
+        });
+    } else if (ii < ni) {
         C acc[kT / 4];
 #pragma unroll
         for (int q = 0; q < kT / 4; ++q) acc[q] = C(0);
@@ -1588,7 +1629,10 @@ __device__ void dag_update(const DevSym& d, int s, int b, int ti, int tj, C* Lb,
     }
     __syncthreads();
     const int ii = tid % kT, j0 = tid / kT;
-    if (ii < ni) {
+    if (std::is_same<C, double>::value && ti == 0) {
+        update_triangle<C, true>(sm.upd.Li, sm.upd.Lj, P + ri + (int64_t)cj * m, m, ni, nj, w,
+                                 [&](int i, int j, C v) { P[(ri + i) + (int64_t)(cj + j) * m] = v; });
+    } else if (ii < ni) {
         C acc[kT / 4];
 #pragma unroll
         for (int q = 0; q < kT / 4; ++q) acc[q] = C(0);
