@@ -680,6 +680,8 @@ __global__ void __launch_bounds__(kThreads) k_diag_front(DevSym d, const int32_t
 // Shared memory of the per-level panel kernel; the three phases of a block
 // step use it in turn.
 template <typename C>
+constexpr int kLjLd = kT + (std::is_same<C, float>::value ? 4 : 1);  // row of a Schur tile's scaled operand
+template <typename C>
 union FrontPanelSmem {
     struct {
         double A[kT][kT + 1];
@@ -694,6 +696,10 @@ union FrontPanelSmem {
         C Li[kT][kT + 1];       // 32 rows of the block column
         C Lj[kT][kT + 1];       // 32 rows of the block column scaled by d
     } upd;
+    struct {
+        C Li[kT][kT + 1];
+        alignas(16) C Lj[kT][kLjLd<C>];
+    } sch;                      // a Schur tile (schur_tile)
 };
 
 // The panel solve L21 = X L11^-T D^-1 of 32 rows r0 .. r0 + nr by the CTA, four lanes per
@@ -1003,26 +1009,42 @@ __global__ void __launch_bounds__(kThreads) k_panel_update(DevSym d, const int32
 }
 
 // Schur complement tile (ti, tj) of the trailing (m-k)^2 part, added into the parent's front.
-template <typename C>
-__global__ void __launch_bounds__(kThreads) k_schur_scatter(DevSym d, const int32_t* __restrict__ items,
-                                                            C* __restrict__ L, C* __restrict__ F22,
-                                                            const C* __restrict__ DS, Strides bs) {
-    L += blockIdx.y * bs.L;
-    F22 += blockIdx.y * bs.F22;
-    DS += blockIdx.y * bs.n;
-    __shared__ C Li[kT][kT + 1];
-    __shared__ C Lj[kT][kT + 1];
+// A thread owns row ii and 8 columns, so that a warp's atomics into the parent hit
+// consecutive rows; what the addition needs (the children's sums, the maps) is loaded
+// before any of the atomics.  FP32 tiles are bound by shared-memory loads, so
+// the 8 columns are consecutive and Lj transposed: three loads per 8 multiply-adds where
+// column by column took nine: factorization of 16 bands 5.74 -> 5.58 ms, of P = 20,000 (mixed) 4.85 ->
+// 4.73 ms, of the sky problem of P = 4,000 8.33 -> 8.17 ms.
+template <typename C, bool kCg>
+__device__ __forceinline__ void schur_tile(const DevSym& d, int s, int ti, int tj, C* Lb, C* Fb, const C* DSb,
+                                           C (*Li)[kT + 1], C (*Lj)[kLjLd<C>]) {
+    constexpr bool kRow = std::is_same<C, float>::value;  // Lj[c][column] and columns 8 warp + q
     const int tid = threadIdx.x;
-    const int s = items[3 * blockIdx.x], ti = items[3 * blockIdx.x + 1], tj = items[3 * blockIdx.x + 2];
     const int f = d.sfirst[s], k = d.sfirst[s + 1] - f;
     const int64_t m = d.srowptr[s + 1] - d.srowptr[s];
     const int64_t mb = m - k;
-    const C* P = L + d.lptr[s];
+    const C* P = Lb + d.lptr[s];
     const int64_t ib = k + (int64_t)ti * kT, jb = k + (int64_t)tj * kT;
     const int ni = (int)(m - ib < kT ? m - ib : kT), nj = (int)(m - jb < kT ? m - jb : kT);
-    // thread owns row ii and columns j0 + 4 q: a warp's lanes run down one
-    // column, so its atomics into the parent hit consecutive rows
-    const int ii = tid % kT, j0 = tid / kT;
+    const int ii = tid % kT, warp = tid / kT;
+    const int64_t il = ib + ii;
+    auto col = [&](int q) { return kRow ? 8 * warp + q : warp + 4 * q; };
+    const int64_t fo = d.f22ptr[s];
+    const int p = d.sparent[s];
+    const int32_t* rel = d.relmap + d.srowptr[s];
+    const int qi = ii < ni ? rel[il] : 0;
+    C f22v[kT / 4];
+    int qjv[kT / 4];
+    auto load_parent = [&]() {
+#pragma unroll
+        for (int q = 0; q < kT / 4; ++q) {
+            const int64_t jl = jb + col(q);
+            const bool on = ii < ni && col(q) < nj && il >= jl;
+            f22v[q] = (fo >= 0 && on) ? ldx<kCg>(Fb + fo + (il - k) + (jl - k) * mb) : C(0);
+            qjv[q] = on ? rel[jl] : -1;
+        }
+    };
+    if (kCg) load_parent();  // (few CTAs an SM: in flight behind the products; else it would cost CTAs)
     C acc[kT / 4];
 #pragma unroll
     for (int q = 0; q < kT / 4; ++q) acc[q] = C(0);
@@ -1030,49 +1052,58 @@ __global__ void __launch_bounds__(kThreads) k_schur_scatter(DevSym d, const int3
         const int cw = min(kT, k - cb);
         __syncthreads();
         for (int e = tid; e < kT * kT; e += kThreads) {
-            int i = e % kT, c = e / kT;
-            Li[i][c] = (i < ni && c < cw) ? P[(ib + i) + (int64_t)(cb + c) * m] : C(0);
-            Lj[i][c] = (i < nj && c < cw) ? P[(jb + i) + (int64_t)(cb + c) * m] * DS[f + cb + c] : C(0);
+            const int i = e % kT, c = e / kT;
+            Li[i][c] = (i < ni && c < cw) ? ldx<kCg>(P + (ib + i) + (int64_t)(cb + c) * m) : C(0);
+            const C v = (i < nj && c < cw) ? ldx<kCg>(P + (jb + i) + (int64_t)(cb + c) * m) * ldx<kCg>(DSb + f + cb + c)
+                                           : C(0);
+            if constexpr (kRow) Lj[c][i] = v;
+            else Lj[i][c] = v;
         }
         __syncthreads();
         if (ii < ni) {
 #pragma unroll 4
             for (int c = 0; c < cw; ++c) {  // only the chunk's cw pivots (grouped leaves: often < 32)
                 const C ai = Li[ii][c];
+                if constexpr (kRow) {
+                    const float4 b0 = *reinterpret_cast<const float4*>(&Lj[c][8 * warp]);
+                    const float4 b1 = *reinterpret_cast<const float4*>(&Lj[c][8 * warp + 4]);
+                    acc[0] -= ai * b0.x;
+                    acc[1] -= ai * b0.y;
+                    acc[2] -= ai * b0.z;
+                    acc[3] -= ai * b0.w;
+                    acc[4] -= ai * b1.x;
+                    acc[5] -= ai * b1.y;
+                    acc[6] -= ai * b1.z;
+                    acc[7] -= ai * b1.w;
+                } else {
 #pragma unroll
-                for (int q = 0; q < kT / 4; ++q) acc[q] -= ai * Lj[j0 + 4 * q][c];
+                    for (int q = 0; q < kT / 4; ++q) acc[q] -= ai * Lj[warp + 4 * q][c];
+                }
             }
         }
     }
-    const int64_t fo = d.f22ptr[s];
-    const int p = d.sparent[s];
+    if (!kCg) load_parent();
     const int kp = d.sfirst[p + 1] - d.sfirst[p];
     const int64_t mp = d.srowptr[p + 1] - d.srowptr[p];
-    C* Pp = L + d.lptr[p];
-    C* Fp = F22 + (d.f22ptr[p] < 0 ? 0 : d.f22ptr[p]);
-    const int32_t* rel = d.relmap + d.srowptr[s];
-    if (ii >= ni) return;
-    const int64_t il = ib + ii;
-    const int qi = rel[il];
-    C f22v[kT / 4];  // the update area's entries and the column maps first, then the atomics
-    int qjv[kT / 4];
+    C* Pp = Lb + d.lptr[p];
+    C* Fp = Fb + (d.f22ptr[p] < 0 ? 0 : d.f22ptr[p]);
 #pragma unroll
     for (int q = 0; q < kT / 4; ++q) {
-        const int64_t jl = jb + j0 + 4 * q;
-        const bool on = j0 + 4 * q < nj && il >= jl;
-        f22v[q] = (fo >= 0 && on) ? F22[fo + (il - k) + (jl - k) * mb] : C(0);
-        qjv[q] = on ? rel[jl] : 0;
-    }
-#pragma unroll
-    for (int q = 0; q < kT / 4; ++q) {
-        const int jj = j0 + 4 * q;
-        const int64_t jl = jb + jj;
-        if (jj >= nj || il < jl) continue;
-        const C v = acc[q] + f22v[q];
         const int qj = qjv[q];
+        if (qj < 0) continue;
+        const C v = acc[q] + f22v[q];
         if (qj < kp) atomicAdd(Pp + qi + (int64_t)qj * mp, v);
         else atomicAdd(Fp + (qi - kp) + (int64_t)(qj - kp) * (mp - kp), v);
     }
+}
+
+template <typename C>
+__global__ void __launch_bounds__(kThreads, 8) k_schur_scatter(DevSym d, const int32_t* __restrict__ items, C* L, C* F22,
+                                                            const C* __restrict__ DS, Strides bs) {
+    __shared__ C Li[kT][kT + 1];
+    __shared__ alignas(16) C Lj[kT][kLjLd<C>];
+    schur_tile<C, false>(d, items[3 * blockIdx.x], items[3 * blockIdx.x + 1], items[3 * blockIdx.x + 2],
+                         L + blockIdx.y * bs.L, F22 + blockIdx.y * bs.F22, DS + blockIdx.y * bs.n, Li, Lj);
 }
 
 // ---------------------------------------------------------------------------
@@ -1660,61 +1691,6 @@ __device__ void dag_update(const DevSym& d, int s, int b, int ti, int tj, C* Lb,
     }
 }
 
-// Schur tile (ti, tj) of the trailing block, added into the parent front (as k_schur_scatter).
-template <typename C>
-__device__ void dag_schur(const DevSym& d, int s, int ti, int tj, C* Lb, C* Fb, const C* DSb, FrontPanelSmem<C>& sm) {
-    const int tid = threadIdx.x;
-    const int f = d.sfirst[s], k = d.sfirst[s + 1] - f;
-    const int64_t m = d.srowptr[s + 1] - d.srowptr[s];
-    const int64_t mb = m - k;
-    const C* P = Lb + d.lptr[s];
-    const int64_t ib = k + (int64_t)ti * kT, jb = k + (int64_t)tj * kT;
-    const int ni = (int)(m - ib < kT ? m - ib : kT), nj = (int)(m - jb < kT ? m - jb : kT);
-    const int ii = tid % kT, j0 = tid / kT;
-    C acc[kT / 4];
-#pragma unroll
-    for (int q = 0; q < kT / 4; ++q) acc[q] = C(0);
-    for (int cb = 0; cb < k; cb += kT) {
-        const int cw = min(kT, k - cb);
-        __syncthreads();
-        for (int e = tid; e < kT * kT; e += kThreads) {
-            const int i = e % kT, c = e / kT;
-            sm.upd.Li[i][c] = (i < ni && c < cw) ? __ldcg(P + (ib + i) + (int64_t)(cb + c) * m) : C(0);
-            sm.upd.Lj[i][c] =
-                (i < nj && c < cw) ? __ldcg(P + (jb + i) + (int64_t)(cb + c) * m) * __ldcg(DSb + f + cb + c) : C(0);
-        }
-        __syncthreads();
-        if (ii < ni) {
-#pragma unroll 4
-            for (int c = 0; c < cw; ++c) {
-                const C ai = sm.upd.Li[ii][c];
-#pragma unroll
-                for (int q = 0; q < kT / 4; ++q) acc[q] -= ai * sm.upd.Lj[j0 + 4 * q][c];
-            }
-        }
-    }
-    const int64_t fo = d.f22ptr[s];
-    const int p = d.sparent[s];
-    const int kp = d.sfirst[p + 1] - d.sfirst[p];
-    const int64_t mp = d.srowptr[p + 1] - d.srowptr[p];
-    C* Pp = Lb + d.lptr[p];
-    C* Fp = Fb + (d.f22ptr[p] < 0 ? 0 : d.f22ptr[p]);
-    const int32_t* rel = d.relmap + d.srowptr[s];
-    if (ii >= ni) return;
-    const int64_t il = ib + ii;
-    const int qi = rel[il];
-#pragma unroll
-    for (int q = 0; q < kT / 4; ++q) {
-        const int jj = j0 + 4 * q;
-        const int64_t jl = jb + jj;
-        if (jj >= nj || il < jl) continue;
-        const C v = acc[q] + (fo >= 0 ? __ldcg(Fb + fo + (il - k) + (jl - k) * mb) : C(0));
-        const int qj = rel[jl];
-        if (qj < kp) atomicAdd(Pp + qi + (int64_t)qj * mp, v);
-        else atomicAdd(Fp + (qi - kp) + (int64_t)(qj - kp) * (mp - kp), v);
-    }
-}
-
 template <typename C>
 __global__ void __launch_bounds__(kThreads, sizeof(C) == 4 ? 4 : 3) k_factor_dag(DevSym d, const DagTask* __restrict__ tasks, int ntasks,
                                                          int nb, int* cnt, int cstride, C* L, C* F22, double* D,
@@ -1766,7 +1742,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(C) == 4 ? 4 : 3) k_factor_dag
             }
             case kDagTrsm: dag_trsm(d, tk.s, tk.a, tk.b, Lb, Db, sm); break;
             case kDagUpdate: dag_update(d, tk.s, tk.a, tk.b >> 16, tk.b & 0xFFFF, Lb, Db, DSb, ab, status, base, sm); break;
-            default: dag_schur(d, tk.s, tk.a, tk.b, Lb, Fb, DSb, sm); break;
+            default: schur_tile<C, true>(d, tk.s, tk.a, tk.b, Lb, Fb, DSb, sm.sch.Li, sm.sch.Lj); break;
         }
         __threadfence();  // every thread's stores of the task are visible device-wide ...
         __syncthreads();
