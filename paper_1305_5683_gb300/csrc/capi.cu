@@ -387,7 +387,11 @@ int upload_plan(spi_ctx* c, const DiagPlan& h, DevDiagPlan& d) {
     d.B = h.B; d.nblocks = h.nblocks; d.nrhs = h.nrhs; d.flops = h.flops; d.work_flops = h.work_flops;
     d.tc_flops = c->dtc.ntc > 0 && h.B <= kDiagTcMaxBlock ? diag_tc_mma_flops(sym_sol(c), c->dtc_h, h) : 0.0;
     std::vector<void*>* tr = &d.allocs;
-    CK(dev_upload(c, &d.order, h.order, tr));
+    std::vector<int32_t> order_tc, order = h.order;
+    if (d.tc_flops > 0) diag_tc_orders(sym_sol(c), c->dtc_h, h, order_tc, order);
+    else diag_fx_order(sym_sol(c), h, order_tc);
+    CK(dev_upload(c, &d.order, order, tr));
+    CK(dev_upload(c, &d.order_tc, order_tc, tr));
     CK(dev_upload(c, &d.blk_ptr, h.blk_ptr, tr));
     CK(dev_upload(c, &d.uptr, h.uptr, tr));
     CK(dev_upload(c, &d.us, h.us, tr));
@@ -2165,9 +2169,9 @@ int spi_normal_update(spi_ctx* c, int64_t ncols, const int32_t* cols, const doub
         CK(cudaMemcpyAsync(N.d_mark, mark.data(), (size_t)n, cudaMemcpyHostToDevice, st));
         CK(cudaMemcpyAsync(N.d_sel, sel.data(), sel.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
         launch_normal_update(N.args, N.d_sel, (int32_t)sel.size(), hv, wd, yd, N.d_mark, true, nv, bv, N.d_flag,
-                      N.smem, st);
+                             N.smem, st);
         launch_normal_update(N.args, N.d_sel, (int32_t)sel.size(), hv, wd, yd, N.d_mark, false, nv, bv, N.d_flag,
-                      N.smem, st);
+                             N.smem, st);
     }
     return normal_finish(c, nvals, b, on_device, st);
 }

@@ -596,7 +596,7 @@ void launch_diag_fx(const DevSym& d, const DevDiagPlan& dp, const DevDiagFx& p, 
     k_fx_pack<<<dim3((unsigned)dp.fx_ntiles, nb), kFxRows, 0, st>>>(d, p.tiles, p.tdiag, dp.fx_tiles, p.ntiles, p.npieces,
                                                                     x.xoff, x.nx, L, D, x.xinv, p.pack, p.rexp, p.fr,
                                                                     bs.L, bs.n);
-    FxArgs a{dp.B, dp.order, dp.blk_ptr, dp.uptr, dp.us, dp.ulo, dp.uhi, dp.uzoff, dp.rel, dp.rhs_out,
+    FxArgs a{dp.B, dp.order_tc, dp.blk_ptr, dp.uptr, dp.us, dp.ulo, dp.uhi, dp.uzoff, dp.rel, dp.rhs_out,
              dp.rhs_zrow, dp.rhs_col, dp.urel, dp.zbase, dp.Z, p.pptr, p.tptr, p.npieces, p.ntiles, p.pack, p.rexp,
              D, p.fr};
     k_diag_fx<<<dim3(dp.nblocks, nb), kFxThreads, fx_smem(dp.B), st>>>(d, a, out, bs, status);

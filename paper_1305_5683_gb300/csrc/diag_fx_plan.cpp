@@ -39,4 +39,22 @@ void diag_fx_used(const Symbolic& S, const DiagFxHost& h, const DiagPlan& dp, st
         if (used[h.tiles[4 * t]]) tiles.push_back((int32_t)t);
 }
 
+void diag_fx_order(const Symbolic& S, const DiagPlan& dp, std::vector<int32_t>& order) {
+    std::vector<double> w((size_t)dp.nblocks, 0.0);
+    order.resize((size_t)dp.nblocks);
+    for (int32_t b = 0; b < dp.nblocks; ++b) {
+        order[(size_t)b] = b;
+        for (int32_t u = dp.uptr[b]; u < dp.uptr[b + 1]; ++u) {
+            const int32_t s = dp.us[u], k = S.k_of(s), m = S.m_of(s);
+            const double N = (double)((dp.uhi[u] - (dp.ulo[u] & ~7) + 15) & ~15) / 64.0;
+            for (int32_t c = 0; c < k; c += kFxRows) {
+                const int32_t cw = std::min(kFxRows, k - c), below = m - c - cw;
+                const double tiles = 1.0 + (below + kFxRows - 1) / kFxRows;
+                w[(size_t)b] += tiles * (3000.0 + N * (2200.0 + 900.0 * ((cw + kFxSub - 1) / kFxSub))) + 3000.0;
+            }
+        }
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return w[x] > w[y]; });
+}
+
 }  // namespace spi

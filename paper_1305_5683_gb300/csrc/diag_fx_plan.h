@@ -33,5 +33,11 @@ struct DiagFxHost {
 void build_diag_fx(const Symbolic& S, DiagFxHost& h);
 // the tiles (positions in h.tiles / 4) of the supernodes that plan dp walks
 void diag_fx_used(const Symbolic& S, const DiagFxHost& h, const DiagPlan& dp, std::vector<int32_t>& tiles);
+// The blocks of plan dp in the order in which they start: the costliest first, in cycles of a
+// CTA: per tile 900 a piece and 2,200 for the read-out of 64 right-hand sides and 3,000
+// whatever their number, 3,000 a chunk.  With about four CTAs per SM the last ones to start set
+// the launch's end: by flops, which the many small supernodes of a long path hardly
+// show in, 6.45 ms, so 5.67 (variances of P = 20,000).
+void diag_fx_order(const Symbolic& S, const DiagPlan& dp, std::vector<int32_t>& order);
 
 }  // namespace spi

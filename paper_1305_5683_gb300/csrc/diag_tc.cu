@@ -744,7 +744,7 @@ void launch_diag_inv_tc(const DevSym& d, const DevDiagPlan& dp, const DevDiagTc&
                         int nb, const Strides& bs, DevStatus* status, int wait_limit, cudaStream_t st) {
     if (p.ntc == 0 || dp.nblocks == 0 || nb == 0) return;
     const uint32_t lim = wait_limit > 0 ? (uint32_t)wait_limit : wait_limit < 0 ? 0u : kTcWaitLimit;
-    DiagArgsTc a{dp.B, dp.order, dp.blk_ptr, dp.uptr, dp.us, dp.ulo, dp.uhi, dp.uzoff, dp.rel, dp.rhs_out,
+    DiagArgsTc a{dp.B, dp.order_tc, dp.blk_ptr, dp.uptr, dp.us, dp.ulo, dp.uhi, dp.uzoff, dp.rel, dp.rhs_out,
                  dp.urel, dp.zbase, reinterpret_cast<float*>(dp.Z)};
     DiagTcArgs t{p.tc, p.tptr, p.npt};
     k_diag_inv_tc<<<dim3(dp.nblocks, nb), kDtRoles, kDtSmem2, st>>>(

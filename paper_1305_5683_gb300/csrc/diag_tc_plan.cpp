@@ -3,6 +3,8 @@
 // left-operand tiles that both the packing kernel and the variance kernel use.
 #include "diag_tc_plan.h"
 
+#include <algorithm>
+
 namespace spi {
 
 // Host plan: T = the supernodes with at least min_k pivots and all their
@@ -60,5 +62,30 @@ double diag_tc_mma_flops(const Symbolic& S, const DiagTcHost& h, const DiagPlan&
             fl += chunks * 3.0 * 2.0 * kDiagTcRows * kDiagTcK * N;
         }
     return fl;
+}
+
+void diag_tc_orders(const Symbolic& S, const DiagTcHost& h, const DiagPlan& dp, std::vector<int32_t>& tc,
+                    std::vector<int32_t>& simt) {
+    std::vector<double> wt((size_t)dp.nblocks, 0.0), ws((size_t)dp.nblocks, 0.0);
+    for (int32_t b = 0; b < dp.nblocks; ++b)
+        for (int32_t u = dp.uptr[b]; u < dp.uptr[b + 1]; ++u) {
+            const int32_t s = dp.us[u], k = S.k_of(s), m = S.m_of(s), nbu = dp.uhi[u] - dp.ulo[u];
+            if (!h.tc[s]) {
+                ws[b] += (double)nbu * k * (2.0 * m - k);
+                continue;
+            }
+            const int32_t T = (k + kDiagTcRows - 1) / kDiagTcRows, R = (m - k + kDiagTcRows - 1) / kDiagTcRows,
+                          nch = (k + kDiagTcK - 1) / kDiagTcK;
+            double chunks = (double)R * (nch + 4);
+            for (int32_t rt = 0; rt < T; ++rt) chunks += diag_tc_row_chunks(T, nch, rt) + 4;
+            wt[b] += chunks * (kDiagTcMaxBlock + ((nbu + 31) & ~31));
+        }
+    auto sorted = [&](const std::vector<double>& w, std::vector<int32_t>& o) {
+        o.resize((size_t)dp.nblocks);
+        for (int32_t b = 0; b < dp.nblocks; ++b) o[(size_t)b] = b;
+        std::stable_sort(o.begin(), o.end(), [&](int32_t x, int32_t y) { return w[x] > w[y]; });
+    };
+    sorted(wt, tc);
+    sorted(ws, simt);
 }
 }  // namespace spi

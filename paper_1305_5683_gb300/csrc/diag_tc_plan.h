@@ -42,5 +42,13 @@ SPI_HD inline int32_t diag_tc_row_chunks(int32_t T, int32_t nch, int32_t rt) { r
 void build_diag_tc(const Symbolic& S, int min_k, DiagTcHost& h);
 // TF32 MMA flops (three products per output, padded tiles) of one pass over a plan
 double diag_tc_mma_flops(const Symbolic& S, const DiagTcHost& h, const DiagPlan& dp);
+// The blocks of plan dp in the order in which they start: the costliest first, by what each
+// kernel's CTA does for them -- on the tensor cores the row tiles' chunks and about four
+// chunks' time per tile, half of it whatever the number of right-hand sides; below them the
+// SIMT kernel's flops.  A launch holds about two CTAs per SM, so the last ones to start set
+// its end: ordered by the flops of the whole path, as the plan is, 3.18 ms, so 2.91 (mixed
+// variances of P = 20,000).
+void diag_tc_orders(const Symbolic& S, const DiagTcHost& h, const DiagPlan& dp, std::vector<int32_t>& tc,
+                    std::vector<int32_t>& simt);
 
 }  // namespace spi

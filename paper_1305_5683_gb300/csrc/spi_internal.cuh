@@ -195,6 +195,7 @@ void launch_refined_var(int32_t n, const double* v, const double* r, const int32
 struct DevDiagPlan {
     int32_t B = 0, nblocks = 0;
     int64_t nrhs = 0;
+    int32_t *order_tc = nullptr;  // the blocks as the tensor-core kernels start them
     int32_t *order = nullptr, *blk_ptr = nullptr, *uptr = nullptr, *us = nullptr, *ulo = nullptr,
             *uhi = nullptr, *uzoff = nullptr, *rel = nullptr, *rhs_out = nullptr, *rhs_zrow = nullptr,
             *rhs_col = nullptr;
