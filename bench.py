@@ -1072,9 +1072,19 @@ def main():
     mean_dia = statistics.mean(t_dia) / 1e3
     achieved = info["diag_flops_all"] / mean_dia / 1e12
     pk64, src64 = peak_of(peaks, "fp64_fma")
-    roof = {"bound": "alu", "kernel": "k_diag_inv (pruned blocked forward solves, FP64)",
-            "achieved": achieved, "peak": pk64, "unit": "TFLOP/s", "frac": achieved / pk64,
-            "peak_source": src64, "traffic": traffic_of("diag.cu", "k_diag_inv")}
+    if args.rhs_block in (0, 16, 32, 64):
+        # FP64 products from exact FP16 digits on the tensor cores: 28 digit products each
+        pk16, src16 = peak_of(peaks, "bf16_tcgen05")
+        roof = {"bound": "tensor", "kernel": "k_diag_fx (pruned blocked forward solves, FP64 products as exact "
+                                             "FP16 digit products)",
+                "achieved": 28 * achieved, "peak": pk16, "unit": "TFLOP/s", "frac": 28 * achieved / pk16,
+                "peak_source": src16 + " (the FP16 rate is the BF16 rate)",
+                "traffic": traffic_of("diag_fx.cu", "k_diag_fx"),
+                "algorithmic_tflops_fp64": achieved, "of_fp64_fma_peak": achieved / pk64}
+    else:
+        roof = {"bound": "alu", "kernel": "k_diag_inv (pruned blocked forward solves, FP64)",
+                "achieved": achieved, "peak": pk64, "unit": "TFLOP/s", "frac": achieved / pk64,
+                "peak_source": src64, "traffic": traffic_of("diag.cu", "k_diag_inv")}
     cpu = None
     if not args.no_cpu_baseline and world == 1:
         _, cpu = cpu_baseline(pb)
