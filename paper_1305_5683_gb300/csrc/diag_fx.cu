@@ -32,9 +32,9 @@
 // reads, by asynchronous bulk copies.
 //
 // Measured (one GB300, all variances, against the SIMT kernel on the FP64 pipe): P =
-// 20,000 (n = 39,465) 70.4 -> 6.9 ms, of which the inverses 0.18, the packing 0.14 and the
-// walk 6.4; 48 problems as a forest (n = 51,264) 3.27 -> 1.47 ms; P = 300 (n = 467) 260 ->
-// 118 us.  Largest error against 64-bit dense algebra the same for both (5e-14, rms
+// 20,000 (n = 39,465) 70.4 -> 5.7 ms, of which the packing 0.14 and the walk 5.5 (the
+// inverses, 0.18, come with the factorization); 48 problems as a forest (n = 51,264) 3.27 ->
+// 1.25 ms; P = 300 (n = 467) 260 -> 118 us.  Largest error against 64-bit dense algebra the same for both (5e-14, rms
 // 2.7e-15 at P = 20,000: the factorization's own).  The walk's 73,840 tiles of 128 x 64
 // take 22,000 cycles of an SM each where the products need 7,900: what bounds it is
 // the workers' chain of latencies -- tensor-memory reads, conversions, the read-modify-
