@@ -655,42 +655,66 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_wide(DevSym d, const int32_
 }
 
 // The FP64 form's wide steps take 64 columns (the diagonal 64 x 64 blocks of a tile's inverse
-// are the inverses of its blocks): a warp's FP64 instruction takes its pipe 64 cycles, so every
-// thread gets 16 products of x_b = X_bb w_b (four threads per row; backward from the
-// transposed copy of X, so that the loads coalesce in both directions) and 16 of L's part,
-// at most 0.7 us each.  One solve at P = 20,000 (134 steps and 12 first passes): 2.89 ms in
-// 32-column steps, 1.81 in 128-column ones (16 us a step of FP64 work that every CTA
-// repeats), 1.29 in 64-column ones, 0.80 with the launches chained; P = 300 150 -> 66 us.
+// are the inverses of its blocks): a warp's FP64 instruction takes its pipe 64 cycles, and
+// every CTA of a step forms x_b for itself.  x_b = X_bb w_b alone is not as accurate as the
+// substitution it replaces: its error is relative to |X_bb| |w_b|, which cancels where the
+// block is ill-conditioned (a Gaussian kernel matrix with condition 1e11: residual 1e-12 of
+// ||N|| ||x||, x off by 9e-2 where substitution gives 4e-6).  So every step corrects x_b once
+// by its residual, x_b += X_bb (w_b - L_bb x_b): the error left is the product of two such
+// errors, below the substitution's own (residual 2e-17 where substitution leaves 5e-17).
+// Triangular products take only their nonzero part: four neighbouring lanes share a row, and
+// the eight warps take the groups of 8 rows so that the two warps of each scheduler have
+// 18 multiply-adds a thread between them (32 with the zeros).  L_bb and this CTA's part of L are
+// loaded before x_b is known.
+// One solve at P = 20,000 (134 steps and 12 first passes): 2.89 ms in 32-column steps, 1.81
+// in 128-column ones, 1.02 in these (0.78 without the correction); P = 300 150 -> 68 us.
+// A step: 0.9 us for each of the three products, 1.4 for L's part, 0.6 to read w.
 constexpr int kW64 = 64;
 constexpr int kLpr = kThreads / kW64;    // threads per row or column
 constexpr int kPer64 = kW64 / kLpr;      // products of each
+static_assert(kThreads == 256 && kLpr == 4, "eight warps of 8 rows, four lanes per row");
 
+// A w x w triangular product's row of this thread and its nq products that can be nonzero, the
+// j-th with column col + 4 j: lower (up to the row's group of 8) or upper (from it on); none in
+// groups beyond w.  An even number where the columns go up to the 64th, and uniform in a warp.
+struct TriRow {
+    int r, col, nq;
+};
+__device__ __forceinline__ TriRow tri_row(int w, bool upper) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = warp < 4 ? warp : 11 - warp;
+    const int all = (w + kLpr - 1) / kLpr, q0 = upper ? 2 * g : 0;
+    return TriRow{8 * g + (lane >> 2), kLpr * q0 + (lane & 3), 8 * g < w ? (upper ? all - q0 : min(2 * g + 2, all)) : 0};
+}
 // This thread's part of the w x w block X at columns 64 b of supernode s (or of X^T, from the
-// transposed copy), and x = X v once v is in shared memory.
+// transposed copy).
 __device__ __forceinline__ void wide_load64(const WideArgs& wa, int band, int s, int b, int k, int w, bool transposed,
-                                            double (&xv)[kPer64]) {
-    const int t = wa.xptr[s] + b / 2, o = (b & 1) * kW64, ld = min(kW, k - (b / 2) * kW);
-    const double* X = (transposed ? wa.xinvt64 : wa.xinv64) + band * wa.xband64 + wa.xoff64[t] + o + (int64_t)o * ld;
-    const int r = threadIdx.x % kW64, h = threadIdx.x / kW64;
+                                            const TriRow& t, double (&xv)[kPer64]) {
+    const int tile = wa.xptr[s] + b / 2, o = (b & 1) * kW64, ld = min(kW, k - (b / 2) * kW);
+    const double* X = (transposed ? wa.xinvt64 : wa.xinv64) + band * wa.xband64 + wa.xoff64[tile] + o + (int64_t)o * ld;
 #pragma unroll
-    for (int q = 0; q < kPer64; ++q) {
-        const int c = kLpr * q + h;
-        xv[q] = (r < w && c < w && (transposed ? c >= r : c <= r)) ? X[r + c * ld] : 0.0;
+    for (int j = 0; j < kPer64; ++j) {
+        const int c = t.col + kLpr * j;
+        xv[j] = (t.r < w && c < w && (transposed ? c >= t.r : c <= t.r)) ? X[t.r + c * ld] : 0.0;
     }
 }
-__device__ __forceinline__ void wide_apply64(const double (&xv)[kPer64], int w, const double* v, double* x,
-                                             double (*part)[kW64]) {
-    const int r = threadIdx.x % kW64, h = threadIdx.x / kW64;
-    double y = 0.0;
+// y0 + the sum over this thread's row of a(j, column) v[column], for every lane of the row.  (The
+// loop is left by a branch: multiply-adds merely predicated off take their time all the same.)
+template <typename A>
+__device__ __forceinline__ double tri_sum(const TriRow& t, double y0, const double* v, A a) {
+    if (t.nq == 0) return y0;
+    double y = (threadIdx.x & (kLpr - 1)) == 0 ? y0 : 0.0;
 #pragma unroll
-    for (int q = 0; q < kPer64; ++q) {
-        if (kLpr * q >= w) break;
-        y = fma(xv[q], v[kLpr * q + h], y);
+    for (int j = 0; j < kPer64; j += 2) {
+        if (j >= t.nq) break;
+        y = fma(a(j, t.col + kLpr * j), v[t.col + kLpr * j], y);
+        y = fma(a(j + 1, t.col + kLpr * j + kLpr), v[t.col + kLpr * j + kLpr], y);
     }
-    part[h][r] = y;
-    __syncthreads();
-    if (h == 0) x[r] = (part[0][r] + part[1][r]) + (part[2][r] + part[3][r]);
-    __syncthreads();
+    y += __shfl_xor_sync(0xffffffffu, y, 1);
+    return y + __shfl_xor_sync(0xffffffffu, y, 2);
+}
+__device__ __forceinline__ void copy8(double* dst, const double* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;"
+                 :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
 
 __global__ void __launch_bounds__(kThreads, 2) k_fwd_wide64(DevSym d, const int32_t* __restrict__ items, int b,
@@ -700,30 +724,50 @@ __global__ void __launch_bounds__(kThreads, 2) k_fwd_wide64(DevSym d, const int3
     L += band * bs.L;
     w += band * bs.n;
     z += band * bs.n;
-    __shared__ double wv[kW64], xb[kW64], part[kLpr][kW64];
+    __shared__ double wv[kW64], xb[kW64], rv[kW64], part[kLpr][kW64];
+    __shared__ double T[kW64][kW64 + 1];  // L_bb, zero above the diagonal
     const int s = items[2 * blockIdx.x], chunk = items[2 * blockIdx.x + 1];
     const int f = d.sfirst[s], k = d.sfirst[s + 1] - f;
     const int64_t m = d.srowptr[s + 1] - d.srowptr[s];
     const double* P = L + d.lptr[s];
     const int32_t* rows = d.srows + d.srowptr[s];
     const int cb = b * kW64, wb = min(kW64, k - cb);
-    const int tid = threadIdx.x, h = tid / kW64;
-    // this thread's part of L, in flight while x_b is formed: a row of the chunk, every fourth column
-    const int64_t r = cb + wb + (int64_t)chunk * kW64 + tid % kW64;
+    const int tid = threadIdx.x, h = tid / kW64, rr = tid % kW64;
+    // all that needs no earlier kernel, in flight while the one before runs: L_bb, the rows of
+    // X_bb, and this thread's part of the rows below (a row of the chunk, every fourth column)
+#pragma unroll
+    for (int q = 0; q < kPer64; ++q) {
+        const int c = kLpr * q + h;
+        if (rr < wb && c < rr) copy8(&T[rr][c], P + (cb + rr) + (int64_t)(cb + c) * m);
+        else T[rr][c] = c == rr ? 1.0 : 0.0;
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const TriRow t = tri_row(wb, false);
+    double xv[kPer64];
+    wide_load64(wa, band, s, b, k, wb, false, t, xv);
+    const int64_t r = cb + wb + (int64_t)chunk * kW64 + rr;
     double l[kPer64];
 #pragma unroll
     for (int q = 0; q < kPer64; ++q) {
         const int c = kLpr * q + h;
         l[q] = (r < m && c < wb) ? P[r + (int64_t)(cb + c) * m] : 0.0;
     }
-    double xv[kPer64];
-    wide_load64(wa, band, s, b, k, wb, false, xv);
     const int32_t row = r < m ? rows[r] : 0;
     chain_wait();
     chain_next();
     if (tid < kW64) wv[tid] = tid < wb ? __ldcg(w + f + cb + tid) : 0.0;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
-    wide_apply64(xv, wb, wv, xb, part);
+    const bool own = (tid & (kLpr - 1)) == 0;
+    const double x1 = tri_sum(t, 0.0, wv, [&](int j, int) { return xv[j]; });
+    if (own) xb[t.r] = x1;
+    __syncthreads();
+    const double res = tri_sum(t, wv[t.r], xb, [&](int, int c) { return -T[t.r][c]; });
+    if (own) rv[t.r] = res;
+    __syncthreads();
+    const double x2 = tri_sum(t, x1, rv, [&](int j, int) { return xv[j]; });
+    if (own) xb[t.r] = x2;
+    __syncthreads();
     if (chunk == 0 && tid < wb) z[f + cb + tid] = xb[tid];
     double acc = 0.0;
 #pragma unroll
@@ -731,7 +775,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_fwd_wide64(DevSym d, const int3
         if (kLpr * q >= wb) break;
         acc = fma(l[q], xb[kLpr * q + h], acc);
     }
-    part[h][tid % kW64] = acc;
+    part[h][rr] = acc;
     __syncthreads();
     if (tid < kW64 && r < m) {
         const double sum = (part[0][tid] + part[1][tid]) + (part[2][tid] + part[3][tid]);
@@ -747,8 +791,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_wide64(DevSym d, const int3
     L += band * bs.L;
     w += band * bs.n;
     x += band * bs.n;
-    __shared__ double yv[kW64], xb[kW64], part[kLpr][kW64];
-    __shared__ double T[kW64][kW64 + 1];  // T[a][r] = L[cb + r][column a of the chunk]
+    __shared__ double yv[kW64], xb[kW64], rv[kW64], part[kLpr][kW64];
+    // L_bb^T (T[c][r] = L_bb[r][c], zero above L_bb's diagonal), then the chunk's part of L: T[a][r] =
+    // L[cb + r][column a of the chunk]
+    __shared__ double T[kW64][kW64 + 1];
     const int s = items[2 * blockIdx.x], chunk = items[2 * blockIdx.x + 1];
     const int f = d.sfirst[s], k = d.sfirst[s + 1] - f;
     const int64_t m = d.srowptr[s + 1] - d.srowptr[s];
@@ -756,23 +802,40 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_wide64(DevSym d, const int3
     const int cb = b * kW64, wb = min(kW64, k - cb);
     const int tid = threadIdx.x, q0 = tid % kW64, h = tid / kW64;
     const int a0 = chunk * kW64, na = min(kW64, cb - a0);
-    double xv[kPer64];
-    wide_load64(wa, band, s, b, k, wb, true, xv);
-    if (na > 0) {  // coalesced down the rows, read back by columns
-        double l[kPer64];
 #pragma unroll
-        for (int q = 0; q < kPer64; ++q) {
-            const int a = kLpr * q + h;
-            l[q] = (q0 < wb && a < na) ? P[(cb + q0) + (int64_t)(a0 + a) * m] : 0.0;
-        }
+    for (int q = 0; q < kPer64; ++q) {  // coalesced down the rows, read back by columns
+        const int a = kLpr * q + h;
+        if (q0 < wb && a < q0) copy8(&T[a][q0], P + (cb + q0) + (int64_t)(cb + a) * m);
+        else T[a][q0] = a == q0 ? 1.0 : 0.0;
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const TriRow t = tri_row(wb, true);
+    double xv[kPer64], l[kPer64];  // the rows of X_bb^T; this thread's part of the chunk (row q0)
+    wide_load64(wa, band, s, b, k, wb, true, t, xv);
 #pragma unroll
-        for (int q = 0; q < kPer64; ++q) T[kLpr * q + h][q0] = l[q];
+    for (int q = 0; q < kPer64; ++q) {
+        const int a = kLpr * q + h;
+        l[q] = (q0 < wb && a < na) ? P[(cb + q0) + (int64_t)(a0 + a) * m] : 0.0;
     }
     chain_wait();
     chain_next();
     if (tid < kW64) yv[tid] = tid < wb ? __ldcg(w + f + cb + tid) : 0.0;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
-    wide_apply64(xv, wb, yv, xb, part);
+    const bool own = (tid & (kLpr - 1)) == 0;
+    const double x1 = tri_sum(t, 0.0, yv, [&](int j, int) { return xv[j]; });
+    if (own) xb[t.r] = x1;
+    __syncthreads();
+    const double res = tri_sum(t, yv[t.r], xb, [&](int, int c) { return -T[t.r][c]; });
+    if (own) rv[t.r] = res;
+    __syncthreads();
+    if (na > 0) {
+#pragma unroll
+        for (int q = 0; q < kPer64; ++q) T[kLpr * q + h][q0] = l[q];
+    }
+    const double x2 = tri_sum(t, x1, rv, [&](int j, int) { return xv[j]; });
+    if (own) xb[t.r] = x2;
+    __syncthreads();
     if (chunk == 0 && tid < wb) x[f + cb + tid] = xb[tid];
     if (na <= 0) return;
     double acc = 0.0;

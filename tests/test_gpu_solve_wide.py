@@ -6,6 +6,7 @@ the 1e-10 of the parity tests."""
 import numpy as np
 import pytest
 
+import exact
 import oracle
 from spigen import SCALE, BAND, generate, generate_bands, random_spd, scaled
 
@@ -62,3 +63,33 @@ def test_bands_with_fused_and_stepped_levels(P, precision):
         pb = bands.band(k)
         ref = oracle.OracleFactor.from_problem(pb).solve(pb.b)
         assert np.abs(x[k] - ref).max() <= (1e-10 if precision == 0 else 1e-8) * np.abs(ref).max()
+
+
+def ill_conditioned(kind, c, n):
+    """Matrices whose diagonal blocks have large inverses: a Gaussian kernel plus a diagonal of
+    10^-c, and the square of a second difference plus 10^-c."""
+    if kind == "kernel":
+        t = np.linspace(0.0, 1.0, n)
+        return np.exp(-((t[:, None] - t) / 0.1) ** 2) + 10.0 ** -c * np.eye(n)
+    a = 2.0 * np.eye(n) - np.eye(n, k=1) - np.eye(n, k=-1)
+    return a @ a + 10.0 ** -c * np.eye(n)
+
+
+@pytest.mark.parametrize("n", [40, 64, 65, 130, 200])
+@pytest.mark.parametrize("kind,c", [("kernel", 4), ("kernel", 8), ("kernel", 11), ("difference", 4), ("difference", 9)])
+def test_ill_conditioned_front(P, kind, c, n):
+    """The steps' inverted blocks leave no larger residual than substitution (the
+    dependency-driven form, dag = 2), whatever the blocks' condition: a backward error within
+    n 2^-53, and within four times substitution's or the unit roundoff."""
+    a = ill_conditioned(kind, c, n)
+    pb = exact.problem(a)
+    rng = np.random.default_rng(n + c)
+    err = {1: [], 2: []}
+    for _ in range(3):
+        b = a @ rng.standard_normal(n)
+        for dag in err:
+            s = P.Solver.for_problem(pb, dag=dag)
+            s.factor(pb.values)
+            err[dag].append(exact.backward_error(a, s.solve(b), b))
+    assert max(err[1]) <= n * EPS
+    assert np.median(err[1]) <= 4 * max(np.median(err[2]), EPS)
