@@ -1693,10 +1693,9 @@ int inverse_block_impl(spi_ctx* c, std::vector<int32_t>& key, double* od, cudaSt
         std::vector<int32_t> piv((size_t)nidx), pos((size_t)nidx);
         for (int64_t t = 0; t < nidx; ++t) { piv[t] = S.iperm[key[t]]; pos[t] = (int32_t)t; }
         DiagPlan h;
-        int rc = ensure_fx(c);
-        if (rc) return rc;
-        build_diag_plan(S, piv, pos, c->fx_state == 1 ? fx_block(nidx) : c->rhs_block_used > 0 ? c->rhs_block_used : 32, h);
-        rc = upload_plan(c, h, c->plan_blk);
+        // (on the FP64 pipe; a block size chosen for the tensor cores says nothing about it)
+        build_diag_plan(S, piv, pos, c->rhs_block_used > 0 && c->fx_state != 1 ? c->rhs_block_used : 32, h);
+        int rc = upload_plan(c, h, c->plan_blk);
         if (rc) return rc;
         // rows of the union of all blocks' paths (ascending pivots), and each
         // block-local Z row's position among them; a block's supernodes own
@@ -1735,8 +1734,7 @@ int inverse_block_impl(spi_ctx* c, std::vector<int32_t>& key, double* od, cudaSt
         c->plan_blk_key.swap(key);
         c->plan_blk_ready = true;
     }
-    launch_inverse_block(c->dsym, c->plan_blk, c->fx_state == 1 ? &c->fx : nullptr, c->ti, c->d_L, c->d_D,
-                         c->d_out, c->d_zg, c->blk_rows, od, nidx, c->d_status, st);
+    launch_inverse_block(c->dsym, c->plan_blk, c->d_L, c->d_D, c->d_out, c->d_zg, c->blk_rows, od, nidx, st);
     return SPI_OK;
 }
 }  // namespace

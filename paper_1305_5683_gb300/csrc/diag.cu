@@ -418,14 +418,17 @@ void launch_t(const DevSym& d, const DevDiagPlan& p, const T* L, const double* D
 // any set of entries of the inverse).  After k_diag_inv<double> has run on a
 // single block, Z holds z_t = L^-1 e_(pivot of slot t) on the union of the
 // block's paths, local row r belonging to pivot zpiv[r].  Since
-// N^-1 = L^-T D^-1 L^-1, G_st = sum_r Z[r][s] Z[r][t] / d_zpiv[r] (or, with the scaled vectors
-// of diag_fx.cu, times the weights wt).  One CTA
+// N^-1 = L^-T D^-1 L^-1, G_st = sum_r Z[r][s] Z[r][t] / d_zpiv[r].  The vectors come from the
+// FP64 pipe's kernel, not from diag_fx.cu: that one's errors are relative to the largest entries
+// of a vector, which a variance (a sum of squares) does not feel but a small covariance does
+// (between unknowns of P = 800, 48 random ones: 1.6e-7 of an entry at worst, 4e-14 in the median,
+// where these vectors give 3e-12 and 7e-15).  One CTA
 // per 32 x 32 tile of the lower triangle of G; rows in chunks of 32 staged in
 // shared memory; thread (jj, i0) owns column jj and rows i0 + 4q of the tile.
 // The result goes to out[rhs_out[s] * ldo + rhs_out[t]] and its mirror.
 __global__ void __launch_bounds__(128) k_inverse_gram(const double* __restrict__ Z, int B, int64_t R,
                                                       const int32_t* __restrict__ zpiv,
-                                                      const double* __restrict__ D, const double* __restrict__ wt,
+                                                      const double* __restrict__ D,
                                                       const int32_t* __restrict__ rhs_out, double* __restrict__ out,
                                                       int64_t ldo) {
     __shared__ double Zs[kT][kT + 1];
@@ -447,7 +450,7 @@ __global__ void __launch_bounds__(128) k_inverse_gram(const double* __restrict__
             Zs[rr][c] = (r < R && s0 + c < B) ? Z[r * B + s0 + c] : 0.0;
             Zt[rr][c] = (r < R && t0 + c < B) ? Z[r * B + t0 + c] : 0.0;
         }
-        if (tid < kT) w[tid] = r0 + tid < R ? (wt ? wt[zpiv[r0 + tid]] : 1.0 / D[zpiv[r0 + tid]]) : 0.0;
+        if (tid < kT) w[tid] = r0 + tid < R ? 1.0 / D[zpiv[r0 + tid]] : 0.0;
         __syncthreads();
 #pragma unroll 4
         for (int rr = 0; rr < kT; ++rr) {
@@ -486,22 +489,17 @@ __global__ void k_gather_blocks(const double* __restrict__ Z, int B, const int64
 
 }  // namespace
 
-void launch_inverse_block(const DevSym& d, const DevDiagPlan& p, const DevDiagFx* fx, const DevTileInv& x, const double* L, const double* D,
-                          double* var_scratch, double* Zg, int64_t R, double* out, int64_t ldo, DevStatus* status,
-                          cudaStream_t st) {
+void launch_inverse_block(const DevSym& d, const DevDiagPlan& p, const double* L, const double* D,
+                          double* var_scratch, double* Zg, int64_t R, double* out, int64_t ldo, cudaStream_t st) {
     if (p.nblocks == 0 || p.nrhs == 0) return;
     Strides bs;
     bs.Z = p.zsize;
     bs.out = p.nrhs;
-    bs.n = d.n;
     cudaMemsetAsync(Zg, 0, (size_t)R * (size_t)p.nrhs * sizeof(double), st);
-    const bool tc = fx && p.fx;
-    if (tc) launch_diag_fx(d, p, *fx, x, L, D, var_scratch, 1, bs, status, st);
-    else launch_t<double>(d, p, L, D, var_scratch, 1, bs, 0, st);
+    launch_t<double>(d, p, L, D, var_scratch, 1, bs, 0, st);
     k_gather_blocks<<<p.nblocks, 256, 0, st>>>(p.Z, p.B, p.zbase, p.blk_ptr, p.rowmap, p.nrhs, Zg);
     const int nt = (int)((p.nrhs + kT - 1) / kT);
-    k_inverse_gram<<<nt * (nt + 1) / 2, 128, 0, st>>>(Zg, (int)p.nrhs, R, p.zpiv, D, tc ? fx->fr : nullptr, p.rhs_out, out,
-                                                       ldo);
+    k_inverse_gram<<<nt * (nt + 1) / 2, 128, 0, st>>>(Zg, (int)p.nrhs, R, p.zpiv, D, p.rhs_out, out, ldo);
 }
 
 namespace {

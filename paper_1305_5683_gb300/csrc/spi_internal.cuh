@@ -263,6 +263,13 @@ void launch_pick_entries(const double* G, const int64_t* src, const int64_t* dst
                          cudaStream_t st);
 // smem_min: the launches' dynamic shared memory is at least this (0: what they need)
 cudaError_t diag_kernel_setup(int B, size_t smem_min);
+// (N^-1)(I, I) for the pivots of a plan with zpiv/rowmap: the blocks' forward
+// solves (variances to var_scratch), their vectors gathered into Zg (R rows x
+// nrhs), then the Gram product into out (ldo = leading dimension, positions
+// from the plan's rhs_out).
+void launch_inverse_block(const DevSym& d, const DevDiagPlan& p, const double* L, const double* D,
+                          double* var_scratch, double* Zg, int64_t R, double* out, int64_t ldo, cudaStream_t st);
+
 // ---- diag_tc.cu: the mixed form's variances on the tensor cores for the
 // supernodes with at least min_k pivots and their ancestors
 struct DevDiagTc {
@@ -316,14 +323,6 @@ size_t diag_fx_pack_bytes(int64_t npieces);
 // 16, 32 or 64)
 void launch_diag_fx(const DevSym& d, const DevDiagPlan& dp, const DevDiagFx& p, const DevTileInv& x, const double* L, const double* D,
                     double* out, int nb, const Strides& bs, DevStatus* status, cudaStream_t st);
-
-// (N^-1)(I, I) for the pivots of a plan with zpiv/rowmap: the blocks' forward
-// solves (variances to var_scratch; on the tensor cores with fx, when the plan has fx
-// set), their vectors gathered into Zg (R rows x nrhs), then the Gram product into
-// out (ldo = leading dimension, positions from the plan's rhs_out).
-void launch_inverse_block(const DevSym& d, const DevDiagPlan& p, const DevDiagFx* fx, const DevTileInv& x, const double* L, const double* D,
-                          double* var_scratch, double* Zg, int64_t R, double* out, int64_t ldo, DevStatus* status,
-                          cudaStream_t st);
 
 // ---- normal.cu: N = H^T W H and b = H^T W y on the device
 struct NormalArgs {

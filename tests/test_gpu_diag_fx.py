@@ -9,6 +9,7 @@ their largest entries)."""
 import numpy as np
 import pytest
 
+import exact
 import oracle
 from spigen import SCALE, BAND, generate, generate_bands, random_spd, scaled, sky_scaled
 
@@ -118,3 +119,21 @@ def test_inverse_block_on_the_scaled_vectors(P, count):
     d = np.sqrt(np.diag(R))
     assert np.abs(G - R).max() <= 1e-10 * np.abs(R).max()
     assert (np.abs(G - R) / np.outer(d, d)).max() <= 64 * 600 * EPS + 1e-10
+
+
+@pytest.mark.parametrize("weak", [1e-3, 1e-8, 1e-14])
+def test_covariances_of_weakly_coupled_unknowns(P, weak):
+    """Two groups of unknowns in one front, coupled `weak` times as strongly as within a group: the
+    covariances between the groups, `weak` times the variances, keep their own digits."""
+    n = 60
+    rng = np.random.default_rng(4)
+    g = np.arange(n) % 2
+    a = rng.uniform(0.5, 1.0, (n, n)) * np.where(g[:, None] == g, 1.0, weak)
+    a = np.tril(a, -1)
+    a = a + a.T + np.diag(np.full(n, float(n)))
+    ref = exact.inverse(a)
+    s = P.Solver.for_problem(exact.problem(a))
+    s.factor(exact.problem(a).values)
+    got = s.inverse_block(np.arange(n, dtype=np.int32))
+    err = np.abs(got / ref.astype(float) - 1)
+    assert err.max() <= 64 * n * EPS
