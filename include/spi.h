@@ -80,14 +80,17 @@ typedef struct spi_options {
     int nd_leaf;     /* nested-dissection leaf size (vertices); 0 = default */
     int batch;       /* maximum number of same-pattern bands of the *_batch calls (device memory
                         is sized for it at the first factorization); 0 or 1 = single problem */
-    int wait_limit;  /* polls allowed to each bounded device wait of spi_factor: the pipeline
-                        waits of the tensor-core kernels (mixed form; default 2^20) and the
+    int wait_limit;  /* polls allowed to each bounded device wait of spi_factor and of the
+                        tensor-core variances of spi_diag_inverse: the waits of the tensor-core
+                        kernels for their copies and products (default 2^20) and the
                         dependency waits of the dependency-driven launch (default 2^25, about
                         100 ns apart): 0 = those defaults, > 0 = that many, < 0 = none, so every
-                        such wait gives up at once and spi_factor returns SPI_ERR_TIMEOUT (a
-                        test of that path).  After giving up, a tensor-core kernel still waits,
-                        with the default limit, for its own MMAs in flight before it frees its
-                        tensor memory; the dependency-driven launch skips its remaining tasks */
+                        such wait gives up at once and the call returns SPI_ERR_TIMEOUT (a
+                        test of that path; with force_schur = 1, dag = 1 and
+                        diag_tc_min_pivots < 0 nothing waits).  After giving up, a tensor-core
+                        kernel still waits, with the default limit, for its own copies and MMAs
+                        in flight before it frees its tensor memory; the dependency-driven
+                        launch skips its remaining tasks */
     int diag_ctas_per_sm;  /* 0 = the variance kernels of spi_diag_inverse take every SM
                         slot they fit in; k > 0: at most k of their CTAs per
                         SM (their shared memory is padded to enforce it), so that work on

@@ -1236,7 +1236,8 @@ void launch_diag(spi_ctx* c, const DevDiagPlan& p, int nb, int64_t nout, double*
                                 tc ? c->dtc.tc : nullptr, st);
         if (tc) launch_diag_inv_tc(c->dsym, p, c->dtc, c->d_D, out, nb, bs, c->d_status, c->opt.wait_limit, st);
     } else {
-        if (p.fx) launch_diag_fx(c->dsym, p, c->fx, c->ti, c->d_L, c->d_D, out, nb, bs, c->d_status, st);
+        if (p.fx) launch_diag_fx(c->dsym, p, c->fx, c->ti, c->d_L, c->d_D, out, nb, bs, c->d_status,
+                                 c->opt.wait_limit, st);
         else launch_diag_inverse(dev_sol(c), p, c->d_L, c->d_D, out, nb, bs, c->diag_smem_pad, st);
     }
 }

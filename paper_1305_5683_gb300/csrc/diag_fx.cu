@@ -206,6 +206,7 @@ struct FxArgs {
     const unsigned char* pack;
     const int32_t* rexp;
     const double *D, *fr;
+    uint32_t wait_limit;          // polls of each wait, then the kernel gives up
 };
 
 // Roles: warps 0-15 cut z into digits, read the products out of tensor memory and
@@ -232,9 +233,9 @@ __device__ __forceinline__ void fx_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(tc_smem_u32(bar)) : "memory");
 }
 // Bounded wait that also gives up when another role has.
-__device__ __forceinline__ bool fx_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
+__device__ __forceinline__ bool fx_wait(uint64_t* bar, uint32_t parity, volatile int* abort, uint32_t limit) {
     uint32_t done = 0;
-    for (uint32_t it = 0; it < kTcWaitLimit && !done; ++it) {
+    for (uint32_t it = 0; it < limit && !done; ++it) {
         asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
                      : "=r"(done) : "r"(tc_smem_u32(bar)), "r"(parity) : "memory");
         if (!done && *abort) return false;
@@ -330,7 +331,7 @@ __global__ void __launch_bounds__(kFxThreads, 1)
                     np += fx_tiles(x, g) * ((min(kFxRows, x.k - g * kFxRows) + kFxSub - 1) / kFxSub);
                 for (int t = 0; t < np && ok; ++t) {
                     const uint32_t st = a_issued % nst;
-                    if (a_issued >= (uint32_t)nst && !fx_wait(bar + kFAE + st, (a_issued / nst - 1) & 1u, abort)) {
+                    if (a_issued >= (uint32_t)nst && !fx_wait(bar + kFAE + st, (a_issued / nst - 1) & 1u, abort, p.wait_limit)) {
                         ok = false;
                         break;
                     }
@@ -357,11 +358,11 @@ __global__ void __launch_bounds__(kFxThreads, 1)
                 for (int g = 0; g < x.G && ok; ++g) {
                     const int w = min(kFxRows, x.k - g * kFxRows), nt = fx_tiles(x, g);
                     for (int i = 0; i < nt && ok; ++i) {
-                        if (tiles_issued > 0 && !fx_wait(bar + kFCE, (tiles_issued - 1) & 1u, abort)) { ok = false; break; }
-                        if (i < 2 && !fx_wait(bar + kFBF, bfull++ & 1u, abort)) { ok = false; break; }
+                        if (tiles_issued > 0 && !fx_wait(bar + kFCE, (tiles_issued - 1) & 1u, abort, p.wait_limit)) { ok = false; break; }
+                        if (i < 2 && !fx_wait(bar + kFBF, bfull++ & 1u, abort, p.wait_limit)) { ok = false; break; }
                         for (int sub = 0; sub * kFxSub < w; ++sub) {
                             const uint32_t st = piece % nst;
-                            if (!fx_wait(bar + kFAF + st, (piece / nst) & 1u, abort)) { ok = false; break; }
+                            if (!fx_wait(bar + kFAF + st, (piece / nst) & 1u, abort, p.wait_limit)) { ok = false; break; }
                             asm volatile("tcgen05.fence::after_thread_sync;");
                             const uint32_t ab = tc_smem_u32(Ar + st * kPiece);
 #pragma unroll
@@ -476,7 +477,7 @@ __global__ void __launch_bounds__(kFxThreads, 1)
                 cut(c0, w, false, true);
                 for (int i = 0; i < nt; ++i, ++tile) {
                     // a warp whose wait ran out does no further work but meets every barrier
-                    if (ok && !__all_sync(0xffffffffu, fx_wait(bar + kFCF, ndone & 1u, abort))) {
+                    if (ok && !__all_sync(0xffffffffu, fx_wait(bar + kFCF, ndone & 1u, abort, p.wait_limit))) {
                         ok = false;
                         *abort = 1;
                     }
@@ -591,14 +592,14 @@ void launch_tile_inverses(const DevSym& d, const DevTileInv& x, const double* L,
 }
 
 void launch_diag_fx(const DevSym& d, const DevDiagPlan& dp, const DevDiagFx& p, const DevTileInv& x, const double* L, const double* D,
-                    double* out, int nb, const Strides& bs, DevStatus* status, cudaStream_t st) {
+                    double* out, int nb, const Strides& bs, DevStatus* status, int wait_limit, cudaStream_t st) {
     if (dp.nblocks == 0 || nb == 0) return;
     k_fx_pack<<<dim3((unsigned)dp.fx_ntiles, nb), kFxRows, 0, st>>>(d, p.tiles, p.tdiag, dp.fx_tiles, p.ntiles, p.npieces,
                                                                     x.xoff, x.nx, L, D, x.xinv, p.pack, p.rexp, p.fr,
                                                                     bs.L, bs.n);
     FxArgs a{dp.B, dp.order_tc, dp.blk_ptr, dp.uptr, dp.us, dp.ulo, dp.uhi, dp.uzoff, dp.rel, dp.rhs_out,
              dp.rhs_zrow, dp.rhs_col, dp.urel, dp.zbase, dp.Z, p.pptr, p.tptr, p.npieces, p.ntiles, p.pack, p.rexp,
-             D, p.fr};
+             D, p.fr, wait_limit > 0 ? (uint32_t)wait_limit : wait_limit < 0 ? 0u : kTcWaitLimit};
     k_diag_fx<<<dim3(dp.nblocks, nb), kFxThreads, fx_smem(dp.B), st>>>(d, a, out, bs, status);
 }
 

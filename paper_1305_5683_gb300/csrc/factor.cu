@@ -1368,7 +1368,7 @@ constexpr size_t kSfSmem =
 template <int kMode>
 __global__ void __launch_bounds__(kSfThreads, 2) k_schur_fx(DevSym d, const int32_t* __restrict__ items, int step,
                                                             double* L, double* F22, const double* __restrict__ D,
-                                                            DevStatus* status, Strides bs) {
+                                                            DevStatus* status, Strides bs, uint32_t wait_limit) {
     L += blockIdx.y * bs.L;
     F22 += blockIdx.y * bs.F22;
     D += blockIdx.y * bs.n;
@@ -1504,7 +1504,7 @@ __global__ void __launch_bounds__(kSfThreads, 2) k_schur_fx(DevSym d, const int3
                     load_a(cg + cc + kFxTileK);
                     load_b(cg + cc + kFxTileK, jb);
                 }
-                ok = !__syncthreads_or(!tc_wait(bar, phase & 1u));
+                ok = !__syncthreads_or(!tc_wait(bar, phase & 1u, wait_limit));
                 if (ok) ++phase;
             }
             if (!ok) break;
@@ -1571,7 +1571,7 @@ __global__ void __launch_bounds__(kSfThreads, 2) k_schur_fx(DevSym d, const int3
         asm volatile("tcgen05.fence::after_thread_sync;");
     }
     if (!ok) {
-        tc_wait(bar, phase & 1u);  // drain before release
+        tc_wait(bar, phase & 1u);  // the products in flight, before tensor memory is released
         if (tid == 0) atomicOr(&status->flags, FLAG_TIMEOUT);
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
@@ -2008,6 +2008,7 @@ void launch_step_t(const DevSym& d, const Launch& l, const int32_t* items, C* L,
                    const double* adiag, DevStatus* status, int nb, const Strides& bs, int wait_limit,
                    cudaStream_t st) {
     const dim3 g(l.count, nb);
+    const uint32_t lim = wait_limit > 0 ? (uint32_t)wait_limit : wait_limit < 0 ? 0u : kTcWaitLimit;
     switch (l.kind) {
         case 0: k_diag_tile<C><<<g, kThreads, 0, st>>>(d, items + l.off, l.step, L, D, DS, adiag, status, bs); break;
         case 1: k_panel_trsm<C><<<g, kThreads, 0, st>>>(d, items + 2 * l.off, l.step, L, D, bs); break;
@@ -2016,8 +2017,7 @@ void launch_step_t(const DevSym& d, const Launch& l, const int32_t* items, C* L,
             break;
         case 7:
         case 9:
-            if constexpr (std::is_same<C, float>::value) {  // tensor-core items exist only in the mixed form
-                const uint32_t lim = wait_limit > 0 ? (uint32_t)wait_limit : wait_limit < 0 ? 0u : kTcWaitLimit;
+            if constexpr (std::is_same<C, float>::value) {  // these items exist only in the mixed form
                 if (l.kind == 7)
                     k_schur_tc<0><<<g, 128, kTcSmem, st>>>(d, items + 3 * l.off, 0, L, F22, DS, status, bs, lim);
                 else
@@ -2025,12 +2025,14 @@ void launch_step_t(const DevSym& d, const Launch& l, const int32_t* items, C* L,
             }
             break;
         case 17:
-            if constexpr (std::is_same<C, double>::value)  // the FP64 form's tensor-core items
-                k_schur_fx<0><<<g, kSfThreads, kSfSmem, st>>>(d, items + 4 * l.off, 0, L, F22, D, status, bs);
-            break;
         case 18:
-            if constexpr (std::is_same<C, double>::value)
-                k_schur_fx<1><<<g, kSfThreads, kSfSmem, st>>>(d, items + 4 * l.off, l.step, L, F22, D, status, bs);
+            if constexpr (std::is_same<C, double>::value) {  // the FP64 form's tensor-core items
+                if (l.kind == 17)
+                    k_schur_fx<0><<<g, kSfThreads, kSfSmem, st>>>(d, items + 4 * l.off, 0, L, F22, D, status, bs, lim);
+                else
+                    k_schur_fx<1><<<g, kSfThreads, kSfSmem, st>>>(d, items + 4 * l.off, l.step, L, F22, D, status, bs,
+                                                                  lim);
+            }
             break;
         case 8: k_diag_front<C><<<g, kThreads, 0, st>>>(d, items + l.off, L, D, DS, adiag, status, bs); break;
         case 12: {

@@ -322,7 +322,7 @@ size_t diag_fx_pack_bytes(int64_t npieces);
 // prepares the operands from the factor, then the variances of plan dp (dp.B
 // 16, 32 or 64)
 void launch_diag_fx(const DevSym& d, const DevDiagPlan& dp, const DevDiagFx& p, const DevTileInv& x, const double* L, const double* D,
-                    double* out, int nb, const Strides& bs, DevStatus* status, cudaStream_t st);
+                    double* out, int nb, const Strides& bs, DevStatus* status, int wait_limit, cudaStream_t st);
 
 // ---- normal.cu: N = H^T W H and b = H^T W y on the device
 struct NormalArgs {

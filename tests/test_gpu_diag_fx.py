@@ -137,3 +137,18 @@ def test_covariances_of_weakly_coupled_unknowns(P, weak):
     got = s.inverse_block(np.arange(n, dtype=np.int32))
     err = np.abs(got / ref.astype(float) - 1)
     assert err.max() <= 64 * n * EPS
+
+
+def test_wait_timeout_reported(P):
+    """wait_limit < 0: the kernel's first wait gives up; it drains its copies and products, frees
+    its tensor memory, and spi_diag_inverse returns SPI_ERR_TIMEOUT.  (The factorization waits
+    nowhere: SIMT Schur complements, launches level by level.)"""
+    pb = generate(scaled(SCALE, 700, seed=9))
+    s = P.Solver.for_problem(pb, wait_limit=-1, force_schur=1, dag=1)
+    s.factor(pb.values)
+    with pytest.raises(P.SpiError) as e:
+        s.diag_inverse()
+    assert e.value.code == 6
+    s = P.Solver.for_problem(pb)
+    s.factor(pb.values)
+    assert rel(s.diag_inverse(), oracle.OracleFactor.from_problem(pb).inv_diag()) <= 1e-10

@@ -190,8 +190,9 @@ def test_bounded_wait_timeout_reported(P):
     with pytest.raises(P.SpiError) as e:
         s.solve(b)
     assert e.value.code == 7
-    # launched level by level, the FP64 form waits nowhere: the same option leaves it untouched
-    s64 = P.Solver(n, cp, ri, ordering=P.SPI_ORDER_NATURAL, wait_limit=-1, dag=1)
+    # launched level by level without tensor-core Schur complements, the FP64 form waits nowhere:
+    # the same option leaves it untouched
+    s64 = P.Solver(n, cp, ri, ordering=P.SPI_ORDER_NATURAL, wait_limit=-1, dag=1, force_schur=1)
     s64.factor(va)
     x_ref = oracle.OracleFactor(n, cp, ri, va).solve(b)
     assert np.abs(s64.solve(b) - x_ref).max() <= 1e-10 * np.abs(x_ref).max()

@@ -76,3 +76,23 @@ def test_badly_scaled_columns(P):
     s.factor(pb.values * t[pb.rowind] * t[col])
     x = s.solve(pb.b * t) * t
     assert np.abs(x - ref).max() <= 64 * pb.n * EPS * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("kind", ["schur", "panel"])
+def test_wait_timeout_reported(P, kind):
+    """wait_limit < 0: the first wait for the products gives up; the kernel drains them, frees its
+    tensor memory and spi_factor returns SPI_ERR_TIMEOUT; a new context on the device works.
+    Without tensor-core launches nothing waits."""
+    pb = two_leaves(32, 128, 5) if kind == "schur" else random_spd(300, 1.0, 3, dominance=300.0)
+    s = P.Solver.for_problem(pb, dag=1, force_panel=1, wait_limit=-1)
+    with pytest.raises(P.SpiError) as e:
+        s.factor(pb.values)
+    assert e.value.code == 6
+    with pytest.raises(P.SpiError) as e:
+        s.solve(pb.b)
+    assert e.value.code == 7
+    ref = oracle.OracleFactor.from_problem(pb).solve(pb.b)
+    for kw in (dict(force_schur=1, wait_limit=-1), dict()):
+        s = P.Solver.for_problem(pb, dag=1, force_panel=1, **kw)
+        s.factor(pb.values)
+        assert np.abs(s.solve(pb.b) - ref).max() <= 64 * pb.n * EPS * np.abs(ref).max()
