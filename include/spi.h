@@ -95,7 +95,9 @@ typedef struct spi_options {
                         slot they fit in; k > 0: at most k of their CTAs per
                         SM (their shared memory is padded to enforce it), so that work on
                         another stream -- a spi_solve running concurrently -- keeps room
-                        on every SM instead of waiting for variance CTAs to finish */
+                        on every SM instead of waiting for variance CTAs to finish.  FP64
+                        form: k > 0 takes the SIMT kernel, since a CTA of the tensor-core
+                        kernel has an SM to itself */
     int diag_unpruned;   /* 0 = pruned solves (the method); 1 = the pruning ablation: every
                             variance from a full forward solve over all supernodes (32 per
                             pass, FP64 panels), var_i = sum_k z_k^2 / d_k, so that the gain

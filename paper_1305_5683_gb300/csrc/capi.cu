@@ -346,6 +346,7 @@ int ensure_fx(spi_ctx* c) {
     if (c->fx_state >= 0) return SPI_OK;
     c->fx_state = 0;
     if (!c->ti.xinv || c->opt.diag_tc_min_pivots < 0 || c->S.n == 0) return SPI_OK;
+    if (c->opt.diag_ctas_per_sm > 0) return SPI_OK;  // a CTA of k_diag_fx takes an SM to itself
     const DiagFxHost& h = c->fx_h;
     DevDiagFx& t = c->fx;
     t = DevDiagFx();

@@ -152,3 +152,17 @@ def test_wait_timeout_reported(P):
     s = P.Solver.for_problem(pb)
     s.factor(pb.values)
     assert rel(s.diag_inverse(), oracle.OracleFactor.from_problem(pb).inv_diag()) <= 1e-10
+
+
+def test_room_for_another_stream(P):
+    """diag_ctas_per_sm keeps its promise: the variances then come from the SIMT kernel, whose CTAs
+    leave room on every SM (the tensor-core kernel's take one each)."""
+    pb = generate(scaled(SCALE, 700, seed=9))
+    v = []
+    for more in (dict(diag_ctas_per_sm=3), dict(diag_ctas_per_sm=3, diag_tc_min_pivots=-1)):
+        s = P.Solver.for_problem(pb, rhs_block=32, **more)
+        s.factor(pb.values)
+        v.append(s.diag_inverse())
+        assert s.info()["launches_diag"] == 1
+    # the same kernel on two factorizations (whose atomics may add in another order)
+    assert rel(v[0], v[1]) <= 1e-13
