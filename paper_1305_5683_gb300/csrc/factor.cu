@@ -461,12 +461,13 @@ __device__ __forceinline__ T ldx(const T* p) {
 
 // 1/d in FP64 with three FP64 operations on the dependency chain (a dependent FP64
 // operation costs about 64 cycles on this GPU, a division 350): the hardware's
-// approximation r0 (within 2^-19.9), refined by one step of the third-order reciprocal
-// iteration (the Newton-Raphson iteration carried one term further: 1/d = r0 / (1 - e) =
+// approximation r0 (within 2^-19.9), refined by one step of the hyperpower iteration of third
+// order (M. Altman, Pacific J. Math. 10, 1960, for inverses in general: 1/d = r0 / (1 - e) =
 // r0 (1 + e + e^2 + ...), e = 1 - d r0), r0 (1 + e + e^2): the dropped e^3 term is below
 // FP64 rounding and the result within 1 ulp of the correctly rounded 1/d (268 million
-// values over the whole exponent range).  Zero,
-// subnormal, huge or non-finite d divide.
+// values over the whole exponent range; a few thousand in tests/test_gpu_pivot_tile.py).  Zero,
+// subnormal, huge or non-finite d divide.  Used where it shortens a chain and where it always
+// was; the panel solves of whole fronts and of the dependency-driven launch divide.
 __device__ __forceinline__ double recip_fp64(double d) {
     const int ex = (__double2hiint(d) >> 20) & 0x7ff;
     if (ex < 4 || ex > 2042) return 1.0 / d;
@@ -787,7 +788,7 @@ __device__ void front_panel_body(const DevSym& d, int s, C* Lb, double* Db, C* D
             if constexpr (std::is_same<C, float>::value) sm.trsm.Bt[j][i] = v;
             else sm.trsm.Bd[i][j] = v;
         }
-        if (tid < kT) sm.trsm.rd[tid] = tid < w ? (C)recip_fp64(ldx<kCg>(Db + f + c0 + tid)) : C(0);
+        if (tid < kT) sm.trsm.rd[tid] = tid < w ? (C)(1.0 / ldx<kCg>(Db + f + c0 + tid)) : C(0);
         __syncthreads();
         if constexpr (std::is_same<C, float>::value) {
             for (int64_t r = c0 + w + tid; r < m; r += kThreads) panel_row1<kCg>(P, m, c0, w, r, sm.trsm.Bt, sm.trsm.rd);
@@ -1632,7 +1633,7 @@ __device__ void dag_trsm(const DevSym& d, int s, int b, int chunk, C* Lb, const 
         const int i = e % kT, j = e / kT;
         sm.trsm.Bd[i][j] = (i < w && j < i) ? __ldcg(P + (c0 + i) + (int64_t)(c0 + j) * m) : C(0);
     }
-    if (tid < kT) sm.trsm.rd[tid] = tid < w ? (C)recip_fp64(__ldcg(Db + f + c0 + tid)) : C(0);
+    if (tid < kT) sm.trsm.rd[tid] = tid < w ? (C)(1.0 / __ldcg(Db + f + c0 + tid)) : C(0);
     __syncthreads();
     const int64_t r0 = c0 + w + (int64_t)chunk * kT;
     panel_rows4<true, C>(P, m, c0, w, r0, (int)(m - r0 < kT ? m - r0 : kT), sm.trsm.Bd, sm.trsm.rd);
