@@ -172,11 +172,52 @@ constexpr int kMaxRestarts = 256;
 const Symbolic& sym_sol(const spi_ctx* c) { return c->piv_ready ? c->S_sol : c->S; }
 const DevSym& dev_sol(const spi_ctx* c) { return c->piv_ready ? c->dsym_sol : c->dsym; }
 
+// The FP64 form's optional operands: the packed pieces of the variances (fx) and the inverted
+// diagonal tiles (ti).  Everything works without them, on the kernels that were there before.
+void free_fx(spi_ctx* c) {
+    for (void* a : c->fx.allocs) cudaFree(a);
+    c->device_bytes -= c->fx.bytes;
+    c->fx = DevDiagFx();
+}
+void free_ti(spi_ctx* c) {
+    for (auto* g : {&c->g_factor, &c->g_solve}) {  // the graphs hold the tiles' addresses
+        for (auto& kv : *g) cudaGraphExecDestroy(kv.second);
+        g->clear();
+    }
+    for (void* a : c->ti.allocs) cudaFree(a);
+    c->device_bytes -= c->ti.bytes;
+    c->ti = DevTileInv();
+    c->wide_ready = false;
+}
+// One of them given up for memory that another buffer needs; false if there is none left.
+bool release_optional(spi_ctx* c) {
+    if (c->fx.allocs.empty() && c->ti.allocs.empty()) return false;
+    cudaDeviceSynchronize();  // an asynchronous call may still be using it
+    if (!c->fx.allocs.empty()) {
+        free_fx(c);
+        c->fx_state = 0;
+    } else {
+        free_ti(c);
+    }
+    return true;
+}
+// cudaMalloc that gives up the optional operands before it fails (release).
+cudaError_t device_malloc(spi_ctx* c, void** p, size_t bytes, bool release = true) {
+    for (;;) {
+        const cudaError_t e = cudaMalloc(p, bytes);
+        if (e == cudaSuccess) return e;
+        *p = nullptr;
+        if (e != cudaErrorMemoryAllocation) return e;
+        cudaGetLastError();
+        if (!release || !release_optional(c)) return e;
+    }
+}
+
 template <class T>
-cudaError_t dev_alloc(spi_ctx* c, T** p, size_t count, std::vector<void*>* track = nullptr) {
+cudaError_t dev_alloc(spi_ctx* c, T** p, size_t count, std::vector<void*>* track = nullptr, bool release = true) {
     *p = nullptr;
     if (count == 0) count = 1;
-    cudaError_t e = cudaMalloc((void**)p, count * sizeof(T));
+    cudaError_t e = device_malloc(c, (void**)p, count * sizeof(T), release);
     if (e == cudaSuccess) {
         (track ? *track : c->allocs).push_back(*p);
         c->device_bytes += (int64_t)(count * sizeof(T));
@@ -185,8 +226,9 @@ cudaError_t dev_alloc(spi_ctx* c, T** p, size_t count, std::vector<void*>* track
 }
 
 template <class T>
-cudaError_t dev_upload(spi_ctx* c, T** p, const std::vector<T>& v, std::vector<void*>* track = nullptr) {
-    cudaError_t e = dev_alloc(c, p, v.size(), track);
+cudaError_t dev_upload(spi_ctx* c, T** p, const std::vector<T>& v, std::vector<void*>* track = nullptr,
+                       bool release = true) {
+    cudaError_t e = dev_alloc(c, p, v.size(), track, release);
     if (e == cudaSuccess && !v.empty()) e = cudaMemcpy(*p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
     return e;
 }
@@ -304,7 +346,7 @@ int ensure_device(spi_ctx* c) {
             t.ntc = h.ntc;
             t.npt = h.npt;
             t.ndt = h.ndt;
-                    t.bands = (int)nb;
+            t.bands = (int)nb;
             build_solve_plan(S, c->SPw, c->opt.batch, h.tc.data());
             CK(dev_upload(c, &c->d_fwd_items_w, c->SPw.fwd_items));
             CK(dev_upload(c, &c->d_bwd_items_w, c->SPw.bwd_items));
@@ -317,27 +359,32 @@ int ensure_device(spi_ctx* c) {
         const DiagFxHost& h = c->fx_h;
         DevTileInv& t = c->ti;
         t = DevTileInv();
-        CK(dev_upload(c, &t.dtiles, h.dtiles));
-        CK(dev_upload(c, &t.xoff, h.xoff));
-        CK(dev_upload(c, &t.xptr, h.xptr));
-        CK(dev_alloc(c, &t.xinv, (size_t)h.nx * nb));
-        CK(dev_alloc(c, &t.xinvt, (size_t)h.nx * nb));
-        t.ncta = (int64_t)h.dtiles.size() / 4;
-        t.nx = h.nx;
-        const std::vector<uint8_t> every((size_t)S.ns, 1);
-        build_solve_plan(S, c->SPw, c->opt.batch, every.data(), true);
-        CK(dev_upload(c, &c->d_fwd_items_w, c->SPw.fwd_items));
-        CK(dev_upload(c, &c->d_bwd_items_w, c->SPw.bwd_items));
-        c->wa = WideArgs{nullptr, t.xptr, 0, t.xinv, t.xinvt, t.xoff, t.nx};
-        c->wide_ready = true;
+        const int64_t before = c->device_bytes;
+        std::vector<void*>* tr = &t.allocs;
+        cudaError_t e = dev_upload(c, &t.dtiles, h.dtiles, tr, false);
+        if (e == cudaSuccess) e = dev_upload(c, &t.xoff, h.xoff, tr, false);
+        if (e == cudaSuccess) e = dev_upload(c, &t.xptr, h.xptr, tr, false);
+        if (e == cudaSuccess) e = dev_alloc(c, &t.xinv, (size_t)h.nx * nb, tr, false);
+        if (e == cudaSuccess) e = dev_alloc(c, &t.xinvt, (size_t)h.nx * nb, tr, false);
+        if (e == cudaSuccess) {
+            const std::vector<uint8_t> every((size_t)S.ns, 1);
+            build_solve_plan(S, c->SPw, c->opt.batch, every.data(), true);
+            e = dev_upload(c, &c->d_fwd_items_w, c->SPw.fwd_items, tr, false);
+            if (e == cudaSuccess) e = dev_upload(c, &c->d_bwd_items_w, c->SPw.bwd_items, tr, false);
+        }
+        t.bytes = c->device_bytes - before;
+        if (e == cudaErrorMemoryAllocation) {
+            free_ti(c);  // 32-column solve steps and SIMT variances
+        } else {
+            CK(e);
+            t.ncta = (int64_t)h.dtiles.size() / 4;
+            t.nx = h.nx;
+            c->wa = WideArgs{nullptr, t.xptr, 0, t.xinv, t.xinvt, t.xoff, t.nx};
+            c->wide_ready = true;
+        }
     }
     c->dev_ready = true;
     return SPI_OK;
-}
-
-void free_fx(DevDiagFx& t) {
-    for (void* a : t.allocs) cudaFree(a);
-    t = DevDiagFx();
 }
 
 // Buffers of the FP64 form's tensor-core variances (operands are prepared from the factor
@@ -353,21 +400,16 @@ int ensure_fx(spi_ctx* c) {
     const size_t nb = (size_t)c->opt.batch, n = (size_t)c->S.n;
     const int64_t before = c->device_bytes;
     std::vector<void*>* tr = &t.allocs;
-    auto alloc = [&]() -> cudaError_t {
-        cudaError_t e = dev_upload(c, &t.pptr, h.pptr, tr);
-        if (e == cudaSuccess) e = dev_upload(c, &t.tptr, h.tptr, tr);
-        if (e == cudaSuccess) e = dev_upload(c, &t.tiles, h.tiles, tr);
-        if (e == cudaSuccess) e = dev_upload(c, &t.tdiag, h.tdiag, tr);
-        if (e == cudaSuccess) e = dev_alloc(c, &t.pack, diag_fx_pack_bytes(h.npieces) * nb, tr);
-        if (e == cudaSuccess) e = dev_alloc(c, &t.rexp, (size_t)h.ntiles * kFxRows * nb, tr);
-        if (e == cudaSuccess) e = dev_alloc(c, &t.fr, n * nb, tr);
-        return e;
-    };
-    const cudaError_t e = alloc();
+    cudaError_t e = dev_upload(c, &t.pptr, h.pptr, tr, false);
+    if (e == cudaSuccess) e = dev_upload(c, &t.tptr, h.tptr, tr, false);
+    if (e == cudaSuccess) e = dev_upload(c, &t.tiles, h.tiles, tr, false);
+    if (e == cudaSuccess) e = dev_upload(c, &t.tdiag, h.tdiag, tr, false);
+    if (e == cudaSuccess) e = dev_alloc(c, &t.pack, diag_fx_pack_bytes(h.npieces) * nb, tr, false);
+    if (e == cudaSuccess) e = dev_alloc(c, &t.rexp, (size_t)h.ntiles * kFxRows * nb, tr, false);
+    if (e == cudaSuccess) e = dev_alloc(c, &t.fr, n * nb, tr, false);
+    t.bytes = c->device_bytes - before;
     if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        free_fx(t);
-        c->device_bytes = before;
+        free_fx(c);
         return SPI_OK;
     }
     CK(e);
@@ -415,6 +457,7 @@ int upload_plan(spi_ctx* c, const DiagPlan& h, DevDiagPlan& d) {
     }
     // FP64 elements per band are enough for both element types
     CK(dev_alloc(c, &d.Z, (size_t)std::max<int64_t>(d.zsize, 1) * (size_t)c->opt.batch, tr));
+    d.fx = d.fx && c->fx_state == 1;  // (its operands may have been given up for Z)
     return SPI_OK;
 }
 
@@ -845,8 +888,9 @@ void reset_device(spi_ctx* c) {
     free_plan(c->plan_all);
     free_plan(c->plan_sub);
     free_plan(c->plan_blk);
-    free_fx(c->fx);
+    free_fx(c);
     c->fx_state = -1;
+    free_ti(c);
     free_factor_plan(c->dfp);
     c->plan_all_ready = c->plan_sub_ready = c->plan_blk_ready = false;
     for (auto* g : {&c->g_factor, &c->g_solve, &c->g_solve_dag}) {
@@ -868,7 +912,6 @@ void reset_device(spi_ctx* c) {
     c->bg = spi_ctx::Background();
     c->nrm = spi_ctx::Normal();
     c->dtc = DevDiagTc();
-    c->ti = DevTileInv();
     c->wide_ready = false;
     c->dev_ready = false;
     c->factor_plan_ready = false;
@@ -1237,7 +1280,7 @@ void launch_diag(spi_ctx* c, const DevDiagPlan& p, int nb, int64_t nout, double*
                                 tc ? c->dtc.tc : nullptr, st);
         if (tc) launch_diag_inv_tc(c->dsym, p, c->dtc, c->d_D, out, nb, bs, c->d_status, c->opt.wait_limit, st);
     } else {
-        if (p.fx) launch_diag_fx(c->dsym, p, c->fx, c->ti, c->d_L, c->d_D, out, nb, bs, c->d_status,
+        if (p.fx && c->fx_state == 1) launch_diag_fx(c->dsym, p, c->fx, c->ti, c->d_L, c->d_D, out, nb, bs, c->d_status,
                                  c->opt.wait_limit, st);
         else launch_diag_inverse(dev_sol(c), p, c->d_L, c->d_D, out, nb, bs, c->diag_smem_pad, st);
     }
@@ -1339,7 +1382,7 @@ int diag_unpruned_impl(spi_ctx* c, const int32_t* idx, int64_t nidx, double* out
     const size_t vec = (size_t)std::min<int64_t>(kR, nidx) * (size_t)n;
     double* buf = nullptr;
     const size_t bytes = (2 * vec + (size_t)n + (size_t)nidx) * sizeof(double) + (size_t)kR * sizeof(int32_t);
-    if (cudaMalloc(&buf, bytes) != cudaSuccess) {
+    if (device_malloc(c, (void**)&buf, bytes) != cudaSuccess) {
         cudaGetLastError();
         return SPI_ERR_OOM;
     }
@@ -1726,7 +1769,7 @@ int inverse_block_impl(spi_ctx* c, std::vector<int32_t>& key, double* od, cudaSt
         c->blk_rows = (int64_t)zpiv.size();
         if (c->blk_rows * nidx > c->zg_cap) {
             if (c->d_zg) { cudaFree(c->d_zg); c->d_zg = nullptr; c->zg_cap = 0; }
-            if (cudaMalloc(&c->d_zg, (size_t)c->blk_rows * (size_t)nidx * sizeof(double)) != cudaSuccess) {
+            if (device_malloc(c, (void**)&c->d_zg, (size_t)c->blk_rows * (size_t)nidx * sizeof(double)) != cudaSuccess) {
                 cudaGetLastError();
                 c->d_zg = nullptr;
                 return SPI_ERR_OOM;
@@ -1799,7 +1842,7 @@ int spi_diag_inverse_refined(spi_ctx* c, const int32_t* idx, int64_t nidx, doubl
     // w, z, xp (pivot order), x (caller order), r; then pivots, indices and outputs of a pass
     double* buf = nullptr;
     const size_t bytes = 5 * vec * sizeof(double) + 2 * (size_t)kR * sizeof(int32_t) + (size_t)nidx * sizeof(double);
-    if (cudaMalloc(&buf, bytes) != cudaSuccess) {
+    if (device_malloc(c, (void**)&buf, bytes) != cudaSuccess) {
         cudaGetLastError();
         return SPI_ERR_OOM;
     }
@@ -1891,7 +1934,7 @@ int spi_inverse_entries(spi_ctx* c, const int32_t* rows, const int32_t* cols, in
     double* od = out;
     double* staged = nullptr;
     if (!on_device) {
-        if (cudaMalloc(&staged, (size_t)nent * sizeof(double)) != cudaSuccess) {
+        if (device_malloc(c, (void**)&staged, (size_t)nent * sizeof(double)) != cudaSuccess) {
             cudaGetLastError();
             return SPI_ERR_OOM;
         }
@@ -1921,7 +1964,7 @@ int spi_inverse_entries(spi_ctx* c, const int32_t* rows, const int32_t* cols, in
     bptr.push_back(e);
     int64_t* d_idx = nullptr;
     int rc = SPI_OK;
-    if (cudaMalloc(&d_idx, 2 * (size_t)nent * sizeof(int64_t)) != cudaSuccess) {
+    if (device_malloc(c, (void**)&d_idx, 2 * (size_t)nent * sizeof(int64_t)) != cudaSuccess) {
         cudaGetLastError();
         if (staged) cudaFree(staged);
         return SPI_ERR_OOM;
@@ -2618,7 +2661,8 @@ void spi_destroy(spi_ctx* c) {
     free_plan(c->plan_all);
     free_plan(c->plan_sub);
     free_plan(c->plan_blk);
-    free_fx(c->fx);
+    free_fx(c);
+    free_ti(c);
     free_factor_plan(c->dfp);
     if (c->d_zg) cudaFree(c->d_zg);
     for (auto& kv : c->g_factor) cudaGraphExecDestroy(kv.second);

@@ -305,6 +305,8 @@ struct DevTileInv {
     int64_t* xoff = nullptr;         // [tiles]
     double* xinv = nullptr;          // [bands][nx]
     double* xinvt = nullptr;         // [bands][nx] their transposes
+    std::vector<void*> allocs;       // (none: not in use)
+    int64_t bytes = 0;
 };
 void launch_tile_inverses(const DevSym& d, const DevTileInv& x, const double* L, int nb, const Strides& bs,
                           cudaStream_t st);
@@ -316,6 +318,7 @@ struct DevDiagFx {
     int32_t* rexp = nullptr;        // [bands][ntiles][128] row exponents
     double* fr = nullptr;           // [bands][n] s^2 / d, s the power of two next to sqrt(d)
     std::vector<void*> allocs;
+    int64_t bytes = 0;
 };
 cudaError_t diag_fx_setup();
 size_t diag_fx_pack_bytes(int64_t npieces);
