@@ -387,6 +387,9 @@ int ensure_device(spi_ctx* c) {
     return SPI_OK;
 }
 
+// Right-hand sides per block that k_diag_fx takes.
+bool fx_takes(int block) { return block == 16 || block == 32 || block == kFxMaxBlock; }
+
 // Buffers of the FP64 form's tensor-core variances (operands are prepared from the factor
 // by every call).  Without the memory for them the SIMT kernel serves alone.
 int ensure_fx(spi_ctx* c) {
@@ -394,6 +397,7 @@ int ensure_fx(spi_ctx* c) {
     c->fx_state = 0;
     if (!c->ti.xinv || c->opt.diag_tc_min_pivots < 0 || c->S.n == 0) return SPI_OK;
     if (c->opt.diag_ctas_per_sm > 0) return SPI_OK;  // a CTA of k_diag_fx takes an SM to itself
+    if (c->opt.rhs_block > 0 && !fx_takes(c->opt.rhs_block)) return SPI_OK;
     const DiagFxHost& h = c->fx_h;
     DevDiagFx& t = c->fx;
     t = DevDiagFx();
@@ -448,7 +452,7 @@ int upload_plan(spi_ctx* c, const DiagPlan& h, DevDiagPlan& d) {
     CK(dev_upload(c, &d.urel, h.urel, tr));
     CK(dev_upload(c, &d.zbase, h.zbase, tr));
     d.zsize = h.zbase.empty() ? 0 : h.zbase.back();
-    d.fx = c->fx_state == 1 && (h.B == 16 || h.B == 32 || h.B == kFxMaxBlock);
+    d.fx = c->fx_state == 1 && fx_takes(h.B);
     if (d.fx) {
         std::vector<int32_t> tiles;
         diag_fx_used(c->S, c->fx_h, h, tiles);

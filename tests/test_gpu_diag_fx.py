@@ -166,3 +166,18 @@ def test_room_for_another_stream(P):
         assert s.info()["launches_diag"] == 1
     # the same kernel on two factorizations (whose atomics may add in another order)
     assert rel(v[0], v[1]) <= 1e-13
+
+
+@pytest.mark.parametrize("block", [8, 48, 128])
+def test_other_block_sizes_hold_no_packed_operands(P, block):
+    """Blocks the tensor-core kernel does not take: one SIMT launch and no more device memory than
+    with the kernel switched off."""
+    pb = generate(scaled(SCALE, 300, seed=2))
+    held = []
+    for more in ({}, {"diag_tc_min_pivots": -1}):
+        s = P.Solver.for_problem(pb, rhs_block=block, **more)
+        s.factor(pb.values)
+        s.diag_inverse()
+        held.append(s.info()["device_bytes"])
+        assert s.info()["launches_diag"] == 1
+    assert held[0] == held[1]
