@@ -132,10 +132,11 @@ typedef struct spi_options {
                         depends on; spi_solve runs both sweeps so (forward steps, backward passes
                         over 32 columns, backward steps) */
     const char* tune_cache; /* path of a text file keeping the autotuner's choices across
-                        processes (one line per device, precision, batch class and bucket, plus
-                        one line each for the factor's and the solve's form and for the
-                        variance right-hand-side block), or NULL; each choice is read before it
-                        would be timed and the file rewritten after a timing */
+                        processes (one line per device, precision, batch class, revision of the
+                        kernels and bucket, plus, per size class of the problem, one line each
+                        for the factor's and the solve's form and for the variance
+                        right-hand-side block), or NULL; each choice is read before it would be
+                        timed and the file rewritten after a timing, other lines kept */
     int pivoting;    /* 0 = symmetric positive definite (the pivot-free LDL^T; a non-positive pivot
                         is SPI_ERR_NOT_SPD).  1 = symmetric indefinite (paper Sec. 5): every front
                         factored with restricted Bunch-Kaufman pivoting -- 1x1 and 2x2 pivots

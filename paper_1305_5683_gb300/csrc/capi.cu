@@ -598,11 +598,15 @@ void factor_launches(spi_ctx* c, int nb, const FactorPlan& F, const spi_ctx::Dev
 // nodes), replayed twice on the caller's values, and the second replay's
 // group times are summed per bucket; every bucket keeps its faster candidate.
 // The table can be kept in a text file (spi_options.tune_cache), one line
-// per bucket: device, precision, batch class, P (panel) or S (Schur), bucket,
-// choice, milliseconds of the two candidates.  The same file keeps the other
-// timed choices, one line each: D (one dependency-driven factor launch or
-// launches level by level), V (the same for the solve) and B (the variance
-// right-hand-side block).
+// per bucket: device, precision, batch class with the revision of the kernels, P (panel) or S
+// (Schur), bucket, choice, milliseconds of the two candidates.  The same file keeps the other
+// timed choices, one line each per size class of the problem (in the bucket's place): D (one
+// dependency-driven factor launch or launches level by level), V (the same for the solve) and B
+// (the variance right-hand-side block).
+
+// Counts up whenever a change of the kernels may change which candidate is faster, so that a
+// file's older choices are timed again (revision 1 wrote no number).
+constexpr int kTuneRevision = 2;
 
 std::string tune_key(spi_ctx* c, int nb) {
     cudaDeviceProp prop;
@@ -610,8 +614,14 @@ std::string tune_key(spi_ctx* c, int nb) {
     if (cudaGetDeviceProperties(&prop, c->device) == cudaSuccess) dev = prop.name;
     for (char& ch : dev)
         if (ch == ' ' || ch == '\t') ch = '_';
-    return dev + " " + (mixed_of(c) ? "mixed" : "fp64") + " " + (nb > 1 ? "batch" : "single");
+    return dev + " " + (mixed_of(c) ? "mixed" : "fp64") + " " + (nb > 1 ? "batch" : "single") + "." +
+           std::to_string(kTuneRevision);
 }
+
+// The size class of the choices made for a whole problem: which form is faster turns with the
+// size (the dependency-driven factorization wins up to a few thousand pointings and takes twice
+// the time at P = 20,000).
+int32_t tune_size(const spi_ctx* c) { return (int32_t)std::floor(std::log2(std::max(1.0, c->S.factor_flops))); }
 
 // The buckets whose choice matters for this tree: panel buckets of fronts that
 // may run either way, Schur buckets of fronts that may use the tensor cores.
@@ -666,9 +676,9 @@ void write_tune_cache(const char* path, const std::string& key, const std::vecto
     const std::string tmp = std::string(path) + ".tmp";
     FILE* fp = std::fopen(tmp.c_str(), "w");
     if (!fp) return;
-    std::fprintf(fp, "# spi autotuner: device precision batch kind bucket choice ms_candidate0 ms_candidate1"
-                     " (P panel, S Schur, D dependency-driven factor, V dependency-driven solve, B variance"
-                     " right-hand-side block)\n");
+    std::fprintf(fp, "# spi autotuner: device precision batch.revision kind bucket choice ms_candidate0 ms_candidate1"
+                     " (P panel, S Schur; by size class: D dependency-driven factor, V dependency-driven solve,"
+                     " B variance right-hand-side block)\n");
     for (const std::string& l : other) std::fputs(l.c_str(), fp);
     for (const TuneLine& t : lines)
         std::fprintf(fp, "%s %c %d %d %.6f %.6f\n", key.c_str(), t.kind, t.bucket, t.choice, t.ms0, t.ms1);
@@ -676,14 +686,15 @@ void write_tune_cache(const char* path, const std::string& key, const std::vecto
     std::rename(tmp.c_str(), path);
 }
 
-// Replace this key's lines of the given kinds by `fresh`, keeping every other line.
-void tune_cache_update(const char* path, const std::string& key, const char* kinds,
-                       const std::vector<TuneLine>& fresh) {
+// Replace this key's lines of the same kinds and buckets by `fresh`, keeping every other line.
+void tune_cache_update(const char* path, const std::string& key, const std::vector<TuneLine>& fresh) {
     if (!path) return;
     std::vector<TuneLine> cached, keep;
     read_tune_cache(path, key, cached, nullptr);
     for (const TuneLine& t : cached)
-        if (!std::strchr(kinds, t.kind)) keep.push_back(t);
+        if (std::none_of(fresh.begin(), fresh.end(),
+                         [&](const TuneLine& f) { return f.kind == t.kind && f.bucket == t.bucket; }))
+            keep.push_back(t);
     keep.insert(keep.end(), fresh.begin(), fresh.end());
     write_tune_cache(path, key, keep);
 }
@@ -796,7 +807,8 @@ int prepare_factor_plan(spi_ctx* c, int nb, const double* vals, cudaStream_t st)
         const std::string key = tune_key(c, nb);
         std::vector<TuneLine> cached;
         read_tune_cache(c->opt.tune_cache, key, cached, nullptr);
-        for (const TuneLine& t : cached) (t.kind == 'P' ? ch.panel : ch.schur)[t.bucket] = (uint8_t)(t.choice != 0);
+        for (const TuneLine& t : cached)
+            if (t.kind == 'P' || t.kind == 'S') (t.kind == 'P' ? ch.panel : ch.schur)[t.bucket] = (uint8_t)(t.choice != 0);
         bool missing = false;
         for (int32_t b : pb) missing |= !ch.panel.count(b);
         for (int32_t b : sb) missing |= !ch.schur.count(b);
@@ -826,7 +838,7 @@ int prepare_factor_plan(spi_ctx* c, int nb, const double* vals, cudaStream_t st)
                 ch.schur[bk] = (uint8_t)(t1 < t0a);
                 lines.push_back(TuneLine{'S', bk, t1 < t0a ? 1 : 0, t0a, t1});
             }
-            tune_cache_update(c->opt.tune_cache, key, "PS", lines);
+            tune_cache_update(c->opt.tune_cache, key, lines);
             c->tune_source = 1;
             c->tune_seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
         }
@@ -853,7 +865,7 @@ int prepare_factor_plan(spi_ctx* c, int nb, const double* vals, cudaStream_t st)
         read_tune_cache(c->opt.tune_cache, key, cached, nullptr);
         int found = -1;
         for (const TuneLine& t : cached)
-            if (t.kind == 'D') found = t.choice;
+            if (t.kind == 'D' && t.bucket == tune_size(c)) found = t.choice;
         const bool timing = c->opt.autotune > 0 || (c->opt.autotune == 0 && S.factor_flops >= 2e8);
         if (found >= 0) {
             ch.dag = found;
@@ -868,8 +880,8 @@ int prepare_factor_plan(spi_ctx* c, int nb, const double* vals, cudaStream_t st)
             c->tune_dag_ms[0] = time_whole_plan(c, nb, vals, F0, st);
             c->tune_dag_ms[1] = F1.dag.empty() ? -1.0 : time_whole_plan(c, nb, vals, F1, st);
             ch.dag = c->tune_dag_ms[1] >= 0.0 && c->tune_dag_ms[0] >= 0.0 && c->tune_dag_ms[1] < c->tune_dag_ms[0];
-            tune_cache_update(c->opt.tune_cache, key, "D",
-                              {TuneLine{'D', 0, ch.dag, c->tune_dag_ms[0], c->tune_dag_ms[1]}});
+            tune_cache_update(c->opt.tune_cache, key,
+                              {TuneLine{'D', tune_size(c), ch.dag, c->tune_dag_ms[0], c->tune_dag_ms[1]}});
             c->tune_source = 1;
             c->tune_seconds += std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
         } else {
@@ -1173,7 +1185,7 @@ int choose_solve_form(spi_ctx* c, int nb, const double* bd, cudaStream_t st) {
         std::vector<TuneLine> cached;
         read_tune_cache(c->opt.tune_cache, key, cached, nullptr);
         for (const TuneLine& t : cached)
-            if (t.kind == 'V') c->solve_dag = t.choice != 0 && !c->SP.dag.empty();
+            if (t.kind == 'V' && t.bucket == tune_size(c)) c->solve_dag = t.choice != 0 && !c->SP.dag.empty();
         if (c->solve_dag >= 0) return SPI_OK;
     }
     const bool timing = c->opt.autotune > 0 || (c->opt.autotune == 0 && c->S.factor_flops >= 2e8);
@@ -1203,8 +1215,8 @@ int choose_solve_form(spi_ctx* c, int nb, const double* bd, cudaStream_t st) {
     cudaEventDestroy(e1);
     if (rc) return rc;
     c->solve_dag = c->tune_solve_ms[1] >= 0 && c->tune_solve_ms[1] < c->tune_solve_ms[0] ? 1 : 0;
-    tune_cache_update(c->opt.tune_cache, key, "V",
-                      {TuneLine{'V', 0, c->solve_dag, c->tune_solve_ms[0], c->tune_solve_ms[1]}});
+    tune_cache_update(c->opt.tune_cache, key,
+                      {TuneLine{'V', tune_size(c), c->solve_dag, c->tune_solve_ms[0], c->tune_solve_ms[1]}});
     return finish(c, st);
 }
 
@@ -1318,7 +1330,8 @@ int make_plan(spi_ctx* c, const std::vector<int32_t>& piv, const std::vector<int
         std::vector<TuneLine> cached;
         read_tune_cache(c->opt.tune_cache, key, cached, nullptr);
         for (const TuneLine& t : cached)
-            if (t.kind == 'B' && std::find(cands.begin(), cands.end(), t.choice) != cands.end()) cands = {t.choice};
+            if (t.kind == 'B' && t.bucket == tune_size(c) && std::find(cands.begin(), cands.end(), t.choice) != cands.end())
+                cands = {t.choice};
     }
     if (cands.size() == 1) {
         DiagPlan h;
@@ -1349,7 +1362,7 @@ int make_plan(spi_ctx* c, const std::vector<int32_t>& piv, const std::vector<int
     cudaEventDestroy(e1);
     if (rc) return rc;
     c->rhs_block_used = bestB;
-    tune_cache_update(c->opt.tune_cache, key, "B", {TuneLine{'B', 0, bestB, best, 0.0}});
+    tune_cache_update(c->opt.tune_cache, key, {TuneLine{'B', tune_size(c), bestB, best, 0.0}});
     DiagPlan h;
     build_diag_plan(sym_sol(c), piv, pos, bestB, h);
     return upload_plan(c, h, dst);
