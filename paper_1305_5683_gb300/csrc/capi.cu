@@ -591,8 +591,8 @@ void factor_launches(spi_ctx* c, int nb, const FactorPlan& F, const spi_ctx::Dev
 // Autotuner of the factorization (tile path per front-size bucket).
 //
 // Two plans are built in which every bucket takes one candidate: all panels
-// on the block-step chain with SIMT Schur complements, and all panels in the
-// persistent per-level kernel with tensor-core Schur complements wherever
+// on the block-step chain with (mixed form) SIMT Schur complements, and all panels in the
+// persistent per-level kernel with (mixed form) tensor-core Schur complements wherever
 // legal.  In both, each (bucket, level) group is launched on its own between
 // timing markers.  Each plan is recorded as a CUDA graph (with its event
 // nodes), replayed twice on the caller's values, and the second replay's
@@ -820,9 +820,11 @@ int prepare_factor_plan(spi_ctx* c, int nb, const double* vals, cudaStream_t st)
             FactorChoice a = ch, b = ch;
             a.panel.clear(); a.schur.clear(); b.panel.clear(); b.schur.clear();
             a.force_panel = ch.force_panel ? ch.force_panel : 1;
-            a.force_schur = ch.force_schur ? ch.force_schur : 1;
             b.force_panel = ch.force_panel ? ch.force_panel : 2;
-            b.force_schur = ch.force_schur ? ch.force_schur : 2;
+            if (mixed_of(c)) {  // (the FP64 form's tensor-core launches are no candidate: both plans have them)
+                a.force_schur = ch.force_schur ? ch.force_schur : 1;
+                b.force_schur = ch.force_schur ? ch.force_schur : 2;
+            }
             std::map<std::pair<int, int32_t>, double> ma, mb;
             int rc = time_plan(c, nb, vals, a, st, ma);
             if (!rc) rc = time_plan(c, nb, vals, b, st, mb);
