@@ -93,3 +93,15 @@ def test_ill_conditioned_front(P, kind, c, n):
             err[dag].append(exact.backward_error(a, s.solve(b), b))
     assert max(err[1]) <= n * EPS
     assert np.median(err[1]) <= 4 * max(np.median(err[2]), EPS)
+
+
+@pytest.mark.parametrize("n,count", [(33, 33), (160, 40), (161, 2), (544, 32), (545, 33), (700, 65)])
+def test_many_right_hand_sides_of_one_factor(P, n, count):
+    """The unpruned variances' full solves, 32 at a time: rows below a step at the edges of 128 and
+    512, a last pass of one right-hand side."""
+    pb = random_spd(n, 1.0, n, dominance=float(n))
+    s = P.Solver.for_problem(pb, diag_unpruned=True)
+    s.factor(pb.values)
+    idx = np.random.default_rng(n).permutation(n)[:count].astype(np.int32)
+    ref = oracle.OracleFactor.from_problem(pb).inv_diag(idx)
+    assert np.abs(s.diag_inverse(idx) / ref - 1).max() <= 64 * n * EPS
