@@ -5,7 +5,8 @@ Bound: both kernels compute z = L^-1 e with a backward error of a few units in t
 last place per multiply-add, at most n of them on a path, so two of them differ by
 at most about n 2^-53 times the condition of the (scaled) triangles; 64 n 2^-53 leaves
 a factor 64 for that condition and the two operands' fixed-point grids (2^-56 of
-their largest entries)."""
+their largest entries).  Tighter: the errors against extended precision next to the SIMT
+kernel's own."""
 import numpy as np
 import pytest
 
@@ -181,3 +182,26 @@ def test_other_block_sizes_hold_no_packed_operands(P, block):
         held.append(s.info()["device_bytes"])
         assert s.info()["launches_diag"] == 1
     assert held[0] == held[1]
+
+
+@pytest.mark.parametrize("dominance", [0.1, 10.0, 300.0])
+def test_accuracy_is_that_of_the_fp64_pipe(P, dominance):
+    """The root mean square error against extended precision at most twice the SIMT kernel's on the
+    same factor (an emulation gives 1.0 times; with six digits instead of seven 30 times or more)."""
+    pb = random_spd(300, 1.0, 3, dominance=dominance)
+    ref = np.diag(exact.inverse(exact.dense(pb)))
+    rms = [float(np.sqrt(np.mean((v / ref - 1) ** 2))) for v in both(P, pb)]
+    assert rms[0] <= 2 * max(rms[1], EPS)
+
+
+@pytest.mark.parametrize("c", [3, 6, 9])
+@pytest.mark.parametrize("n", [64, 130, 300])
+def test_ill_conditioned_front(P, n, c):
+    """A Gaussian kernel matrix plus 10^-c on the diagonal: multiplying by the tiles' inverses, the
+    variances are off by no more than with substitution (both by the factorization's own error)."""
+    t = np.linspace(0.0, 1.0, n)
+    a = np.exp(-((t[:, None] - t) / 0.1) ** 2) + 10.0 ** -c * np.eye(n)
+    pb = exact.problem(a)
+    ref = np.diag(exact.inverse(a))
+    err = [float(np.abs(v / ref - 1).max()) for v in both(P, pb)]
+    assert err[0] <= 1.5 * err[1] + 64 * n * EPS
