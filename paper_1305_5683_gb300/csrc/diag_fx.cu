@@ -275,8 +275,11 @@ __device__ __forceinline__ int fx_tiles(const FxNode& x, int g) {
     return 1 + (x.m - fx_base(x, g) + kFxRows - 1) / kFxRows;
 }
 
+// (kLimit: p.wait_limit polls per wait; a limit that is not a constant costs 2 to 4 % of the kernel)
+template <bool kLimit>
 __global__ void __launch_bounds__(kFxThreads, 1)
     k_diag_fx(DevSym d, FxArgs p, double* __restrict__ out, Strides bs, DevStatus* status) {
+    const uint32_t limit = kLimit ? p.wait_limit : kTcWaitLimit;
     const int band = blockIdx.y;
     out += band * bs.out;
     const int B = p.B, nst = fx_stages(B);
@@ -331,7 +334,7 @@ __global__ void __launch_bounds__(kFxThreads, 1)
                     np += fx_tiles(x, g) * ((min(kFxRows, x.k - g * kFxRows) + kFxSub - 1) / kFxSub);
                 for (int t = 0; t < np && ok; ++t) {
                     const uint32_t st = a_issued % nst;
-                    if (a_issued >= (uint32_t)nst && !fx_wait(bar + kFAE + st, (a_issued / nst - 1) & 1u, abort, p.wait_limit)) {
+                    if (a_issued >= (uint32_t)nst && !fx_wait(bar + kFAE + st, (a_issued / nst - 1) & 1u, abort, limit)) {
                         ok = false;
                         break;
                     }
@@ -358,11 +361,11 @@ __global__ void __launch_bounds__(kFxThreads, 1)
                 for (int g = 0; g < x.G && ok; ++g) {
                     const int w = min(kFxRows, x.k - g * kFxRows), nt = fx_tiles(x, g);
                     for (int i = 0; i < nt && ok; ++i) {
-                        if (tiles_issued > 0 && !fx_wait(bar + kFCE, (tiles_issued - 1) & 1u, abort, p.wait_limit)) { ok = false; break; }
-                        if (i < 2 && !fx_wait(bar + kFBF, bfull++ & 1u, abort, p.wait_limit)) { ok = false; break; }
+                        if (tiles_issued > 0 && !fx_wait(bar + kFCE, (tiles_issued - 1) & 1u, abort, limit)) { ok = false; break; }
+                        if (i < 2 && !fx_wait(bar + kFBF, bfull++ & 1u, abort, limit)) { ok = false; break; }
                         for (int sub = 0; sub * kFxSub < w; ++sub) {
                             const uint32_t st = piece % nst;
-                            if (!fx_wait(bar + kFAF + st, (piece / nst) & 1u, abort, p.wait_limit)) { ok = false; break; }
+                            if (!fx_wait(bar + kFAF + st, (piece / nst) & 1u, abort, limit)) { ok = false; break; }
                             asm volatile("tcgen05.fence::after_thread_sync;");
                             const uint32_t ab = tc_smem_u32(Ar + st * kPiece);
 #pragma unroll
@@ -477,7 +480,7 @@ __global__ void __launch_bounds__(kFxThreads, 1)
                 cut(c0, w, false, true);
                 for (int i = 0; i < nt; ++i, ++tile) {
                     // a warp whose wait ran out does no further work but meets every barrier
-                    if (ok && !__all_sync(0xffffffffu, fx_wait(bar + kFCF, ndone & 1u, abort, p.wait_limit))) {
+                    if (ok && !__all_sync(0xffffffffu, fx_wait(bar + kFCF, ndone & 1u, abort, limit))) {
                         ok = false;
                         *abort = 1;
                     }
@@ -582,7 +585,10 @@ __global__ void __launch_bounds__(kFxThreads, 1)
 size_t diag_fx_pack_bytes(int64_t npieces) { return (size_t)npieces * kPiece; }
 
 cudaError_t diag_fx_setup() {
-    return cudaFuncSetAttribute(k_diag_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fx_smem(kFxMaxBlock));
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_diag_fx<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fx_smem(kFxMaxBlock));
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_diag_fx<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fx_smem(kFxMaxBlock));
 }
 
 void launch_tile_inverses(const DevSym& d, const DevTileInv& x, const double* L, int nb, const Strides& bs,
@@ -600,7 +606,9 @@ void launch_diag_fx(const DevSym& d, const DevDiagPlan& dp, const DevDiagFx& p, 
     FxArgs a{dp.B, dp.order_tc, dp.blk_ptr, dp.uptr, dp.us, dp.ulo, dp.uhi, dp.uzoff, dp.rel, dp.rhs_out,
              dp.rhs_zrow, dp.rhs_col, dp.urel, dp.zbase, dp.Z, p.pptr, p.tptr, p.npieces, p.ntiles, p.pack, p.rexp,
              D, p.fr, wait_limit > 0 ? (uint32_t)wait_limit : wait_limit < 0 ? 0u : kTcWaitLimit};
-    k_diag_fx<<<dim3(dp.nblocks, nb), kFxThreads, fx_smem(dp.B), st>>>(d, a, out, bs, status);
+    const dim3 g(dp.nblocks, nb);
+    if (wait_limit == 0) k_diag_fx<false><<<g, kFxThreads, fx_smem(dp.B), st>>>(d, a, out, bs, status);
+    else k_diag_fx<true><<<g, kFxThreads, fx_smem(dp.B), st>>>(d, a, out, bs, status);
 }
 
 }  // namespace spi
