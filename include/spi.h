@@ -156,11 +156,17 @@ typedef struct spi_options {
                         tiles also let the mixed solve take 128 columns per step there.  0 = the
                         default (32); < 0 = none (SIMT variances, 32-column solve steps).
                         Variance blocks of more than 128 right-hand sides (rhs_block > 128) stay
-                        on the SIMT kernel.  FP64 form: >= 0 the variances run on the tensor
-                        cores from exact integer pieces of the operands, at FP64 accuracy
-                        (blocks of 16, 32 or 64 right-hand sides, chosen by their number when
-                        rhs_block = 0; other rhs_block values, and a device without memory for
-                        the packed operands, take the SIMT kernel); < 0 the SIMT kernel */
+                        on the SIMT kernel.  FP64 form: 0 = the variances run on the tensor cores
+                        (products from exact integer pieces of the operands) where that is
+                        expected to be faster, which a rule on the widths and numbers of the
+                        supernodes and blocks decides per index set; > 0 = wherever possible;
+                        < 0 = never.  Blocks have 16, 32 or 64 right-hand sides there, chosen by
+                        their number when rhs_block = 0; other rhs_block values, diag_ctas_per_sm
+                        > 0, and a device without memory for the packed operands, take the SIMT
+                        kernel.  The pieces keep 56 bits below the largest entry of a row over
+                        128 columns (after scaling by the pivots), so a variance has the error
+                        of FP64 arithmetic; products of entries far below that largest one have
+                        fewer digits of their own (as in the Schur complements, force_schur) */
 } spi_options;
 
 typedef struct spi_stats {

@@ -140,6 +140,7 @@ struct spi_ctx {
     // variances of the FP64 form on the tensor cores: set up at the first variance call
     // (-1: not yet, 0: not in use, 1: ready)
     int fx_state = -1;
+    int last_diag_launches = 1;
     DevDiagFx fx;
     DiagFxHost fx_h;
     // the FP64 form's inverted diagonal tiles (made at the end of every factorization)
@@ -390,14 +391,18 @@ int ensure_device(spi_ctx* c) {
 // Right-hand sides per block that k_diag_fx takes.
 bool fx_takes(int block) { return block == 16 || block == 32 || block == kFxMaxBlock; }
 
+// Whether the FP64 form's tensor-core variances may be used in this context at all.
+bool fx_possible(const spi_ctx* c) {
+    return c->fx_state != 0 && c->ti.xinv && c->opt.diag_tc_min_pivots >= 0 && c->S.n > 0 &&
+           c->opt.diag_ctas_per_sm <= 0 &&  // (a CTA of k_diag_fx takes an SM to itself)
+           (c->opt.rhs_block <= 0 || fx_takes(c->opt.rhs_block));
+}
+
 // Buffers of the FP64 form's tensor-core variances (operands are prepared from the factor
 // by every call).  Without the memory for them the SIMT kernel serves alone.
 int ensure_fx(spi_ctx* c) {
     if (c->fx_state >= 0) return SPI_OK;
     c->fx_state = 0;
-    if (!c->ti.xinv || c->opt.diag_tc_min_pivots < 0 || c->S.n == 0) return SPI_OK;
-    if (c->opt.diag_ctas_per_sm > 0) return SPI_OK;  // a CTA of k_diag_fx takes an SM to itself
-    if (c->opt.rhs_block > 0 && !fx_takes(c->opt.rhs_block)) return SPI_OK;
     const DiagFxHost& h = c->fx_h;
     DevDiagFx& t = c->fx;
     t = DevDiagFx();
@@ -429,7 +434,7 @@ void free_plan(DevDiagPlan& p) {
     p = DevDiagPlan();
 }
 
-int upload_plan(spi_ctx* c, const DiagPlan& h, DevDiagPlan& d) {
+int upload_plan(spi_ctx* c, const DiagPlan& h, DevDiagPlan& d, bool fx = false) {
     free_plan(d);
     d.B = h.B; d.nblocks = h.nblocks; d.nrhs = h.nrhs; d.flops = h.flops; d.work_flops = h.work_flops;
     d.tc_flops = c->dtc.ntc > 0 && h.B <= kDiagTcMaxBlock ? diag_tc_mma_flops(sym_sol(c), c->dtc_h, h) : 0.0;
@@ -452,7 +457,7 @@ int upload_plan(spi_ctx* c, const DiagPlan& h, DevDiagPlan& d) {
     CK(dev_upload(c, &d.urel, h.urel, tr));
     CK(dev_upload(c, &d.zbase, h.zbase, tr));
     d.zsize = h.zbase.empty() ? 0 : h.zbase.back();
-    d.fx = c->fx_state == 1 && fx_takes(h.B);
+    d.fx = fx && c->fx_state == 1;
     if (d.fx) {
         std::vector<int32_t> tiles;
         diag_fx_used(c->S, c->fx_h, h, tiles);
@@ -1292,15 +1297,20 @@ void launch_diag(spi_ctx* c, const DevDiagPlan& p, int nb, int64_t nout, double*
     Strides bs = c->bs;
     bs.Z = p.zsize;
     bs.out = nout;
+    c->last_diag_launches = 1;
     if (mixed_of(c)) {
         const bool tc = c->dtc.ntc > 0 && p.B <= kDiagTcMaxBlock;
+        if (tc) c->last_diag_launches = 2;
         launch_diag_inverse_f32(c->dsym, p, c->d_L32, c->d_D, out, nb, bs, c->diag_smem_pad,
                                 tc ? c->dtc.tc : nullptr, st);
         if (tc) launch_diag_inv_tc(c->dsym, p, c->dtc, c->d_D, out, nb, bs, c->d_status, c->opt.wait_limit, st);
     } else {
-        if (p.fx && c->fx_state == 1) launch_diag_fx(c->dsym, p, c->fx, c->ti, c->d_L, c->d_D, out, nb, bs, c->d_status,
-                                 c->opt.wait_limit, st);
-        else launch_diag_inverse(dev_sol(c), p, c->d_L, c->d_D, out, nb, bs, c->diag_smem_pad, st);
+        if (p.fx && c->fx_state == 1) {
+            c->last_diag_launches = 2;
+            launch_diag_fx(c->dsym, p, c->fx, c->ti, c->d_L, c->d_D, out, nb, bs, c->d_status, c->opt.wait_limit, st);
+            return;
+        }
+        launch_diag_inverse(dev_sol(c), p, c->d_L, c->d_D, out, nb, bs, c->diag_smem_pad, st);
     }
 }
 
@@ -1317,12 +1327,23 @@ int fx_block(int64_t nrhs) { return nrhs <= 152 * 16 ? 16 : nrhs <= 152 * 32 ? 3
 int make_plan(spi_ctx* c, const std::vector<int32_t>& piv, const std::vector<int32_t>& pos, DevDiagPlan& dst,
               int nb, int64_t nout, double* out, cudaStream_t st) {
     std::vector<int> cands;
-    {
-        const int rc = ensure_fx(c);
-        if (rc) return rc;
+    // the FP64 form's tensor-core kernel where it is the faster one
+    if (fx_possible(c)) {
+        DiagPlan h;
+        build_diag_plan(c->S, piv, pos, c->opt.rhs_block > 0 ? c->opt.rhs_block : fx_block((int64_t)piv.size() * nb), h);
+        const bool pays = c->opt.diag_tc_min_pivots > 0 || diag_fx_pays(c->S, h, nb);
+        if (pays) {
+            const int rc = ensure_fx(c);
+            if (rc) return rc;
+        }
+        if (pays && c->fx_state == 1) {
+            if (c->opt.rhs_block == 0 && c->rhs_block_used == 0 && piv.size() >= 4096) c->rhs_block_used = h.B;
+            return upload_plan(c, h, dst, true);
+        }
+        if (!pays) cands = {c->opt.rhs_block > 0 ? c->opt.rhs_block : 16};
     }
-    if (c->opt.rhs_block > 0) cands.push_back(c->opt.rhs_block);
-    else if (c->fx_state == 1) cands.push_back(fx_block((int64_t)piv.size() * nb));
+    if (!cands.empty()) {
+    } else if (c->opt.rhs_block > 0) cands.push_back(c->opt.rhs_block);
     else if (c->rhs_block_used > 0) cands.push_back(c->rhs_block_used);
     else if (mixed_of(c)) cands = {32, 64, 128};
     else cands = {16, 32, 64};
@@ -2614,7 +2635,7 @@ int spi_info(const spi_ctx* c, spi_stats* o) {
     for (const Launch& l : sp.fwd_launches) ls += l.count > 0;
     for (const Launch& l : sp.bwd_launches) ls += l.count > 0;
     o->launches_solve = S.n ? 2 + ls : 0;
-    o->launches_diag = S.n ? (c->fx_state == 1 || c->dtc.ntc > 0 ? 2 : 1) : 0;
+    o->launches_diag = S.n ? c->last_diag_launches : 0;
     o->refine_steps = c->refine_steps;
     o->solve_relres = c->solve_relres;
     o->rhs_block = c->rhs_block_used > 0 ? c->rhs_block_used : c->opt.rhs_block;

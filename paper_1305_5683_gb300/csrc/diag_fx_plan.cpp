@@ -39,22 +39,52 @@ void diag_fx_used(const Symbolic& S, const DiagFxHost& h, const DiagPlan& dp, st
         if (used[h.tiles[4 * t]]) tiles.push_back((int32_t)t);
 }
 
+namespace {
+// Cycles of a CTA for block b.
+double block_cycles(const Symbolic& S, const DiagPlan& dp, int32_t b) {
+    double w = 0.0;
+    for (int32_t u = dp.uptr[b]; u < dp.uptr[b + 1]; ++u) {
+        const int32_t s = dp.us[u], k = S.k_of(s), m = S.m_of(s);
+        const double N = (double)((dp.uhi[u] - (dp.ulo[u] & ~7) + 15) & ~15) / 64.0;
+        for (int32_t c = 0; c < k; c += kFxRows) {
+            const int32_t cw = std::min(kFxRows, k - c), below = m - c - cw;
+            const double tiles = 1.0 + (below + kFxRows - 1) / kFxRows;
+            w += tiles * (3000.0 + N * (2200.0 + 900.0 * ((cw + kFxSub - 1) / kFxSub))) + 3000.0;
+        }
+    }
+    return w;
+}
+}  // namespace
+
 void diag_fx_order(const Symbolic& S, const DiagPlan& dp, std::vector<int32_t>& order) {
     std::vector<double> w((size_t)dp.nblocks, 0.0);
     order.resize((size_t)dp.nblocks);
     for (int32_t b = 0; b < dp.nblocks; ++b) {
         order[(size_t)b] = b;
-        for (int32_t u = dp.uptr[b]; u < dp.uptr[b + 1]; ++u) {
-            const int32_t s = dp.us[u], k = S.k_of(s), m = S.m_of(s);
-            const double N = (double)((dp.uhi[u] - (dp.ulo[u] & ~7) + 15) & ~15) / 64.0;
-            for (int32_t c = 0; c < k; c += kFxRows) {
-                const int32_t cw = std::min(kFxRows, k - c), below = m - c - cw;
-                const double tiles = 1.0 + (below + kFxRows - 1) / kFxRows;
-                w[(size_t)b] += tiles * (3000.0 + N * (2200.0 + 900.0 * ((cw + kFxSub - 1) / kFxSub))) + 3000.0;
-            }
-        }
+        w[(size_t)b] = block_cycles(S, dp, b);
     }
     std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return w[x] > w[y]; });
+}
+
+bool diag_fx_pays(const Symbolic& S, const DiagPlan& dp, int bands) {
+    double sum = 0.0, most = 0.0, nodes = 0.0, most_nodes = 0.0, cols = 0.0, active = 0.0, rows = 0.0;
+    for (int32_t b = 0; b < dp.nblocks; ++b) {
+        const double w = block_cycles(S, dp, b), nd = dp.uptr[b + 1] - dp.uptr[b];
+        double cl = 0.0, ac = 0.0, rw = 0.0;
+        for (int32_t u = dp.uptr[b]; u < dp.uptr[b + 1]; ++u) {
+            const int32_t k = S.k_of(dp.us[u]), below = S.m_of(dp.us[u]) - k;
+            cl += k;
+            ac += (double)k * (dp.uhi[u] - dp.ulo[u]);
+            rw += (double)k * ((below + 63) / 64);
+        }
+        sum += w, most = std::max(most, w), nodes += nd, most_nodes = std::max(most_nodes, nd);
+        cols = std::max(cols, cl), active = std::max(active, ac), rows = std::max(rows, rw);
+    }
+    constexpr double kMhz = 2070.0, kSms = 152.0, kFp64 = 1.13e6;  // flops per us of the FP64 pipe
+    const double fx = 58.0 + 1.1 * most_nodes + 2.4 * most / kMhz +
+                      bands / kSms * (0.75 * sum / kMhz + 7.4 * nodes);
+    const double simt = 42.0 + 0.58 * cols + 0.48 * active / dp.B + 0.23 * rows + 0.69 * bands * dp.work_flops / kFp64;
+    return fx <= simt;
 }
 
 }  // namespace spi

@@ -40,4 +40,16 @@ void diag_fx_used(const Symbolic& S, const DiagFxHost& h, const DiagPlan& dp, st
 // show in, 6.45 ms, so 5.67 (variances of P = 20,000).
 void diag_fx_order(const Symbolic& S, const DiagPlan& dp, std::vector<int32_t>& order);
 
+// Whether k_diag_fx serves plan dp of `bands` bands faster than the SIMT kernel in blocks of 16.  It
+// costs about 7 us of an SM per supernode of a block whatever its width, and so loses where the
+// supernodes are narrow and the blocks many: 8 bands of P = 800 0.70 against 0.41 ms, 3,000
+// problems of order 8 0.35 against 0.10 ms, one unknown of P = 300 137 against 109 us; it wins from a
+// few thousand pointings, a few dozen columns per supernode or one band on (P = 1,500 215 us against
+// 350, 400 problems of order 60 182 against 258 us, P = 20,000 5.7 ms against 70).  Both times in us
+// are fits (relative least squares, coefficients >= 0) to 120 calls measured with either kernel: 26
+// problems of order 8 to 41,000, 1 to 32 bands, 1 to all unknowns.  They are right within 30 % (fx)
+// and a factor 2 (SIMT), and the sides differ by more nearly everywhere: the choice was the slower one
+// in three calls, by 5 to 25 %.
+bool diag_fx_pays(const Symbolic& S, const DiagPlan& dp, int bands);
+
 }  // namespace spi

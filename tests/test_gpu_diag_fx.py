@@ -29,9 +29,9 @@ def P():
 
 
 def both(P, pb, values=None, idx=None, **kw):
-    """(tensor cores, SIMT) variances of one problem."""
+    """(tensor cores, SIMT) variances of one problem, whichever the rule would choose."""
     out = []
-    for more in (kw, {"diag_tc_min_pivots": -1}):
+    for more in (dict(kw, diag_tc_min_pivots=1), {"diag_tc_min_pivots": -1}):
         s = P.Solver.for_problem(pb, **more)
         s.factor(pb.values if values is None else values)
         out.append(s.diag_inverse(idx))
@@ -73,7 +73,7 @@ def test_index_subsets(P, count):
 def test_wide_front_and_repeat(P):
     """A sky front of many chunks; two calls give the same bits (fixed summation order)."""
     pb = generate(sky_scaled(600, 3.0, 12))
-    s = P.Solver.for_problem(pb)
+    s = P.Solver.for_problem(pb, diag_tc_min_pivots=1)
     s.factor(pb.values)
     a, b = s.diag_inverse(), s.diag_inverse()
     assert np.array_equal(a, b)
@@ -97,13 +97,13 @@ def test_badly_scaled_columns(P):
 
 def test_fp64_bands_and_forest(P):
     bands = generate_bands(scaled(BAND, 700, seed=2), 3)
-    s = P.Solver(bands.n, bands.colptr, bands.rowind, batch=3)
+    s = P.Solver(bands.n, bands.colptr, bands.rowind, batch=3, diag_tc_min_pivots=1)
     s.factor_batch(bands.values)
     v = s.diag_inverse_batch().reshape(3, -1)
     for k in range(3):
         assert rel(v[k], oracle.OracleFactor.from_problem(bands.band(k)).inv_diag()) <= 1e-10
     probs = [random_spd(m, 0.2, m) for m in (3, 40, 150)]
-    s = P.Solver.for_problems(probs)
+    s = P.Solver.for_problems(probs, diag_tc_min_pivots=1)
     s.factor(np.concatenate([p.values for p in probs]))
     v = s.diag_inverse()
     assert rel(v, np.concatenate([oracle.OracleFactor.from_problem(p).inv_diag() for p in probs])) <= 1e-10
@@ -145,7 +145,7 @@ def test_wait_timeout_reported(P):
     its tensor memory, and spi_diag_inverse returns SPI_ERR_TIMEOUT.  (The factorization waits
     nowhere: SIMT Schur complements, launches level by level.)"""
     pb = generate(scaled(SCALE, 700, seed=9))
-    s = P.Solver.for_problem(pb, wait_limit=-1, force_schur=1, dag=1)
+    s = P.Solver.for_problem(pb, wait_limit=-1, force_schur=1, dag=1, diag_tc_min_pivots=1)
     s.factor(pb.values)
     with pytest.raises(P.SpiError) as e:
         s.diag_inverse()
@@ -205,3 +205,17 @@ def test_ill_conditioned_front(P, n, c):
     ref = np.diag(exact.inverse(a))
     err = [float(np.abs(v / ref - 1).max()) for v in both(P, pb)]
     assert err[0] <= 1.5 * err[1] + 64 * n * EPS
+
+
+def test_narrow_supernodes_stay_on_the_simt_kernel(P):
+    """The rule's two sides, and the option over it: many problems of order 8 against one wide front."""
+    small = [random_spd(8, 1.0, i, dominance=8.0) for i in range(400)]
+    wide = [random_spd(400, 1.0, 1, dominance=400.0)]
+    for probs, rule in ((small, 1), (wide, 2)):
+        v = {}
+        for forced, launches in ((0, rule), (1, 2), (-1, 1)):
+            s = P.Solver.for_problems(probs, diag_tc_min_pivots=forced)
+            s.factor(np.concatenate([p.values for p in probs]))
+            v[forced] = s.diag_inverse()
+            assert s.info()["launches_diag"] == launches
+        assert rel(v[0], v[-1]) <= 64 * 400 * EPS and rel(v[1], v[-1]) <= 64 * 400 * EPS

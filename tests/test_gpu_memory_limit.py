@@ -13,7 +13,7 @@ import numpy as np
 import paper_1305_5683_gb300 as P
 from spigen import random_spd
 pbs = [random_spd({ORDER}, 1.0, i, dominance={ORDER}.0) for i in range({COUNT})]
-s = P.Solver.for_problems(pbs)
+s = P.Solver.for_problems(pbs, diag_tc_min_pivots=1)
 idx = np.arange(0, {ORDER}, 4, dtype=np.int32)
 for scale in (1.0, 2.0):
     s.factor(np.concatenate([p.values for p in pbs]) * scale)
