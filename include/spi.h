@@ -123,8 +123,9 @@ typedef struct spi_options {
                         least 256 trailing rows and 32 pivots) */
     int dag;         /* 0 = as chosen by the autotuner (timed: one dependency-driven launch against
                         launches level by level, for spi_factor at the first factorization and for
-                        spi_solve at the first solve), else on for spi_factor and launches level by
-                        level for spi_solve; 1 = launches level by level; 2 = the
+                        spi_solve at the first solve), else on for spi_factor, and for spi_solve
+                        in mixed precision without inverted diagonal tiles (launches level by
+                        level otherwise); 1 = launches level by level; 2 = the
                         dependency-driven form: spi_factor runs every level below the first one
                         with a tensor-core launch as one persistent kernel whose CTAs take the tasks
                         (pivot tiles, panel-solve chunks, update and Schur tiles, whole small

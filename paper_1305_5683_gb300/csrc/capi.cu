@@ -143,7 +143,9 @@ struct spi_ctx {
     int last_diag_launches = 1;
     DevDiagFx fx;
     DiagFxHost fx_h;
-    // the FP64 form's inverted diagonal tiles (made at the end of every factorization)
+    // the FP64 form's inverted diagonal tiles: not available, made by every factorization (solve
+    // and variances), or by the variance calls that need them (allocated by the first one)
+    enum TileInverses { kTiNone, kTiFactor, kTiVariances } ti_use = kTiNone;
     DevTileInv ti;
     double last_diag_tc_flops = 0;
     // the mixed solve's plan with 128-column steps for those supernodes (their inverted
@@ -188,8 +190,11 @@ void free_ti(spi_ctx* c) {
     for (void* a : c->ti.allocs) cudaFree(a);
     c->device_bytes -= c->ti.bytes;
     c->ti = DevTileInv();
+    c->ti_use = spi_ctx::kTiNone;
     c->wide_ready = false;
 }
+// Memory for the inverses; without it they stay out of use.
+cudaError_t alloc_ti(spi_ctx* c, bool transposes);
 // One of them given up for memory that another buffer needs; false if there is none left.
 bool release_optional(spi_ctx* c) {
     if (c->fx.allocs.empty() && c->ti.allocs.empty()) return false;
@@ -358,34 +363,48 @@ int ensure_device(spi_ctx* c) {
     if (!mixed_of(c) && !c->opt.pivoting && S.n > 0) {
         build_diag_fx(S, c->fx_h);
         const DiagFxHost& h = c->fx_h;
-        DevTileInv& t = c->ti;
-        t = DevTileInv();
-        const int64_t before = c->device_bytes;
-        std::vector<void*>* tr = &t.allocs;
-        cudaError_t e = dev_upload(c, &t.dtiles, h.dtiles, tr, false);
-        if (e == cudaSuccess) e = dev_upload(c, &t.xoff, h.xoff, tr, false);
-        if (e == cudaSuccess) e = dev_upload(c, &t.xptr, h.xptr, tr, false);
-        if (e == cudaSuccess) e = dev_alloc(c, &t.xinv, (size_t)h.nx * nb, tr, false);
-        if (e == cudaSuccess) e = dev_alloc(c, &t.xinvt, (size_t)h.nx * nb, tr, false);
-        if (e == cudaSuccess) {
-            const std::vector<uint8_t> every((size_t)S.ns, 1);
-            build_solve_plan(S, c->SPw, c->opt.batch, every.data(), true);
-            e = dev_upload(c, &c->d_fwd_items_w, c->SPw.fwd_items, tr, false);
-            if (e == cudaSuccess) e = dev_upload(c, &c->d_bwd_items_w, c->SPw.bwd_items, tr, false);
-        }
-        t.bytes = c->device_bytes - before;
-        if (e == cudaErrorMemoryAllocation) {
-            free_ti(c);  // 32-column solve steps and SIMT variances
-        } else {
-            CK(e);
-            t.ncta = (int64_t)h.dtiles.size() / 4;
-            t.nx = h.nx;
-            c->wa = WideArgs{nullptr, t.xptr, 0, t.xinv, t.xinvt, t.xoff, t.nx};
-            c->wide_ready = true;
+        c->ti_use = spi_ctx::kTiVariances;
+        if (wide_solve_pays(S, h, (int)nb)) {
+            CK(alloc_ti(c, true));
+            DevTileInv& t = c->ti;
+            if (t.xinv) {
+                const std::vector<uint8_t> every((size_t)S.ns, 1);
+                build_solve_plan(S, c->SPw, c->opt.batch, every.data(), true);
+                const int64_t before = c->device_bytes;
+                cudaError_t e = dev_upload(c, &c->d_fwd_items_w, c->SPw.fwd_items, &t.allocs, false);
+                if (e == cudaSuccess) e = dev_upload(c, &c->d_bwd_items_w, c->SPw.bwd_items, &t.allocs, false);
+                t.bytes += c->device_bytes - before;
+                if (e == cudaErrorMemoryAllocation) {
+                    free_ti(c);
+                } else {
+                    CK(e);
+                    c->wa = WideArgs{nullptr, t.xptr, 0, t.xinv, t.xinvt, t.xoff, t.nx};
+                    c->ti_use = spi_ctx::kTiFactor;
+                    c->wide_ready = true;
+                }
+            }
         }
     }
     c->dev_ready = true;
     return SPI_OK;
+}
+
+cudaError_t alloc_ti(spi_ctx* c, bool transposes) {
+    const DiagFxHost& h = c->fx_h;
+    const size_t nb = (size_t)c->opt.batch;
+    DevTileInv& t = c->ti;
+    const int64_t before = c->device_bytes;
+    std::vector<void*>* tr = &t.allocs;
+    cudaError_t e = dev_upload(c, &t.dtiles, h.dtiles, tr, false);
+    if (e == cudaSuccess) e = dev_upload(c, &t.xoff, h.xoff, tr, false);
+    if (e == cudaSuccess) e = dev_upload(c, &t.xptr, h.xptr, tr, false);
+    if (e == cudaSuccess) e = dev_alloc(c, &t.xinv, (size_t)h.nx * nb, tr, false);
+    if (e == cudaSuccess && transposes) e = dev_alloc(c, &t.xinvt, (size_t)h.nx * nb, tr, false);
+    t.bytes = c->device_bytes - before;
+    t.ncta = (int64_t)h.dtiles.size() / 4;
+    t.nx = h.nx;
+    if (e != cudaSuccess) free_ti(c);
+    return e == cudaErrorMemoryAllocation ? cudaSuccess : e;
 }
 
 // Right-hand sides per block that k_diag_fx takes.
@@ -393,7 +412,7 @@ bool fx_takes(int block) { return block == 16 || block == 32 || block == kFxMaxB
 
 // Whether the FP64 form's tensor-core variances may be used in this context at all.
 bool fx_possible(const spi_ctx* c) {
-    return c->fx_state != 0 && c->ti.xinv && c->opt.diag_tc_min_pivots >= 0 && c->S.n > 0 &&
+    return c->fx_state != 0 && c->ti_use != spi_ctx::kTiNone && c->opt.diag_tc_min_pivots >= 0 && c->S.n > 0 &&
            c->opt.diag_ctas_per_sm <= 0 &&  // (a CTA of k_diag_fx takes an SM to itself)
            (c->opt.rhs_block <= 0 || fx_takes(c->opt.rhs_block));
 }
@@ -403,6 +422,10 @@ bool fx_possible(const spi_ctx* c) {
 int ensure_fx(spi_ctx* c) {
     if (c->fx_state >= 0) return SPI_OK;
     c->fx_state = 0;
+    if (!c->ti.xinv) {
+        CK(alloc_ti(c, false));
+        if (!c->ti.xinv) return SPI_OK;
+    }
     const DiagFxHost& h = c->fx_h;
     DevDiagFx& t = c->fx;
     t = DevDiagFx();
@@ -463,6 +486,11 @@ int upload_plan(spi_ctx* c, const DiagPlan& h, DevDiagPlan& d, bool fx = false) 
         diag_fx_used(c->S, c->fx_h, h, tiles);
         d.fx_ntiles = (int64_t)tiles.size();
         CK(dev_upload(c, &d.fx_tiles, tiles, tr));
+        if (c->ti_use == spi_ctx::kTiVariances) {
+            diag_fx_used_inverses(c->S, c->fx_h, h, tiles);
+            d.fx_ninv = (int64_t)tiles.size() / 4;
+            CK(dev_upload(c, &d.fx_inv, tiles, tr));
+        }
     }
     // FP64 elements per band are enough for both element types
     CK(dev_alloc(c, &d.Z, (size_t)std::max<int64_t>(d.zsize, 1) * (size_t)c->opt.batch, tr));
@@ -1136,7 +1164,7 @@ int factor_impl(spi_ctx* c, int nb, const double* values, int values_on_device, 
         // the variances' tensor-core operands (inverted diagonal tiles, packed TF32 pairs)
         if (mixed) launch_diag_tc_pack(c->dsym, c->dtc, c->d_L32, nb, c->bs, s2);
         // the FP64 form's inverted diagonal tiles (solves, variances)
-        if (c->ti.xinv) launch_tile_inverses(c->dsym, c->ti, c->d_L, nb, c->bs, s2);
+        if (c->ti_use == spi_ctx::kTiFactor) launch_tile_inverses(c->dsym, c->ti, c->d_L, nb, c->bs, s2);
     }));
     rc = finish(c, st);
     if (rc == SPI_OK) {
@@ -1183,8 +1211,10 @@ cudaError_t solve_core(spi_ctx* c, int nb, const double* b, double* x, cudaStrea
 
 // The solve's form (dependency-driven launch or launches level by level), decided
 // at the first solve when spi_options.dag = 0: timed on the caller's right-hand
-// side when spi_options.autotune allows (the faster of two runs each), else the
-// dependency-driven launch.
+// side when spi_options.autotune allows (the faster of two runs each), else by rule: level by
+// level in FP64 and with wide steps, the dependency-driven launch for the other mixed problems.
+// (FP64 in 32-column steps, launches chained, against the dependency-driven launch: order 500 152
+// and 248 us, 32 bands of P = 800 460 and 608, 3,000 problems of order 8 122 and 188.)
 int choose_solve_form(spi_ctx* c, int nb, const double* bd, cudaStream_t st) {
     if (c->solve_dag >= 0) return SPI_OK;
     const std::string key = tune_key(c, nb);
@@ -1197,7 +1227,7 @@ int choose_solve_form(spi_ctx* c, int nb, const double* bd, cudaStream_t st) {
     }
     const bool timing = c->opt.autotune > 0 || (c->opt.autotune == 0 && c->S.factor_flops >= 2e8);
     if (!timing || c->SP.dag.empty()) {
-        c->solve_dag = c->SP.dag.empty() || c->wide_ready ? 0 : 1;
+        c->solve_dag = c->SP.dag.empty() || c->wide_ready || !mixed_of(c) ? 0 : 1;
         return SPI_OK;
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1306,7 +1336,7 @@ void launch_diag(spi_ctx* c, const DevDiagPlan& p, int nb, int64_t nout, double*
         if (tc) launch_diag_inv_tc(c->dsym, p, c->dtc, c->d_D, out, nb, bs, c->d_status, c->opt.wait_limit, st);
     } else {
         if (p.fx && c->fx_state == 1) {
-            c->last_diag_launches = 2;
+            c->last_diag_launches = p.fx_ninv > 0 ? 3 : 2;
             launch_diag_fx(c->dsym, p, c->fx, c->ti, c->d_L, c->d_D, out, nb, bs, c->d_status, c->opt.wait_limit, st);
             return;
         }
@@ -1331,7 +1361,13 @@ int make_plan(spi_ctx* c, const std::vector<int32_t>& piv, const std::vector<int
     if (fx_possible(c)) {
         DiagPlan h;
         build_diag_plan(c->S, piv, pos, c->opt.rhs_block > 0 ? c->opt.rhs_block : fx_block((int64_t)piv.size() * nb), h);
-        const bool pays = c->opt.diag_tc_min_pivots > 0 || diag_fx_pays(c->S, h, nb);
+        double extra = 0.0;
+        if (c->ti_use == spi_ctx::kTiVariances) {
+            std::vector<int32_t> own;
+            diag_fx_used_inverses(c->S, c->fx_h, h, own);
+            extra = tile_inverse_us(c->S, own, nb);
+        }
+        const bool pays = c->opt.diag_tc_min_pivots > 0 || diag_fx_pays(c->S, h, nb, extra);
         if (pays) {
             const int rc = ensure_fx(c);
             if (rc) return rc;

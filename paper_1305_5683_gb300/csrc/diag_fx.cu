@@ -57,7 +57,8 @@ constexpr int kPiece = kDig * kSlice;              // bytes of a packed piece
 // vectors down the 32-row blocks, lane = row, two columns per warp.  Bound by the FP64
 // pipe (64 cycles per warp instruction) and the chain of columns, so a tile is spread
 // over w / 8 CTAs, every step is two independent multiply-adds per warp, and the values
-// passed between steps are shuffled or read from shared memory.  X's transpose is stored too.  (One column per warp
+// passed between steps are shuffled or read from shared memory.  X's transpose is stored too (xinvt
+// not null).  (One column per warp
 // was quicker for one small front, 21 against 27 us, but 354 against 193 us for all of
 // P = 20,000.)
 __global__ void __launch_bounds__(128) k_fx_tinv(DevSym d, const int32_t* __restrict__ dtiles,
@@ -76,15 +77,19 @@ __global__ void __launch_bounds__(128) k_fx_tinv(DevSym d, const int32_t* __rest
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int col = q0 + 2 * warp;
     double* X = xinv + (int64_t)blockIdx.y * nx + xoff[t];  // column-major, leading dimension w
-    double* Xt = xinvt + (int64_t)blockIdx.y * nx + xoff[t];  // its transpose
+    double* Xt = xinvt ? xinvt + (int64_t)blockIdx.y * nx + xoff[t] : nullptr;  // its transpose, for the solve
+    auto put = [&](int i, int j, double v) {
+        X[i + j * w] = v;
+        if (Xt) Xt[j + i * w] = v;
+    };
     __shared__ double xs[4][kFxRows][2];
     double (*x)[2] = xs[warp];
     if (col >= w) return;
     const bool two = col + 1 < w;
     const int jb = col / 32;
     for (int r = lane; r < 32 * jb; r += 32) {  // above the columns' own block
-        X[r + col * w] = Xt[col + r * w] = 0.0;
-        if (two) X[r + (col + 1) * w] = Xt[col + 1 + r * w] = 0.0;
+        put(r, col, 0.0);
+        if (two) put(r, col + 1, 0.0);
     }
     for (int i = jb; 32 * i < w; ++i) {
         const int r = 32 * i + lane;
@@ -115,8 +120,8 @@ __global__ void __launch_bounds__(128) k_fx_tinv(DevSym d, const int32_t* __rest
         x[r][0] = a0;
         x[r][1] = a1;
         __syncwarp();
-        if (on) X[r + col * w] = Xt[col + r * w] = a0;
-        if (on && two) X[r + (col + 1) * w] = Xt[col + 1 + r * w] = a1;
+        if (on) put(r, col, a0);
+        if (on && two) put(r, col + 1, a1);
     }
 }
 
@@ -600,6 +605,12 @@ void launch_tile_inverses(const DevSym& d, const DevTileInv& x, const double* L,
 void launch_diag_fx(const DevSym& d, const DevDiagPlan& dp, const DevDiagFx& p, const DevTileInv& x, const double* L, const double* D,
                     double* out, int nb, const Strides& bs, DevStatus* status, int wait_limit, cudaStream_t st) {
     if (dp.nblocks == 0 || nb == 0) return;
+    if (dp.fx_ninv > 0) {  // (the factorization did not make them)
+        DevTileInv part = x;
+        part.dtiles = dp.fx_inv;
+        part.ncta = dp.fx_ninv;
+        launch_tile_inverses(d, part, L, nb, bs, st);
+    }
     k_fx_pack<<<dim3((unsigned)dp.fx_ntiles, nb), kFxRows, 0, st>>>(d, p.tiles, p.tdiag, dp.fx_tiles, p.ntiles, p.npieces,
                                                                     x.xoff, x.nx, L, D, x.xinv, p.pack, p.rexp, p.fr,
                                                                     bs.L, bs.n);

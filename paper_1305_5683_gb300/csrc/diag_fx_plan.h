@@ -33,6 +33,20 @@ struct DiagFxHost {
 void build_diag_fx(const Symbolic& S, DiagFxHost& h);
 // the tiles (positions in h.tiles / 4) of the supernodes that plan dp walks
 void diag_fx_used(const Symbolic& S, const DiagFxHost& h, const DiagPlan& dp, std::vector<int32_t>& tiles);
+// The diagonal tiles' columns (positions in h.dtiles / 4) of the supernodes that plan dp walks
+void diag_fx_used_inverses(const Symbolic& S, const DiagFxHost& h, const DiagPlan& dp, std::vector<int32_t>& dtiles);
+// Whether the inverses of all diagonal tiles are made by every factorization, for the solve's wide
+// steps: where they shorten the solve by at least what they take.  us of each: a solve gains 6 per
+// step saved in each sweep (and about 9 at any size), measured over the problems of diag_fx_pays; the
+// inverses take tile_inverse_us.  P = 20,000: 175 us against 863 a solve; 48 trees of 50-2,000
+// pointings 147 against 85; 400 problems of order 60 98 against 16 (factorization 127 us with
+// the inverses left out, 213 with them), 32 bands of P = 800 107 against 24.  Where they are not
+// made, the solve takes 32-column steps and the tensor-core variances make those they need.
+bool wide_solve_pays(const Symbolic& S, const DiagFxHost& h, int bands);
+// us of k_fx_tinv for `bands` bands of the listed column groups ([][4] as DiagFxHost::dtiles): its
+// FP64 instructions at 1.45 times their share of the pipe, and at least the chain of the widest tile
+// (measured: 104 us for 400 tiles of order 60, 194 for 60 fronts of order 300, 52 for one tile of 128)
+double tile_inverse_us(const Symbolic& S, const std::vector<int32_t>& dtiles, int bands);
 // The blocks of plan dp in the order in which they start: the costliest first, in cycles of a
 // CTA: per tile 900 a piece and 2,200 for the read-out of 64 right-hand sides and 3,000
 // whatever their number, 3,000 a chunk.  With about four CTAs per SM the last ones to start set
@@ -50,6 +64,7 @@ void diag_fx_order(const Symbolic& S, const DiagPlan& dp, std::vector<int32_t>& 
 // problems of order 8 to 41,000, 1 to 32 bands, 1 to all unknowns.  They are right within 30 % (fx)
 // and a factor 2 (SIMT), and the sides differ by more nearly everywhere: the choice was the slower one
 // in three calls, by 5 to 25 %.
-bool diag_fx_pays(const Symbolic& S, const DiagPlan& dp, int bands);
+// extra: us of further work that only k_diag_fx needs.
+bool diag_fx_pays(const Symbolic& S, const DiagPlan& dp, int bands, double extra);
 
 }  // namespace spi

@@ -212,6 +212,8 @@ struct DevDiagPlan {
                           //   plan's supernodes
     int32_t* fx_tiles = nullptr;
     int64_t fx_ntiles = 0;
+    int32_t* fx_inv = nullptr;  // the column groups of diagonal tiles that the call itself inverts
+    int64_t fx_ninv = 0;        //   (DevTileInv::dtiles; 0: the factorization made them)
     std::vector<void*> allocs;
 };
 
@@ -304,7 +306,7 @@ struct DevTileInv {
     int32_t* xptr = nullptr;         // [ns] first tile of each supernode
     int64_t* xoff = nullptr;         // [tiles]
     double* xinv = nullptr;          // [bands][nx]
-    double* xinvt = nullptr;         // [bands][nx] their transposes
+    double* xinvt = nullptr;         // [bands][nx] their transposes (null: made for the variances only)
     std::vector<void*> allocs;       // (none: not in use)
     int64_t bytes = 0;
 };

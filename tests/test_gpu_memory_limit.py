@@ -7,7 +7,7 @@ import pytest
 import shim
 
 pytestmark = pytest.mark.gpu
-ORDER, COUNT = 160, 24
+ORDER, COUNT = 320, 12  # (the solve's wide steps pay from about here on)
 CODE = f"""
 import numpy as np
 import paper_1305_5683_gb300 as P
@@ -44,8 +44,8 @@ def test_results_under_every_limit(P, tmp_path):
     code = f"OUT = {out!r}\n" + CODE
     _, _, peak = shim.run(so, tmp_path, code)
     ref = dict(np.load(out))
-    tiles = 2 * 8 * COUNT * (128 ** 2 + (ORDER - 128) ** 2)   # the inverses and their transposes
-    pieces = COUNT * (8 + 8 + 2) * 7 * 4096                     # 128 x 16 pieces of the two chunks
+    tiles = 2 * 8 * COUNT * (2 * 128 ** 2 + 64 ** 2)  # the inverses and their transposes
+    pieces = COUNT * (3 * 8 + 2 * 8 + 4) * 7 * 4096    # 128 x 16 pieces of the three chunks
     for limit in (peak - 1, peak - pieces // 2, peak - pieces + 1, peak - pieces - tiles // 4,
                   peak - pieces - tiles + 4096):
         _, kernels, used = shim.run(so, tmp_path, code, limit=limit)

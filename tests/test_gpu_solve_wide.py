@@ -8,6 +8,7 @@ import pytest
 
 import exact
 import oracle
+import shim
 from spigen import SCALE, BAND, generate, generate_bands, random_spd, scaled
 
 pytestmark = pytest.mark.gpu
@@ -75,6 +76,22 @@ def ill_conditioned(kind, c, n):
     return a @ a + 10.0 ** -c * np.eye(n)
 
 
+def beside_a_chain(pb):
+    """The forest of pb and a front of 400 columns, whose many steps make the factorization prepare
+    the wide steps of every supernode (alone, a small pb may be solved in 32-column steps)."""
+    return [pb, random_spd(400, 1.0, 7, dominance=400.0)]
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 63, 64, 65, 127, 128, 129, 191, 193, 256, 257, 330])
+def test_wide_steps_of_every_width(P, n):
+    probs = beside_a_chain(random_spd(n, 1.0, n, dominance=float(n)))
+    s = P.Solver.for_problems(probs, dag=1)
+    s.factor(np.concatenate([p.values for p in probs]))
+    x = s.solve(np.concatenate([p.b for p in probs]))[:n]
+    ref = oracle.OracleFactor.from_problem(probs[0]).solve(probs[0].b)
+    assert np.abs(x - ref).max() <= 64 * max(n, 16) * EPS * np.abs(ref).max()
+
+
 @pytest.mark.parametrize("n", [40, 64, 65, 130, 200])
 @pytest.mark.parametrize("kind,c", [("kernel", 4), ("kernel", 8), ("kernel", 11), ("difference", 4), ("difference", 9)])
 def test_ill_conditioned_front(P, kind, c, n):
@@ -82,17 +99,50 @@ def test_ill_conditioned_front(P, kind, c, n):
     dependency-driven form, dag = 2), whatever the blocks' condition: a backward error within
     n 2^-53, and within four times substitution's or the unit roundoff."""
     a = ill_conditioned(kind, c, n)
-    pb = exact.problem(a)
+    probs = beside_a_chain(exact.problem(a))
+    values, rest = np.concatenate([p.values for p in probs]), probs[1].b
     rng = np.random.default_rng(n + c)
     err = {1: [], 2: []}
     for _ in range(3):
         b = a @ rng.standard_normal(n)
         for dag in err:
-            s = P.Solver.for_problem(pb, dag=dag)
-            s.factor(pb.values)
-            err[dag].append(exact.backward_error(a, s.solve(b), b))
+            s = P.Solver.for_problems(probs, dag=dag)
+            s.factor(values)
+            err[dag].append(exact.backward_error(a, s.solve(np.concatenate([b, rest]))[:n], b))
     assert max(err[1]) <= n * EPS
     assert np.median(err[1]) <= 4 * max(np.median(err[2]), EPS)
+
+
+def test_inverses_are_made_where_they_pay(P, tmp_path):
+    """The factorization inverts the diagonal tiles for a long chain of steps, and not for many small
+    fronts, whose solve they shorten by less than they take; there the tensor-core variances, when
+    asked for, make their own.  Both against the SIMT kernel and the oracle's x."""
+    code = """
+import numpy as np
+import paper_1305_5683_gb300 as P
+from spigen import random_spd
+pbs = [random_spd({n}, 1.0, i, dominance={n}.0) for i in range({count})]
+s = P.Solver.for_problems(pbs, dag=1, diag_tc_min_pivots=1)
+s.factor(np.concatenate([p.values for p in pbs]))
+x = s.solve(np.concatenate([p.b for p in pbs]))
+if {variances}:
+    v = [s.diag_inverse(), s.diag_inverse(np.arange(5, dtype=np.int32))]
+    r = P.Solver.for_problems(pbs, diag_tc_min_pivots=-1)
+    r.factor(np.concatenate([p.values for p in pbs]))
+    w = r.diag_inverse()
+    assert abs(v[0] / w - 1).max() < 1e-12 and abs(v[1] / w[:5] - 1).max() < 1e-12
+    assert s.info()["launches_diag"] == {launches}
+np.save({out!r}, x)
+"""
+    so, out = shim.build(tmp_path), str(tmp_path / "x.npy")
+    for n, count, variances, launches, made in ((400, 1, False, 0, True), (400, 1, True, 2, True), (60, 100, False, 0, False),
+                                                (60, 100, True, 3, True)):
+        _, kernels, _ = shim.run(so, tmp_path, code.format(n=n, count=count, variances=variances, launches=launches, out=out))
+        assert any("k_fx_tinv" in k for k in kernels) == made
+        assert any("k_fwd_wide64" in k for k in kernels) == (n == 400)
+        x = np.load(out)[:n]
+        pb = random_spd(n, 1.0, 0, dominance=float(n))
+        assert np.abs(x - oracle.OracleFactor.from_problem(pb).solve(pb.b)).max() <= 64 * n * EPS * np.abs(x).max()
 
 
 @pytest.mark.parametrize("n,count", [(33, 33), (160, 40), (161, 2), (544, 32), (545, 33), (700, 65)])
