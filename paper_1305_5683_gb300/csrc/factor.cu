@@ -529,17 +529,20 @@ __device__ void factor_pivot_tile(double (*A)[kT + 1], double* dv, S* P, int64_t
         for (int q = 0; q < kT * kT / kThreads; ++q)
             if (warp + 4 * q <= lane) A[lane][warp + 4 * q] = (double)v[q];
     }
-    // this thread's entries (warps 0-2): e = tid + 96 q of the column-by-column list; by its
-    // distance from the end, columns 31, 30, ... hold 1, 2, ... entries
+    // this thread's entries (warps 0-2): e = tid + 96 q of the column-by-column list of a tile of width
+    // w, which is the end of the full tile's list moved up by 32 - w; nq of them, uniform in a warp
+    // (a multiply-add merely predicated off takes the pipe as long)
+    const int tri = (w - 2) * (w - 1) / 2;
+    const int nq = warp < 3 && w > 2 ? max(0, (tri - 32 * warp + kTriThreads - 1) / kTriThreads) : 0;
     int oi[kTriOwn], oj[kTriOwn];
     double ov[kTriOwn];
 #pragma unroll
     for (int q = 0; q < kTriOwn; ++q) {
         const int e = tid + kTriThreads * q;
-        const bool on = warp < 3 && e < kTri;
-        const uint16_t t = on ? kTriTable.at[kTri - 1 - e] : (uint16_t)0;
-        oi[q] = t >> 8;
-        oj[q] = t & 255;
+        const bool on = q < nq && e < tri;
+        const uint16_t t = on ? kTriTable.at[tri - 1 - e] : (uint16_t)0;
+        oi[q] = on ? (t >> 8) - (kT - w) : 0;
+        oj[q] = on ? (t & 255) - (kT - w) : 0;
     }
     const double ad = tid < w ? adiag[f + c0 + tid] : 0.0;
     __syncthreads();
@@ -561,7 +564,7 @@ __device__ void factor_pivot_tile(double (*A)[kT + 1], double* dv, S* P, int64_t
     if (warp == 3 && lane > 0) A[0][lane] = lc[0][lane];
     for (int c = 0; c + 1 < w; ++c) {
         if (warp == 3) {
-            if (c > 0) nx = in[(c + 1) & 1][lane];
+            if (c > 0) nx = lane < w ? in[(c + 1) & 1][lane] : 0.0;
             a = fma(-l, an, nx);  // rows above c + 1 hold nothing of use
             const double d = __shfl_sync(0xffffffffu, a, c + 1);
             an = __shfl_sync(0xffffffffu, a, min(c + 2, kT - 1));
@@ -572,11 +575,20 @@ __device__ void factor_pivot_tile(double (*A)[kT + 1], double* dv, S* P, int64_t
             if (lane > c + 1) A[c + 1][lane] = l;
         } else {
             const double *cl = lc[c & 1], *ca = ac[c & 1];
-#pragma unroll
-            for (int q = 0; q < kTriOwn; ++q) {
+            auto apply = [&](int q) {
                 if (oj[q] >= c + 2) {
                     ov[q] = fma(-ca[oi[q]], cl[oj[q]], ov[q]);
                     if (oj[q] == c + 2) in[c & 1][oi[q]] = ov[q];
+                }
+            };
+            if (w == kT) {  // (without the loop's exits: 1 % of a factorization of full tiles)
+#pragma unroll
+                for (int q = 0; q < kTriOwn; ++q) apply(q);
+            } else {
+#pragma unroll
+                for (int q = 0; q < kTriOwn; ++q) {
+                    if (q >= nq) break;
+                    apply(q);
                 }
             }
         }
