@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(kThreads) k_diag_inv(DevSym d, DiagArgs p, con
                         // second pivot of a 2x2 block: the cross term 2 z_p z_c (D^-1)_pc with its
                         // partner p = c - 1, whose z is final (this block column or the last one)
                         const int j = f + cb + c;
-                        if (d.pair[j] == j - 1) {
+                        if (j > 0 && d.pair[j] == j - 1) {  // (pivot 0 has no predecessor: -1 marks it a 1x1 pivot)
                             const T zp = c > 0 ? Zd[(c - 1) * B + t] : Z[(int64_t)(zo + cb - 1) * B + lo + t];
                             v += 2.0 * (double)zp * (double)zc * d.dinv_b[j];
                         }
