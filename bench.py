@@ -268,9 +268,10 @@ def priority_stream(dev):
     """A stream of the highest priority, for the mixed form's factorization and solve.
     The variances of the same factor run beside the solve on a second stream; on this
     stream the solve's short launches are dispatched ahead of the variance kernel's
-    pending CTAs instead of behind them.  The FP64 form keeps default priorities: its
-    variance kernel runs at the FP64 pipe's rate, and a solve dispatched ahead of it
-    takes that rate away instead of filling gaps (measured: FP64 step 87.1 -> 89.1 ms)."""
+    pending CTAs instead of behind them.  The FP64 form keeps default priorities:
+    while its variances ran on the FP64 pipe, a solve dispatched ahead of them took that
+    pipe's rate away (step 87.1 -> 89.1 ms); not measured again since they run on the
+    tensor cores."""
     import torch
     try:
         _, hi = torch.cuda.Stream.priority_range()

@@ -13,9 +13,13 @@
 // the products of a 128-column chunk are accumulated in one FP32 accumulator:
 // at most 7 x 128 x 2^14 < 2^24, so every sum is exact, whatever its order.
 // The seven level sums are put together in 64-bit integers and rounded once to
-// FP64.  What is dropped (levels > 6 and the 57th bits) is 2^-56 of the
-// largest entries per product, below the rounding of an FP64 dot product.  To
-// keep "largest entry" meaningful the kernel works with S^-1 L S and y = S^-1 z, S the
+// FP64.  What is dropped is bounded by the product of the row's and the column's largest
+// entries, not by the product itself: at most 24 x 2^-56 of it for the levels > 6 and 4 x
+// 2^-56 for the operands' rounding to their grids, about 2^-56 to 2^-54 rms.  The sums of
+// squares taken here are served by that (an entry far below its column's largest adds as
+// little to the variance); entries of N^-1 off the diagonal, which can be far smaller than
+// the products they are summed from, are not, so covariances take the SIMT kernel's FP64
+// solves (diag.cu).  To keep "largest entry" meaningful the kernel works with S^-1 L S and y = S^-1 z, S the
 // powers of two next to D^1/2 (no rounding), so that the scale of an unknown cancels:
 // the rows have the scale of N's entries over the square roots of their diagonal ones, y
 // that of the variances' square roots, and (N^-1)_ii = sum_k y_k^2 f_k with f = S^2 / D
@@ -280,7 +284,9 @@ __device__ __forceinline__ int fx_tiles(const FxNode& x, int g) {
     return 1 + (x.m - fx_base(x, g) + kFxRows - 1) / kFxRows;
 }
 
-// (kLimit: p.wait_limit polls per wait; a limit that is not a constant costs 2 to 4 % of the kernel)
+// (kLimit: p.wait_limit polls per wait; a limit that is not a constant costs 2 to 4 % of the kernel.
+// 576 threads put five warps on one of the four schedulers, 96 registers each: ptxas spills 196
+// bytes of stores and 292 of loads.)
 template <bool kLimit>
 __global__ void __launch_bounds__(kFxThreads, 1)
     k_diag_fx(DevSym d, FxArgs p, double* __restrict__ out, Strides bs, DevStatus* status) {

@@ -690,10 +690,10 @@ __global__ void __launch_bounds__(kThreads) k_diag_front(DevSym d, const int32_t
     diag_front_body(d, items[blockIdx.x], L, D, DS, adiag, status, (int)(blockIdx.y * bs.n));
 }
 
-// Shared memory of the per-level panel kernel; the three phases of a block
-// step use it in turn.
 template <typename C>
 constexpr int kLjLd = kT + (std::is_same<C, float>::value ? 4 : 1);  // row of a Schur tile's scaled operand
+// Shared memory of the per-level panel kernel, whose block step's three phases use it in
+// turn, and of the dependency-driven kernel's tasks.
 template <typename C>
 union FrontPanelSmem {
     struct {
@@ -778,7 +778,7 @@ __device__ __forceinline__ void panel_row1(float* P, int64_t m, int c0, int w, i
 }
 
 // A whole front's panel by one CTA: per 32-column block step, the FP64 pivot
-// tile, the panel solve of every row below it (one thread per row), then the
+// tile, the panel solve of every row below it (FP64 four lanes per row, FP32 a thread), then the
 // rank-32 update of the remaining panel columns in 32 x 32 tiles.  The Schur
 // complement is left to the Schur tiles.
 template <typename C, bool kCg>
@@ -862,6 +862,8 @@ __device__ void front_panel_body(const DevSym& d, int s, C* Lb, double* Db, C* D
 // its own, so a small front costs one launch per level instead of three or
 // more per 32-column block step.  A front with a diagonal pivot block (~s in
 // the list) is scaled column by column.  The CTAs never wait on one another.
+// (FP32: four CTAs per SM leave 128 registers, and ptxas spills 248 bytes; FP64 at three
+// spills none.  k_factor_dag<float> spills 52.)
 template <typename C>
 __global__ void __launch_bounds__(kThreads, sizeof(C) == 4 ? 4 : 3) k_front_panel(DevSym d, const int32_t* __restrict__ items, int nitems,
                                                           int nb, C* __restrict__ L, double* __restrict__ D,

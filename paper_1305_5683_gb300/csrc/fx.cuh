@@ -4,7 +4,8 @@
 // entry and cut into seven signed 8-bit digits, exact in FP16; the products of digits i and
 // j with i + j = l accumulate exactly in one FP32 accumulator per level l <= 6 (integers
 // below 2^24 for up to 128 products); the level sums are joined in 64-bit integers and
-// rounded once.  Shared by the variance kernel (diag_fx.cu) and the Schur complements
+// rounded once.  The error of a product is bounded relative to the product of the two
+// operands' largest entries (28 x 2^-56 at most, about 2^-56 to 2^-54 rms), not to the result.  Shared by the variance kernel (diag_fx.cu) and the Schur complements
 // (factor.cu).
 #pragma once
 #include <cuda_fp16.h>

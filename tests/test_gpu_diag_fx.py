@@ -110,7 +110,7 @@ def test_fp64_bands_and_forest(P):
 
 
 @pytest.mark.parametrize("count", [1, 16, 40, 512])
-def test_inverse_block_on_the_scaled_vectors(P, count):
+def test_inverse_block_beside_variances(P, count):
     pb = generate(scaled(SCALE, 1200, seed=9))
     idx = np.sort(np.random.default_rng(count).permutation(pb.n)[:count]).astype(np.int32)
     s = P.Solver.for_problem(pb)
