@@ -1372,7 +1372,7 @@ __global__ void __launch_bounds__(128) k_schur_tc(DevSym d, const int32_t* __res
 // each), one cutting while the other multiplies or reads out.  The SIMT kernels are
 // bound by the FP64 pipe: 79,000 cycles of an SM for the multiply-adds of 128 x 32 x 32.
 // Factorization of P = 20,000: 16.8 -> 8.3 ms; its leaves' Schur complements (41,335 tiles, 13
-// pivots on average) take 1.2 ms, 47 % of the issue slots in use (cutting, joining, scattering).
+// pivots on average) take 1.2 ms, 53 % of the issue slots in use (cutting, joining, scattering).
 // A non-finite operand makes its row or column of C NaN.
 constexpr int kSfThreads = 256;
 constexpr int kSfPlaneA = kFxTileM * kFxTileK * 2;  // bytes of a digit plane of the rows
